@@ -30,7 +30,7 @@ int ensure_workspace(sqcg_ctx* ctx) {
             cudaMalloc((void**)&ctx->xh32, n * sizeof(float2)) == cudaSuccess &&
             cudaMalloc((void**)&ctx->xff, n * sizeof(float4)) == cudaSuccess &&
             cudaMalloc((void**)&ctx->partials, 4 * (size_t)ctx->max_blocks * sizeof(double)) == cudaSuccess &&
-            cudaMalloc((void**)&ctx->fin_aux, 64 * sizeof(float2)) == cudaSuccess &&
+            cudaMalloc((void**)&ctx->fin_aux, 96 * sizeof(float2)) == cudaSuccess &&
             cudaMalloc((void**)&ctx->fin_cnt, 32 * sizeof(unsigned)) == cudaSuccess &&
             cudaMalloc((void**)&ctx->st, sizeof(SolverState)) == cudaSuccess &&
             cudaMallocHost((void**)&ctx->st_host, sizeof(SolverState)) == cudaSuccess;

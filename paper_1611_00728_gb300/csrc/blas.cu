@@ -92,8 +92,7 @@ __global__ void __launch_bounds__(kThreads, 5)
 k_sr_update(float2* __restrict__ r, const float2* __restrict__ sv, float2* __restrict__ p, float2* __restrict__ q,
             float2* __restrict__ xh, int Vh, SolverState* st, double* cpart) {
   pdl_wait();
-  const volatile SolverState* vs = st;
-  if (vs->done || vs->need_update) return;  // uniform over the grid: the step did not complete
+  if (!gate_open(st, GATE_STEP)) return;  // uniform over the grid: the step did not complete
   const float alpha = (float)st->alpha, beta = (float)st->beta;
   float2 cross[1] = {make_float2(0.f, 0.f)};  // float-float, as the step's other sums
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Vh; i += gridDim.x * blockDim.x) {
@@ -224,9 +223,8 @@ __global__ void __launch_bounds__(kThreads)
 k_ms_xpay(MSPtrs P, const typename V2<R>::T* __restrict__ r, typename V2<R>::T* __restrict__ p, int Vh,
           const SolverState* st) {
   typedef typename V2<R>::T R2;
-  const volatile SolverState* vs = st;
-  const int done = vs->done;
-  if (done && !vs->ms_final) return;
+  const int done = !gate_open(st, GATE_ITER);
+  if (done && !st->ms_final) return;
   const int ns = st->nshift;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Vh; i += gridDim.x * blockDim.x) {
     R2 rc[3];
@@ -419,7 +417,7 @@ int launch_finish2(sqcg_ctx* ctx, int nblocks, int fin, int gate, cudaStream_t s
 }
 
 int launch_finish_sr(sqcg_ctx* ctx, int nblocks, int coff, int cn, int gate, cudaStream_t s, bool pdl) {
-  SQCG_CUDA_TRY(launch_kernel(k_finish_sr, kFinishSRBlocks, kFinishSRThreads, 0, s, pdl, ctx->st, ctx->partials,
+  SQCG_CUDA_TRY(launch_kernel(k_finish_sr, finish_sr_blocks(nblocks), kFinishSRThreads, 0, s, pdl, ctx->st, ctx->partials,
                               nblocks, coff, cn, gate, ctx->fin_aux, ctx->fin_cnt));
   return SQCG_OK;
 }

@@ -17,13 +17,33 @@
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Whether this kernel of a captured loop runs; every thread of the block calls it. One thread of the block
+// reads the state (past L1: the finisher that wrote it may have run while this block was resident). All
+// threads reading it, as an earlier version did, sent every warp of the grid to one L2 line: 131 k requests
+// a pass at 32^4 with eight warps per 32 sites, which took 43 us.
+struct GateWords {
+  int done, upd;
+};
+__device__ __forceinline__ GateWords gate_load(const SolverState* st, int gate, bool first) {
+  GateWords w = {0, 0};
+  if (gate != GATE_NONE && first) {
+    const volatile SolverState* v = st;
+    w.done = v->done;
+    w.upd = v->need_update;
+  }
+  return w;
+}
+__device__ __forceinline__ int gate_value(GateWords w, int gate) {
+  return gate == GATE_NONE || (!w.done && (gate == GATE_UPDATE ? w.upd != 0 : gate == GATE_STEP ? w.upd == 0 : true));
+}
 __device__ __forceinline__ bool gate_open(const SolverState* st, int gate) {
   if (gate == GATE_NONE) return true;
-  const volatile SolverState* v = st;
-  if (v->done) return false;
-  if (gate == GATE_UPDATE) return v->need_update != 0;
-  if (gate == GATE_STEP) return v->need_update == 0;
-  return true;
+  __shared__ int open;
+  const bool first = threadIdx.x == 0 && threadIdx.y == 0;
+  const GateWords w = gate_load(st, gate, first);
+  if (first) open = gate_value(w, gate);
+  __syncthreads();
+  return open != 0;
 }
 
 // sum over the block; the result is valid in thread 0. blockDim.x must be a
@@ -262,9 +282,14 @@ __device__ __forceinline__ void block_partial(double v, double* partials) {
 // Second stage: one block of kFinishThreads threads (each adds only a few partials).
 constexpr int kFinishThreads = 1024;
 // the single-reduction step's finisher: a few blocks share the partial sums (finish_partials_sr)
-constexpr int kFinishSRBlocks = 8;
+constexpr int kFinishSRMaxBlocks = 32;  // the last to arrive adds the blocks' totals with one warp
 constexpr int kFinishSRThreads = 256;
-static_assert(3 * kFinishSRBlocks <= 64, "the finisher's per-block slots (fin_aux holds 64)");
+static_assert(3 * kFinishSRMaxBlocks <= 96, "the finisher's per-block slots (fin_aux holds 96)");
+// one block per 512 partials of a sum (two rows of loads a thread), so the time does not grow with them
+inline int finish_sr_blocks(int n) {
+  const int b = (n + 511) / 512;
+  return b < kFinishSRMaxBlocks ? b : kFinishSRMaxBlocks;
+}
 
 __device__ __forceinline__ void finish_partials(SolverState* st, const double* partials, int n, int fin) {
   double s = 0.0;
@@ -462,22 +487,28 @@ __device__ __forceinline__ void finish_partials_sr(SolverState* st, const double
   const int c0 = (int)((long)cn * b / nb), c1 = (int)((long)cn * (b + 1) / nb);
   float2 v[3];
   ffs_block_sums3(partials, a0, coff + c0, c1 - c0, 2 * n + a0, a1 - a0, v);  // v = {d, c, g} of the range
-  __shared__ int last;
-  if (threadIdx.x == 0) {
+  if (threadIdx.x >= 32) return;
+  int last = 1;
+  if (threadIdx.x == 0 && nb > 1) {
 #pragma unroll
     for (int k = 0; k < 3; ++k) aux[3 * b + k] = v[k];
     __threadfence();
     last = atomicAdd(cnt, 1u) == (unsigned)nb - 1u;
   }
-  __syncthreads();
-  if (!last || threadIdx.x != 0) return;
-  __threadfence();
-  float2 t[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-  for (int j = 0; j < nb; ++j)
+  if (nb > 1) {
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    __threadfence();
 #pragma unroll
-    for (int k = 0; k < 3; ++k) t[k] = ffs_add(t[k], __ldcg(&aux[3 * j + k]));
+    for (int k = 0; k < 3; ++k) {
+      v[k] = (int)threadIdx.x < nb ? __ldcg(&aux[3 * threadIdx.x + k]) : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+        v[k] = ffs_add(v[k], make_float2(__shfl_down_sync(0xffffffffu, v[k].x, o), __shfl_down_sync(0xffffffffu, v[k].y, o)));
+    }
+  }
+  if (threadIdx.x != 0) return;
   *cnt = 0u;
-  sr_step(st, ffs_value(t[0]), ffs_value(t[1]), ffs_value(t[2]));
+  sr_step(st, ffs_value(v[0]), ffs_value(v[1]), ffs_value(v[2]));
 }
 
 __device__ __forceinline__ void finish_partials2(SolverState* st, const double* partials, int n, int fin) {
