@@ -16,8 +16,8 @@ void sqcg_set_last_cuda_error(cudaError_t e, const char* what, const char* file,
 int ensure_workspace(sqcg_ctx* ctx) {
   if (ctx->st) return SQCG_OK;
   const size_t n = (size_t)ctx->g.Vh * 3;
-  // the largest grid of any reducing kernel: Dslash uses 128-thread blocks
-  ctx->max_blocks = grid_for(ctx->g.Vh, 128);
+  // the largest grid of any reducing kernel: a Dslash block has 128 sites, a split one 32
+  ctx->max_blocks = grid_for(ctx->g.Vh, 32);
   bool ok = cudaMalloc((void**)&ctx->r64, n * sizeof(double2)) == cudaSuccess &&
             cudaMalloc((void**)&ctx->p64, n * sizeof(double2)) == cudaSuccess &&
             cudaMalloc((void**)&ctx->Ap64, n * sizeof(double2)) == cudaSuccess &&
@@ -114,7 +114,10 @@ int sqcg_create(const int dims[4], int flags, void* cuda_stream, sqcg_ctx** out)
   }
   c->ru_delta = 0.001;
   c->ru_interval = 100;
-  if (cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
     sqcg_set_last_cuda_error(cudaGetLastError(), "cudaStreamCreate", __FILE__, __LINE__);
     free(c);
     return SQCG_ERR_CUDA;

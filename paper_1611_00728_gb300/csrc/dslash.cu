@@ -127,6 +127,96 @@ __global__ void __launch_bounds__(kThreads, (sizeof(R) == 4 && EPI == EPI_SR_DOT
   (void)srs; (void)srq; (void)srr; (void)sdot;
 }
 
+// The same passes with a site's hops split over warps (dslash_split() says where): a block takes 32
+// consecutive output sites; of its SPLIT warps, warp w does 16 / SPLIT of their hops (dslash_part), the
+// partial sums meet in shared memory and warp c < 3 runs the epilogue of colour c.
+//
+// What bounds the one-thread form on a small lattice is the chain of 16 hops in a thread, each waiting for
+// its loads: at 8^4 there are 16 blocks on 152 SMs and a pass takes 7.7 us (FP32, full links) whatever the
+// rest of the chip does. Split, the chain is two hops and eight times the warps are in flight: 2.5 us
+// (FP64 22.8 -> 7.3 us; timed in a graph of 20 launches, links in L2). The gate of a captured loop is read
+// while the hops run and decides at the barrier: a block lives for about two loads, and waiting for the
+// state first would add a third.
+template <typename R, bool RECON, bool EIGHT, int SPLIT>
+__global__ void __launch_bounds__(32 * SPLIT) k_dslash_split(DArgs<R> a) {
+  typedef typename V2<R>::T R2;
+  __shared__ R2 sm[SPLIT][3][32];
+  __shared__ int open;
+  pdl_wait();
+  pdl_launch_dependents();
+  const bool first = threadIdx.x == 0 && threadIdx.y == 0;
+  const GateWords gw = gate_load(a.st, a.gate, first);
+  const int Vh = a.g.Vh;
+  const int i = blockIdx.x * 32 + threadIdx.x, c = threadIdx.y;
+  const bool valid = i < Vh;
+  if (valid) {
+    R2 acc[3];
+    dslash_part<R, RECON, EIGHT, SPLIT>(a, i, threadIdx.y, acc, PlainIn<R2, true>{a.in, Vh});
+#pragma unroll
+    for (int k = 0; k < 3; ++k) sm[threadIdx.y][k][threadIdx.x] = acc[k];
+  }
+  if (first) open = gate_value(gw, a.gate);
+  __syncthreads();
+  if (!open) return;
+  double part = 0.0;                 // FP64 arithmetic: the colour's dot or norm
+  float s0 = 0.f, s1 = 0.f, s2 = 0.f;  // FP32: the colour's <y, out>, <y, q>, |y|^2
+  if (c < 3 && valid) {
+    R2 d = sm[0][c][threadIdx.x];
+#pragma unroll
+    for (int w = 1; w < SPLIT; ++w) {
+      const R2 u = sm[w][c][threadIdx.x];
+      d.x += u.x;
+      d.y += u.y;
+    }
+    const size_t k = (size_t)c * Vh + i;
+    if (a.epi == EPI_PLAIN) {
+      static_cast<R2*>(a.out)[k] = d;
+    } else if (a.epi == EPI_TRUE_RESID) {  // b - sigma x + D in, in FP64
+      const double sig = a.sigma_dev ? *a.sigma_dev : a.sigma;
+      const double2 xc = __ldg(static_cast<const double2*>(a.y) + k);
+      const double2 bc = __ldg(a.b + k);
+      const double re = bc.x - sig * xc.x + (double)d.x, im = bc.y - sig * xc.y + (double)d.y;
+      if (a.out_f32) {
+        const float2 o = make_float2((float)re, (float)im);
+        static_cast<float2*>(a.out)[k] = o;
+        if (a.out2) static_cast<float2*>(a.out2)[k] = o;
+      } else {
+        const double2 o = make_double2(re, im);
+        static_cast<double2*>(a.out)[k] = o;
+        if (a.out2) static_cast<double2*>(a.out2)[k] = o;
+      }
+      part = re * re + im * im;
+    } else {  // sigma y - D in, and its sums
+      const R sig = (R)(a.sigma_dev ? *a.sigma_dev : a.sigma);
+      const R2 yc = ldg2(static_cast<const R2*>(a.y) + k);
+      const R2 o = mk<R2>(sig * yc.x - d.x, sig * yc.y - d.y);
+      static_cast<R2*>(a.out)[k] = o;
+      const R dot = fma(yc.x, o.x, yc.y * o.y);
+      part = (double)dot;
+      s0 = (float)dot;
+      if (a.epi == EPI_SR_DOTS || a.epi == EPI_SR_DOTS2) s2 = (float)fma(yc.x, yc.x, yc.y * yc.y);
+      if (a.epi == EPI_SR_DOTS) {
+        const R2 qc = ldg2(static_cast<const R2*>(a.y3) + k);
+        s1 = (float)fma(yc.x, qc.x, yc.y * qc.y);
+      }
+    }
+  }
+  if (a.fin == FIN_NONE || a.epi == EPI_PLAIN || a.epi == EPI_NORMAL) return;
+  if (sizeof(R) == 8) {
+    const double t = colour_sum(part);
+    if (first) a.partials[blockIdx.x] = t;
+  } else {
+    float2 v[3] = {make_float2(s0, 0.f), make_float2(s1, 0.f), make_float2(s2, 0.f)};
+    colour_sum_ffs<3>(v);
+    if (first) {
+      float2* slot = ffs_slots(a.partials);
+      slot[blockIdx.x] = v[0];
+      if (a.epi == EPI_SR_DOTS) slot[gridDim.x + blockIdx.x] = v[1];
+      if (a.epi != EPI_NORMAL_DOT) slot[2 * gridDim.x + blockIdx.x] = v[2];
+    }
+  }
+}
+
 template <typename R, typename RO, bool RECON, bool EIGHT>
 int launch_t(sqcg_ctx* ctx, const DslashLaunch& L, cudaStream_t s) {
   typedef typename V2<R>::T R2;
@@ -160,9 +250,12 @@ int launch_t(sqcg_ctx* ctx, const DslashLaunch& L, cudaStream_t s) {
   a.fin = L.fin;
   if ((L.gate != GATE_NONE || L.fin != FIN_NONE) && (ctx->st == nullptr || ctx->partials == nullptr))
     return SQCG_ERR_INVALID_ARG;
-  const int grid = grid_for(ctx->g.Vh, kThreads);
+  a.epi = L.epi;
+  a.out_f32 = sizeof(RO) == 4;
   const bool sr = L.epi == EPI_SR_DOTS || L.epi == EPI_SR_DOTS2;
   const bool reduces = (L.epi == EPI_NORMAL_DOT || sr || L.epi == EPI_TRUE_RESID) && L.fin != FIN_NONE;
+  const int split = dslash_split(ctx, L.prec, L.gate != GATE_NONE);
+  const int grid = grid_for(ctx->g.Vh, split > 1 ? 32 : kThreads);
   if (reduces && grid > ctx->max_blocks) return SQCG_ERR_INVALID_ARG;  // partials hold 3 sums and more
   // programmatic dependent launch where the caller says a kernel precedes this one, and for the
   // finisher, which always follows the Dslash
@@ -177,7 +270,12 @@ int launch_t(sqcg_ctx* ctx, const DslashLaunch& L, cudaStream_t s) {
     case EPI_SR_DOTS2: kern = k_dslash<R, RO, RECON, EIGHT, EPI_SR_DOTS2>; break;
     default: return SQCG_ERR_INVALID_ARG;
   }
-  SQCG_CUDA_TRY(launch_kernel(kern, grid, kThreads, 0, s, pdl, a));
+  dim3 block(kThreads);
+  if (split > 1) {
+    block = dim3(32, split);
+    kern = split == 4 ? k_dslash_split<R, RECON, EIGHT, 4> : k_dslash_split<R, RECON, EIGHT, 8>;
+  }
+  SQCG_CUDA_TRY(launch_kernel(kern, grid, block, 0, s, pdl, a));
   if (reduces)
     return L.epi == EPI_SR_DOTS ? launch_finish_sr(ctx, grid, grid, grid, L.gate, s, fpdl)
            : L.epi == EPI_SR_DOTS2
@@ -198,6 +296,27 @@ int launch_r(sqcg_ctx* ctx, const DslashLaunch& L, cudaStream_t s) {
 }
 
 }  // namespace
+
+// Measured on the GB300 (us a pass, links in L2 up to 20^4; 128-site tiles a SM in brackets), with
+// 1 / 4 / 8 warps a site group:
+//   FP32 full links   8^4 [0.1] 7.7/5.1/2.5, 16^4 [1.7] 8.0/6.2/5.5, 20^4 [4.1] 14.6/17.0/11.3,
+//                     24^4 [8.5] 33.2/41.1/31.4, 32^4 [27] 97.8/119.5/91.0: 8 everywhere outside captured
+//                     loops (on large lattices eight short chains keep more of the link loads in flight than
+//                     one thread can hold). Inside them a block also waits for the pass before it, and the
+//                     mixed CG's step takes 52.6/52.0/49.3 at 20^4 but 235/270/261 at 32^4
+//   FP32 12-real      8^4 5.2/3.3/2.5, 10x12x14x16 [0.7] 5.3/3.8/3.5, 16^4 5.9/5.0/5.5, 20^4 8.8/10.2/11.8,
+//                     32^4 78.8/83.1/82.9 (CG step: 12^4 [0.5] 24.4/19.6/18.6, 14^4 [1.0] 24.2/21.5/22.7,
+//                     16^4 25.7/25.3/26.1, 18^4 [2.7] 28.2/32.7/32.1); 8-way: 24^4 32.9/29.4/29.2,
+//                     28^4 [16] 46.3/50.5/50.9
+//   FP64              8^4 22.8/8.5/7.3, 10x12x14x16 23.1/16.4/17.6, 16^4 37.8/35.9/37.8, 20^4 99.6/85.5/89.4,
+//                     24^4 169.6/170.6/179.0 (there the FP64 pipe is the bound)
+//   float-float       8^4 14.4/5.1/3.8, 16^4 16.5/12.2/13.5, 24^4 85.9/68.0/72.8, 28^4 114.2/118.1/131.2
+int dslash_split(const sqcg_ctx* ctx, int prec, bool gated) {
+  const int tiles = grid_for(ctx->g.Vh, kThreads), nsm = ctx->nsm;
+  if (prec == SQCG_F32 && !ctx->recon) return gated && tiles > 5 * nsm ? 1 : 8;
+  if (prec == SQCG_F32) return 4 * tiles <= 3 * nsm ? 8 : tiles <= (ctx->eightway && !gated ? 9 : 2) * nsm ? 4 : 1;
+  return 2 * tiles <= nsm ? 8 : tiles <= (prec == SQCG_FF ? 10 : 5) * nsm ? 4 : 1;
+}
 
 int launch_dslash(sqcg_ctx* ctx, const DslashLaunch& L, cudaStream_t s) {
   if (!ctx->have_links) return SQCG_ERR_NO_LINKS;

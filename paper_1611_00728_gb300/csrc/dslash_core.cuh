@@ -105,6 +105,7 @@ struct DArgs {
   SolverState* st;
   double* partials;
   int gate, fin;
+  int epi, out_f32;  // the split kernel: its epilogue (DslashEpi), and whether out is FP32
 };
 
 // D at output site i of parity a.par; returns the three colour components.
@@ -203,6 +204,67 @@ __device__ __forceinline__ void dslash_site_in(const DArgs<R>& a, int i, typenam
         }
       }
     }
+  }
+}
+
+// The share of D at output site i of one of SPLIT warps that work on the same 32 sites: hops
+// part * 16 / SPLIT and following, in the order 4 mu + 2 (long) + (backward). part is uniform over the
+// warp, so every branch here is.
+template <typename R, bool RECON, bool EIGHT, int SPLIT, typename In>
+__device__ __forceinline__ void dslash_part(const DArgs<R>& a, int i, int part, typename V2<R>::T (&acc)[3],
+                                            const In& in_at) {
+  typedef typename V2<R>::T R2;
+  const Geom& g = a.g;
+  const int Vh = g.Vh;
+  const int xh = i % g.Lxh;
+  int r = i / g.Lxh;
+  const int y = r % g.Ly;
+  r /= g.Ly;
+  const int z = r % g.Lz;
+  const int t = r / g.Lz;
+  const int x = 2 * xh + ((y + z + t + a.par) & 1);
+  const int row = i - xh;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) acc[c] = mk<R2>(R(0), R(0));
+  constexpr int NH = 16 / SPLIT;
+#pragma unroll
+  for (int j = 0; j < NH; ++j) {
+    const int h = part * NH + j;
+    const int mu = h >> 2, k = (h >> 1) & 1, bwd = h & 1;
+    const int d = k ? 3 : 1;
+    int nb;
+    if (mu == 0) {
+      int xn = bwd ? x - d : x + d;
+      if (xn >= g.Lx) xn -= g.Lx;
+      if (xn < 0) xn += g.Lx;
+      nb = row + (xn >> 1);
+    } else {
+      const int cmu = (mu == 1) ? y : (mu == 2) ? z : t;
+      const int Lmu = (mu == 1) ? g.Ly : (mu == 2) ? g.Lz : g.Lt;
+      const int smu = (mu == 1) ? g.sy : (mu == 2) ? g.sz : g.st;
+      nb = bwd ? i - d * smu : i + d * smu;
+      if (!bwd && cmu + d >= Lmu) nb -= Lmu * smu;
+      if (bwd && cmu - d < 0) nb += Lmu * smu;
+    }
+    R2 U[9], v[3];
+    in_at(v, nb);
+    const bool own = EIGHT || !bwd;  // the link is read at the thread's own index
+    if (k == 0) {
+      const R2* base = !bwd ? a.fat_p : EIGHT ? a.fatb_p : a.fat_q;
+      load_link<R, R2, false>(U, base + (size_t)mu * 9 * Vh, Vh, own ? i : nb, R(1));
+    } else {
+      R inv_s = R(1);
+      if (RECON) {  // eta_mu(n) and the boundary sign of the hop (see dslash_site_in)
+        const int e = (mu == 0) ? 0 : (mu == 1) ? x : (mu == 2) ? x + y : x + y + z;
+        inv_s = (e & 1) ? -a.inv_s0 : a.inv_s0;
+        if (mu == 3 && g.apbc && (bwd ? t < 3 : t + 3 >= g.Lt)) inv_s = -inv_s;
+        if (EIGHT && bwd) inv_s = -inv_s;
+      }
+      const R2* base = !bwd ? a.lng_p : EIGHT ? a.lngb_p : a.lng_q;
+      load_link<R, R2, RECON>(U, base + (size_t)mu * a.nl * Vh, Vh, own ? i : nb, inv_s);
+    }
+    if (own) acc_mv<R>(acc, U, v);
+    else sub_mdv<R>(acc, U, v);
   }
 }
 

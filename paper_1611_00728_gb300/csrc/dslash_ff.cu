@@ -135,6 +135,110 @@ __global__ void __launch_bounds__(kThreads) k_dslash_ff(FArgs a) {
   }
 }
 
+// h += (bh, bl) in float-float
+__device__ __forceinline__ void ff_add(float& h, float& l, float bh, float bl) {
+  const float s = __fadd_rn(h, bh);
+  const float v = __fsub_rn(s, h);
+  float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, v)), __fsub_rn(bh, v));
+  e = __fadd_rn(e, __fadd_rn(l, bl));
+  h = __fadd_rn(s, e);
+  l = __fsub_rn(e, __fsub_rn(h, s));
+}
+
+// The same passes for small lattices, split as k_dslash_split (dslash.cu): a block is 32 sites x SPLIT
+// warps, warp w takes 16 / SPLIT of the hops (in the order 4 mu + 2 (long) + (backward)), warp c < 3 sums
+// and finishes colour c.
+template <int SPLIT>
+__global__ void __launch_bounds__(32 * SPLIT) k_dslash_ff_split(FArgs a, int true_resid) {
+  __shared__ float4 sm[SPLIT][3][32];
+  if (!gate_open(a.st, a.gate)) return;
+  const Geom& g = a.g;
+  const int Vh = g.Vh;
+  const int i = blockIdx.x * 32 + threadIdx.x, c = threadIdx.y;
+  const bool valid = i < Vh;
+  if (valid) {
+    const int xh = i % g.Lxh;
+    int r = i / g.Lxh;
+    const int y = r % g.Ly;
+    r /= g.Ly;
+    const int z = r % g.Lz;
+    const int t = r / g.Lz;
+    const int x = 2 * xh + ((y + z + t + a.par) & 1);
+    const int row = i - xh;
+    float4 acc[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    constexpr int NH = 16 / SPLIT;
+#pragma unroll
+    for (int j = 0; j < NH; ++j) {
+      const int h = threadIdx.y * NH + j;
+      const int mu = h >> 2, k = (h >> 1) & 1, bwd = h & 1;
+      const int d = k ? 3 : 1;
+      int nb;
+      if (mu == 0) {
+        int xn = bwd ? x - d : x + d;
+        if (xn >= g.Lx) xn -= g.Lx;
+        if (xn < 0) xn += g.Lx;
+        nb = row + (xn >> 1);
+      } else {
+        const int cmu = (mu == 1) ? y : (mu == 2) ? z : t;
+        const int Lmu = (mu == 1) ? g.Ly : (mu == 2) ? g.Lz : g.Lt;
+        const int smu = (mu == 1) ? g.sy : (mu == 2) ? g.sz : g.st;
+        nb = bwd ? i - d * smu : i + d * smu;
+        if (!bwd && cmu + d >= Lmu) nb -= Lmu * smu;
+        if (bwd && cmu - d < 0) nb += Lmu * smu;
+      }
+      const float4* base = (k ? (bwd ? a.lng_q : a.lng_p) : (bwd ? a.fat_q : a.fat_p)) + (size_t)mu * 9 * Vh;
+      float4 U[9], v[3];
+      ld_link(U, base, Vh, bwd ? nb : i);
+      ld_vec(v, a.in, Vh, nb);
+      if (bwd) ff_mdv_sub(acc, U, v);
+      else ff_mv(acc, U, v);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      ff_norm(acc[k].x, acc[k].y);
+      ff_norm(acc[k].z, acc[k].w);
+      sm[threadIdx.y][k][threadIdx.x] = acc[k];
+    }
+  }
+  __syncthreads();
+  double part = 0.0;
+  if (c < 3 && valid) {
+    float4 d = sm[0][c][threadIdx.x];
+#pragma unroll
+    for (int w = 1; w < SPLIT; ++w) {
+      const float4 u = sm[w][c][threadIdx.x];
+      ff_add(d.x, d.y, u.x, u.y);
+      ff_add(d.z, d.w, u.z, u.w);
+    }
+    const size_t k = (size_t)c * Vh + i;
+    if (!true_resid) {
+      a.out_ff[k] = d;
+    } else {  // r = b - sigma x + D in, the sum formed in FP64
+      const double sig = a.sigma_dev ? *a.sigma_dev : a.sigma;
+      const double2 xc = __ldg(a.x + k);
+      const double2 bc = __ldg(a.b + k);
+      const double re = bc.x - sig * xc.x + ((double)d.x + (double)d.y);
+      const double im = bc.y - sig * xc.y + ((double)d.z + (double)d.w);
+      a.out32[k] = make_float2((float)re, (float)im);
+      part = re * re + im * im;
+    }
+  }
+  if (true_resid && a.fin != FIN_NONE) {
+    const double s = colour_sum(part);
+    if (threadIdx.x == 0 && threadIdx.y == 0) a.partials[blockIdx.x] = s;
+  }
+}
+
+int launch_ff_split(int split, int grid, const FArgs& a, int true_resid, cudaStream_t s) {
+  const dim3 block(32, split);
+  if (split == 4) k_dslash_ff_split<4><<<grid, block, 0, s>>>(a, true_resid);
+  else k_dslash_ff_split<8><<<grid, block, 0, s>>>(a, true_resid);
+  SQCG_CUDA_TRY(cudaGetLastError());
+  return SQCG_OK;
+}
+
 __global__ void k_split_ff(const double2* __restrict__ in, float4* __restrict__ out, size_t n) {
   for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x)
     out[k] = split_ff(in[k]);
@@ -179,20 +283,26 @@ int launch_dslash_ff(sqcg_ctx* ctx, const FFLaunch& L, cudaStream_t s) {
   a.gate = L.gate;
   a.fin = L.fin;
   if ((L.gate != GATE_NONE || L.fin != FIN_NONE) && (!ctx->st || !ctx->partials)) return SQCG_ERR_INVALID_ARG;
-  const int grid = grid_for(ctx->g.Vh, kThreads);
+  const int split = dslash_split(ctx, SQCG_FF, L.gate != GATE_NONE);
+  const int grid = grid_for(ctx->g.Vh, split > 1 ? 32 : kThreads);
   if (L.true_resid) {
     if (!L.out32 || !L.x || !L.b) return SQCG_ERR_INVALID_ARG;
     if (L.fin != FIN_NONE && grid > ctx->max_blocks) return SQCG_ERR_INVALID_ARG;
     a.out32 = static_cast<float2*>(L.out32);
     a.x = static_cast<const double2*>(L.x);
     a.b = static_cast<const double2*>(L.b);
-    k_dslash_ff<FFE_TRUE_RESID><<<grid, kThreads, 0, s>>>(a);
-    SQCG_CUDA_TRY(cudaGetLastError());
+    if (split > 1) {
+      SQCG_TRY(launch_ff_split(split, grid, a, 1, s));
+    } else {
+      k_dslash_ff<FFE_TRUE_RESID><<<grid, kThreads, 0, s>>>(a);
+      SQCG_CUDA_TRY(cudaGetLastError());
+    }
     if (L.fin != FIN_NONE) return launch_finish(ctx, grid, L.fin, L.gate, s);
     return SQCG_OK;
   }
   if (!L.out_ff) return SQCG_ERR_INVALID_ARG;
   a.out_ff = static_cast<float4*>(L.out_ff);
+  if (split > 1) return launch_ff_split(split, grid, a, 0, s);
   k_dslash_ff<FFE_PLAIN><<<grid, kThreads, 0, s>>>(a);
   SQCG_CUDA_TRY(cudaGetLastError());
   return SQCG_OK;

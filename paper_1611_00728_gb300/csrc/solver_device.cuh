@@ -399,6 +399,37 @@ __device__ __forceinline__ void block_sum_ffs(float2 (&v)[N]) {
   }
 }
 
+// The sums over the three colour warps of a split block: totals in thread (0, 0), fixed order.
+template <int N>
+__device__ __forceinline__ void colour_sum_ffs(float2 (&v)[N]) {
+  __shared__ float2 part[N][3];
+  if (threadIdx.y < 3) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < N; ++k)
+        v[k] = ffs_add(v[k], make_float2(__shfl_down_sync(0xffffffffu, v[k].x, o), __shfl_down_sync(0xffffffffu, v[k].y, o)));
+    if (threadIdx.x == 0)
+#pragma unroll
+      for (int k = 0; k < N; ++k) part[k][threadIdx.y] = v[k];
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && threadIdx.y == 0)
+#pragma unroll
+    for (int k = 0; k < N; ++k) v[k] = ffs_add(ffs_add(part[k][0], part[k][1]), part[k][2]);
+}
+
+__device__ __forceinline__ double colour_sum(double v) {
+  __shared__ double part[3];
+  if (threadIdx.y < 3) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (threadIdx.x == 0) part[threadIdx.y] = v;
+  }
+  __syncthreads();
+  return part[0] + part[1] + part[2];
+}
+
 // Three float-float sums over slots [o0, o0 + n), [o1, o1 + n1), [o2, o2 + n) of ffs partials, each
 // thread taking every blockDim.x-th slot into four interleaved accumulators (four rows of loads in
 // flight), merged in a fixed order; then the block tree. Totals in thread 0 as FP64.

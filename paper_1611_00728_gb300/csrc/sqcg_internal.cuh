@@ -161,6 +161,7 @@ struct sqcg_ctx {
   Geom g;
   cudaStream_t stream;
   cudaStream_t cap_stream;  // private stream used only to capture graphs
+  int nsm;                  // SMs of the device the context was created on
 
   bool have_links;
   bool recon;
@@ -262,6 +263,9 @@ struct DslashLaunch {
 };
 
 int launch_dslash(sqcg_ctx* ctx, const DslashLaunch& L, cudaStream_t s);
+// warps that share a site's hops in the Dslash of this precision (SQCG_F64, SQCG_F32, SQCG_FF) on this
+// lattice; 1: one thread does them all. gated: a pass of a captured loop, which reads the solver state first
+int dslash_split(const sqcg_ctx* ctx, int prec, bool gated);
 
 int launch_cg_update_x(sqcg_ctx* ctx, int mixed, double2* x, cudaStream_t s);
 int launch_loop_control(sqcg_ctx* ctx, cudaStream_t s);

@@ -220,3 +220,28 @@ def test_float_float_pack_round_trip_and_free_field(sqcg):
         got = lat.unpack(out, sqcg.FF)
     want = oracle.dslash(L, fat, lng, pw, 0)
     assert np.linalg.norm(got - want) / np.linalg.norm(want) <= 1e-13
+
+
+# Each form of the split Dslash at a remainder of its 32-site groups (SMs: 152): 78.75 groups and a quarter of
+# an SM's tile (8 warps a group in every precision), 367.5 groups (4 warps in FP64 and float-float), 600.25
+# groups (4 warps in the 12-real FP32 form), and 3 tiles a SM (one thread a site for 12-real FP32).
+@pytest.mark.parametrize("L", [(6, 6, 10, 14), (14, 14, 10, 12), (14, 14, 14, 14), (18, 18, 18, 20)])
+@pytest.mark.parametrize("eight", [False, True])
+@pytest.mark.parametrize("recon", [False, True])
+def test_split_dslash_remainders(sqcg, links_cache, L, recon, eight):
+    """D on both parities and the normal operator at lattice sizes on both sides of every line of the rule that
+    chooses how many warps share a site's hops, against the oracle at the bars above (float-float: 1e-12)."""
+    fat, lng = links_cache(L, 1003)
+    psi = synth.gaussian_source(L, 2003)
+    want = [oracle.dslash(L, fat, lng, psi, par) for par in (0, 1)]
+    want_a = oracle.normal_op(L, fat, lng, 0.04, psi)
+    with sqcg.Lattice(L) as lat:
+        lat.load_links(fat, lng, recon12=recon, eight_way=eight)
+        for prec, bar in ((0, 1e-12), (1, 1e-5), (2, 1e-12)):
+            d_in, out = lat.pack(psi, prec), lat.new_spinor(prec)
+            for par in (0, 1):
+                lat.dslash(par, d_in, out, prec)
+                assert rel(lat.unpack(out, prec), want[par]) <= bar, (prec, par)
+            if prec != 2:
+                lat.normal_op(0.04, d_in, out, prec)
+                assert rel(lat.unpack(out, prec), want_a) <= bar, prec
