@@ -26,9 +26,9 @@ constexpr int kSRKernelsPerIter = 4;  // enqueue_sr_head (2 + finisher) + the up
 // about 3.4 us and a WHILE pass 3.5 us (a CUDA-graph probe of empty bodies), against ~200 us a step
 // at 32^4; the 32^4 mixed solve took 44.6, 43.5, 43.0 and 42.9 ms with 1, 2, 4 and 8 steps a pass.
 constexpr int kSRUnroll = 8;
-// the persistent loop runs where a parity has at most this many 128-site tiles a SM (measured
-// crossover on the GB300: 20^4, 4.1 tiles a SM, gains; 24^4, 8.5, loses)
-constexpr int kPersistentMaxTilesPerSM = 5;
+// the persistent loop runs where a parity has at most this many 32-site groups a SM. Measured, us an iteration,
+// persistent / graph loop: 18^4 (11 groups) 22.6 / 27.8, 20^4 (17) 36.1 / 40.3, 22^4 (25) 83 / 63
+constexpr int kPersistentMaxGroupsPerSM = 20;
 constexpr int kSRKernelsPerUpdatePersistent = 4;  // flush, Dslash pair, finisher (no head)
 constexpr int kSRKernelsPerUpdate = 7;  // enqueue_sr_reliable: flush, 2 FP64 + finisher, 2 FP32 + finisher
 
@@ -373,44 +373,40 @@ int run_eager(sqcg_ctx* ctx, int kind, int mixed, const void* b, void* const* x,
   return SQCG_OK;
 }
 
-// The single-reduction mixed loop as the persistent kernel (cg_persistent.cu): one launch runs the
-// iterations up to the next reliable update; the host reads the state, runs the true-residual pass
-// and launches again. *segments = persistent launches, *updates_run = true-residual passes.
-//
-// Which loop runs: the persistent kernel where every 128-site tile of a parity has its own resident
-// block (each phase is one wave, so a grid barrier replaces a kernel boundary at no cost in balance,
-// and the launch and finisher latency it removes dominates small lattices); the graph-launched
-// loop on larger lattices, where a phase takes several waves and the barrier across all resident
-// blocks costs more than the kernel boundaries it replaces. SQCG_PERSISTENT=0 or 1 forces one.
+// Which loop runs: the persistent kernel (cg_persistent.cu) on small lattices, where launch and finisher
+// latency dominate, the graph-launched loop on larger ones, where a phase is long and the 24 warps a SM that
+// its registers allow hold fewer loads in flight than the Dslash kernels. The line is at
+// kPersistentMaxGroupsPerSM. SQCG_PERSISTENT=0 or 1 forces one.
 bool use_persistent(sqcg_ctx* ctx) {
   const char* m = getenv("SQCG_PERSISTENT");
   if (m && strcmp(m, "0") == 0) return false;
-  const int G = persistent_grid(ctx);
-  if (G <= 0) return false;
-  if (m && strcmp(m, "1") == 0) return true;
-  int dev = 0, nsm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  const int ntiles = grid_for(ctx->g.Vh, 128);
-  return G >= ntiles && ntiles <= kPersistentMaxTilesPerSM * nsm;  // one block a tile, few a SM
+  if (!(m && strcmp(m, "1") == 0) && grid_for(ctx->g.Vh, 32) > kPersistentMaxGroupsPerSM * ctx->nsm) return false;
+  return persistent_grid(ctx) > 0;
 }
 
-int run_persistent(sqcg_ctx* ctx, const void* b, void* x, int max_iter, cudaStream_t s, int* segments,
-                   int* updates_run) {
+// The single-reduction mixed loop as the persistent kernel: a launch runs the iterations up to the next
+// reliable update or the end, the true-residual pass follows, gated by the state it left. As many
+// such segments are queued at once as the residual's way down takes at the trigger's factor, so the host
+// reads the state once for a usual solve; segments past the end exit at once. *segments: how many ran or were
+// gated off. The last partial solution is flushed behind every queue.
+int run_persistent(sqcg_ctx* ctx, const void* b, void* x, double tol, int max_iter, cudaStream_t s, int* segments) {
   SolverState* h = ctx->st_host;
   h->use_if = 0;
   SQCG_TRY(write_state(ctx, s));
   *segments = 0;
-  *updates_run = 0;
-  for (int k = 0; k < max_iter + 4; ++k) {
-    SQCG_TRY(launch_sr_persistent(ctx, max_iter + 2 - h->iter, s));
-    *segments += 1;
+  int queue = tol < 1.0 ? (int)ceil(log(tol) / log(ctx->ru_delta)) : 1;
+  if (queue < 1) queue = 1;
+  if (queue > 8) queue = 8;
+  while (*segments < max_iter + 4) {
+    for (int k = 0; k < queue; ++k) {
+      SQCG_TRY(launch_sr_persistent(ctx, max_iter + 2, s));
+      SQCG_TRY(enqueue_sr_reliable(ctx, b, x, s, false));
+    }
+    *segments += queue;
+    SQCG_TRY(launch_flush_partial_x(ctx, (double2*)x, GATE_NONE, s));
     SQCG_TRY(read_state(ctx, s));
-    if (h->done || !h->need_update) break;
-    SQCG_TRY(enqueue_sr_reliable(ctx, b, x, s, false));
-    *updates_run += 1;
+    if (h->done) break;
+    queue = 1;
   }
   return SQCG_OK;
 }
@@ -460,7 +456,7 @@ int cg_solve_sigma(sqcg_ctx* ctx, double sigma, const void* b, void* x, double t
   if (h->pAp == 0.0) {
     const int wp = mixed ? SQCG_F32 : SQCG_F64;
     SQCG_TRY(layout_convert(ctx, SQCG_F64, b, wp, r0, s));
-    SQCG_TRY(layout_convert(ctx, SQCG_F64, b, wp, p0, s));
+    if (!mixed) SQCG_TRY(layout_convert(ctx, SQCG_F64, b, wp, p0, s));  // the mixed loop's p starts at zero
     // the initial-residual step of the device state, with |r|^2 = |b|^2
     const double v = h->bb;
     if (!isfinite(v)) {
@@ -481,7 +477,7 @@ int cg_solve_sigma(sqcg_ctx* ctx, double sigma, const void* b, void* x, double t
     SQCG_TRY(launch_dslash(ctx, L, s));
     L = DslashLaunch{};
     L.out_parity = 0; L.prec = SQCG_F64; L.out_prec = mixed ? SQCG_F32 : SQCG_F64; L.epi = EPI_TRUE_RESID;
-    L.in = ctx->tmp64; L.out = r0; L.out2 = p0;
+    L.in = ctx->tmp64; L.out = r0; L.out2 = mixed ? nullptr : p0;
     L.y = x; L.b = b; L.sigma = sigma; L.fin = FIN_INIT;
     SQCG_TRY(launch_dslash(ctx, L, s));
     SQCG_TRY(read_state(ctx, s));
@@ -511,9 +507,9 @@ int cg_solve_sigma(sqcg_ctx* ctx, double sigma, const void* b, void* x, double t
       SQCG_CUDA_TRY(cudaMemsetAsync(ctx->partials + sr_update_partials(ctx), 0,
                                     (size_t)ctx->max_blocks * sizeof(double), s));
     }
-    int segments = -1, pupdates = 0;
+    int segments = -1;
     if (mixed && !eager_mode() && use_persistent(ctx)) {
-      SQCG_TRY(run_persistent(ctx, b, x, max_iter, s, &segments, &pupdates));
+      SQCG_TRY(run_persistent(ctx, b, x, tol, max_iter, s, &segments));
     } else if (eager_mode()) {
       SQCG_TRY(run_eager(ctx, kind, mixed, b, xs, 1, max_iter, s, &loops));
     } else {
@@ -521,15 +517,14 @@ int cg_solve_sigma(sqcg_ctx* ctx, double sigma, const void* b, void* x, double t
       SQCG_TRY(capture(ctx, kind, mixed, b, xs, 1, &g));
       SQCG_TRY(run_loop(ctx, g, max_iter, s, &loops));
     }
-    if (mixed) {  // whatever the partial solution still holds (nothing after a converged update)
+    if (mixed && segments >= 0) {  // persistent launches, true-residual passes, final flush
+      launches += segments * (1 + kSRKernelsPerUpdatePersistent) + 1;
+    } else if (mixed) {  // whatever the partial solution still holds (nothing after a converged update)
       SQCG_TRY(launch_flush_partial_x(ctx, (double2*)x, GATE_NONE, s));
       SQCG_CUDA_TRY(cudaStreamSynchronize(s));
-      if (segments >= 0)  // persistent launches, true-residual passes, final flush
-        launches += segments + pupdates * kSRKernelsPerUpdatePersistent + 1;
-      else
-        launches += eager_mode() ? loops * kSRKernelsPerIter + h->updates * kSRKernelsPerUpdate + 1
-                                 : loops * (kSRUnroll * kSRKernelsPerIter + 1) +  // passes: steps, control
-                                       h->updates * (kSRKernelsPerUpdate + 1) + 1;  // IF bodies; final flush
+      launches += eager_mode() ? loops * kSRKernelsPerIter + h->updates * kSRKernelsPerUpdate + 1
+                               : loops * (kSRUnroll * kSRKernelsPerIter + 1) +  // passes: steps, control
+                                     h->updates * (kSRKernelsPerUpdate + 1) + 1;  // IF bodies; final flush
     } else {
       launches += loops * kCGKernelsPerIter + h->updates * kCGKernelsPerUpdate;
     }

@@ -196,8 +196,8 @@ struct sqcg_ctx {
   int max_blocks;
   int blas_grid;  // blocks of the streaming BLAS kernels (0 until first use)
   int pers_grid;        // blocks of the persistent CG loop (0 until first use, -1 unavailable)
-  double* pers_part;    // its partial sums: [3][pers_grid] step sums, [2][pers_grid] cross terms
-  unsigned* pers_bar;   // its grid-barrier words
+  const void* pers_fn;  // the kernel (link form and lattice size) that the grid was found for
+  void* pers_sync;      // its posted sums and grid-barrier words
   float2* pers_rq;      // its second buffers of r and q ([3][Vh] each)
   SolverState* st;       // device
   SolverState* st_host;  // pinned host mirror

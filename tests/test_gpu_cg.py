@@ -713,3 +713,53 @@ def test_mixed_cg_update_arithmetic(sqcg, links_cache, arith, L, m, tol):
     res = oracle.true_rel_residual(L, fat, lng, 4 * m * m, b, x)
     assert res <= tol
     assert abs(res - info.true_rel_resid) <= 1e-3 * tol, (res, info.true_rel_resid)
+
+
+# Every form of the persistent loop at a remainder of its 32-site groups (152 SMs): fewer groups than SMs (79, the
+# last with 24 sites), three groups a block (420), four (601, the last with 8 sites), eleven (1641).
+@pytest.mark.parametrize("L,recon,eight", [((6, 6, 10, 14), False, False), ((6, 6, 10, 14), True, True),
+                                           ((10, 12, 14, 16), True, False), ((10, 12, 14, 16), False, True),
+                                           ((14, 14, 14, 14), True, False), ((14, 14, 14, 14), False, False),
+                                           ((18, 18, 18, 18), True, False), ((18, 18, 18, 18), False, False)])
+def test_persistent_loop_by_groups_per_block(sqcg, links_cache, monkeypatch, L, recon, eight):
+    """The persistent loop reaches the tolerance on the oracle's own residual in the graph loop's iterations (both
+    form the same CG iterates; sums and their rounding differ), also from a nonzero start."""
+    m, tol = 0.05, 1e-9
+    fat, lng = links_cache(L, 1007)
+    b = synth.gaussian_source(L, 2700)
+    with sqcg.Lattice(L) as lat:
+        lat.load_links(fat, lng, recon12=recon, eight_way=eight)
+        db = lat.pack(b)
+        iters = []
+        for loop in ("0", "1"):
+            monkeypatch.setenv("SQCG_PERSISTENT", loop)
+            x = lat.new_spinor()
+            info = lat.cg_solve(m, db, x, tol=tol, mode=sqcg.MODE_MIXED)
+            assert info.status == 0
+            assert oracle.true_rel_residual(L, fat, lng, 4 * m * m, b, lat.unpack(x)) <= tol
+            iters.append(info.iters)
+        assert abs(iters[0] - iters[1]) <= 2, iters
+        x = lat.pack(1e-3 * b)
+        info = lat.cg_solve(m, db, x, tol=tol, mode=sqcg.MODE_MIXED)
+        assert info.status == 0
+        assert oracle.true_rel_residual(L, fat, lng, 4 * m * m, b, lat.unpack(x)) <= tol
+
+
+@pytest.mark.parametrize("power", [-50, 50])
+def test_persistent_loop_outside_the_float_float_step(sqcg, links_cache, monkeypatch, power):
+    """A source scaled by a power of two (exact in every precision) far enough that |r|^2 leaves the range of the
+    float-float scalar step: the FP64 step takes over and the solve takes the unscaled one's iterations."""
+    L, m, tol = (8, 8, 8, 8), 0.1, 1e-3
+    fat, lng = links_cache(L, 1001)
+    b = synth.gaussian_source(L, 2701)
+    monkeypatch.setenv("SQCG_PERSISTENT", "1")
+    with sqcg.Lattice(L) as lat:
+        lat.load_links(fat, lng)
+        out = []
+        for scale in (1.0, 2.0 ** power):
+            x = lat.new_spinor()
+            info = lat.cg_solve(m, lat.pack(scale * b), x, tol=tol, mode=sqcg.MODE_MIXED)
+            assert info.status == 0
+            out.append((info.iters, lat.unpack(x) / scale))
+        assert out[0][0] == out[1][0]
+        assert rel(out[1][1], out[0][1]) <= 1e-5  # FP32 vectors, scalars rounded to FP32 from either step
