@@ -133,14 +133,16 @@ __device__ __forceinline__ void apply_link(const float2 (&u)[9], bool dag, const
 // convolution layer
 // ---------------------------------------------------------------------------
 enum InMode { IN_FULL = 0, IN_EVEN_SCALED = 1 };
-enum OutMode { OUT_FULL = 0, OUT_GATE_TRAIN = 1, OUT_GATE_INFER = 2, OUT_EVEN_SCALED = 3 };
+enum OutMode { OUT_GATE_BWD = 0, OUT_GATE_TRAIN = 1, OUT_GATE_INFER = 2, OUT_EVEN_SCALED = 3 };
 
 struct ConvArgs {
   Geom g;
   const float2* fat[2];   // FP32 fat links of each parity, [mu][9][Vh]
   const float2* in;       // IN_FULL: [CIN][2][3][Vh]; IN_EVEN_SCALED: even vector [3][Vh]
-  float2* out;            // OUT_FULL / OUT_GATE_*: [COUT][2][3][Vh]; OUT_EVEN_SCALED: even vector [3][Vh]
-  float2* pre;            // OUT_GATE_TRAIN: pre-activations [COUT][2][3][Vh]
+  float2* out;            // OUT_GATE_*: [COUT][2][3][Vh]; OUT_EVEN_SCALED: even vector [3][Vh]
+  float2* pre;            // pre-activations [COUT][2][3][Vh]: written by OUT_GATE_TRAIN, read by OUT_GATE_BWD
+  const float2* sub;      // OUT_EVEN_SCALED: subtracted from the result (may be null)
+  double* partials;       // OUT_GATE_BWD: [block][2 COUT] sums of dL/dgate_a, dL/dgate_b
   const float2* W;        // [9][COUT][CIN] complex (FP32 copy of BF16 values)
   const float* gate_a;    // [COUT]
   const float* gate_b;
@@ -150,6 +152,37 @@ struct ConvArgs {
   int par0;               // first output parity handled (threads cover npar parities)
   int npar;
 };
+
+// One channel of the gate h = a sigmoid(ga |a|^2 + gb) backwards at one site: from the pre-activation a and
+// g = dL/dh, dL/da in place of g, and the site's terms of dL/dga and dL/dgb.
+__device__ __forceinline__ void gate_backward(const float2 (&h)[3], float ga, float gb, float2 (&g)[3], float& da,
+                                              float& db) {
+  float n2 = 0.f, proj = 0.f;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    n2 = fmaf(h[c].x, h[c].x, fmaf(h[c].y, h[c].y, n2));
+    proj = fmaf(h[c].x, g[c].x, fmaf(h[c].y, g[c].y, proj));
+  }
+  const float sg = 1.f / (1.f + __expf(-(ga * n2 + gb)));
+  const float gp = sg * (1.f - sg);
+  const float coef = 2.f * ga * gp * proj;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) g[c] = make_float2(sg * g[c].x + coef * h[c].x, sg * g[c].y + coef * h[c].y);
+  da = gp * n2 * proj;
+  db = gp * proj;
+}
+
+// The block's sums of the gate terms in red[2 CH][SITES + 1] (128 threads): FP64, in a fixed order.
+template <int SITES>
+__device__ __forceinline__ void gate_partials(const float (&red)[2 * CH][SITES + 1], double* partials) {
+  const int v = threadIdx.x >> 3, seg = threadIdx.x & 7;
+  double t = 0.0;
+#pragma unroll
+  for (int k = 0; k < SITES / 8; ++k) t += (double)red[v][seg * (SITES / 8) + k];
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o, 8);
+  if (seg == 0) partials[(size_t)blockIdx.x * 2 * CH + v] = t;
+}
 
 // one lane per site: the layers with one input or one output channel (the 8 -> 8 layer is
 // k_conv88 below)
@@ -162,9 +195,11 @@ __global__ void __launch_bounds__(kThreads, 4) k_conv(ConvArgs a) {
   const Geom& g = a.g;
   const int Vh = g.Vh;
   const int gid = blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= a.npar * Vh) return;
-  const int par = a.par0 + gid / Vh;
-  const int i = gid % Vh;
+  const bool valid = gid < a.npar * Vh;
+  if (!valid && OUT != OUT_GATE_BWD) return;  // with sums to form, lanes past the end compute site 0 and add nothing
+  const int sv = valid ? gid : 0;
+  const int par = a.par0 + sv / Vh;
+  const int i = sv % Vh;
   const int q = 1 - par;
   const Site s = site_of(g, i, par);
   const float sc = (IN == IN_EVEN_SCALED) ? (float)*a.scale : 1.f;
@@ -251,7 +286,32 @@ __global__ void __launch_bounds__(kThreads, 4) k_conv(ConvArgs a) {
   if (OUT == OUT_EVEN_SCALED) {
     const float os = (float)*a.scale;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) a.out[(size_t)c * Vh + i] = make_float2(acc[0][c].x * os, acc[0][c].y * os);
+    for (int c = 0; c < 3; ++c) {
+      float2 z = make_float2(acc[0][c].x * os, acc[0][c].y * os);
+      if (a.sub) {
+        const float2 e = __ldg(a.sub + (size_t)c * Vh + i);
+        z.x -= e.x;
+        z.y -= e.y;
+      }
+      a.out[(size_t)c * Vh + i] = z;
+    }
+  } else if constexpr (OUT == OUT_GATE_BWD) {
+    __shared__ float red[2 * CH][kThreads + 1];
+#pragma unroll
+    for (int o = 0; o < COUT; ++o) {
+      float2 h[3];
+      float da, db;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) h[c] = __ldg(a.pre + (((size_t)o * 2 + par) * 3 + c) * Vh + i);
+      gate_backward(h, a.gate_a[o], a.gate_b[o], acc[o], da, db);
+      if (valid)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) a.out[(((size_t)o * 2 + par) * 3 + c) * Vh + i] = acc[o][c];
+      red[o][threadIdx.x] = valid ? da : 0.f;
+      red[CH + o][threadIdx.x] = valid ? db : 0.f;
+    }
+    __syncthreads();
+    gate_partials<kThreads>(red, a.partials);
   } else {
 #pragma unroll
     for (int o = 0; o < COUT; ++o) {
@@ -365,6 +425,26 @@ __global__ void __launch_bounds__(kThreads, 5) k_conv88(ConvArgs a) {
         mix1(tap, 4 * (1 - h) + k, pt);
       }
     }
+  }
+  if constexpr (OUT == OUT_GATE_BWD) {
+    __shared__ float red[2 * CH][kThreads / 2 + 1];
+#pragma unroll
+    for (int o4 = 0; o4 < 4; ++o4) {
+      const int o = 4 * h + o4;
+      float2 pa[3];
+      float da, db;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) pa[c] = __ldg(a.pre + (((size_t)o * 2 + par) * 3 + c) * Vh + i);
+      gate_backward(pa, a.gate_a[o], a.gate_b[o], acc[o4], da, db);
+      if (valid)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) a.out[(((size_t)o * 2 + par) * 3 + c) * Vh + i] = acc[o4][c];
+      red[o][threadIdx.x >> 1] = valid ? da : 0.f;
+      red[CH + o][threadIdx.x >> 1] = valid ? db : 0.f;
+    }
+    __syncthreads();
+    gate_partials<kThreads / 2>(red, a.partials);
+    return;
   }
   if (!valid) return;
 #pragma unroll
@@ -550,179 +630,196 @@ __global__ void __launch_bounds__(kThreads, 3) k_conv88_tc(ConvArgs a) {
 // ---------------------------------------------------------------------------
 // training kernels
 // ---------------------------------------------------------------------------
-// gradient through the gate: given pre-activation a and dL/dh, write dL/da and
-// accumulate dL/dgate_a, dL/dgate_b per channel (block partials [blk][2*CH])
-__global__ void __launch_bounds__(kRedThreads) k_gate_bwd(const float2* __restrict__ pre, const float2* __restrict__ gh,
-                                                          float2* __restrict__ ga, const float* gate_a,
-                                                          const float* gate_b, int Vh, double* partials) {
-  const int n = 2 * Vh;
-  const int gid = blockIdx.x * blockDim.x + threadIdx.x;
-  __shared__ double red[2 * CH][kRedThreads / 32];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int o = 0; o < CH; ++o) {
-    double da = 0.0, db = 0.0;
-    if (gid < n) {
-      const int par = gid / Vh, i = gid % Vh;
-      float2 h[3], g[3];
-      float n2 = 0.f, proj = 0.f;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const size_t k = (((size_t)o * 2 + par) * 3 + c) * Vh + i;
-        h[c] = pre[k];
-        g[c] = gh[k];
-        n2 = fmaf(h[c].x, h[c].x, fmaf(h[c].y, h[c].y, n2));
-        proj = fmaf(h[c].x, g[c].x, fmaf(h[c].y, g[c].y, proj));
-      }
-      const float sg = 1.f / (1.f + __expf(-(gate_a[o] * n2 + gate_b[o])));
-      const float gp = sg * (1.f - sg);
-      const float coef = 2.f * gate_a[o] * gp * proj;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const size_t k = (((size_t)o * 2 + par) * 3 + c) * Vh + i;
-        ga[k] = make_float2(sg * g[c].x + coef * h[c].x, sg * g[c].y + coef * h[c].y);
-      }
-      da = (double)(gp * n2 * proj);
-      db = (double)(gp * proj);
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      da += __shfl_down_sync(0xffffffffu, da, off);
-      db += __shfl_down_sync(0xffffffffu, db, off);
-    }
-    if (lane == 0) {
-      red[o][wid] = da;
-      red[CH + o][wid] = db;
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < 2 * CH) {
-    double s = 0.0;
-    for (int w = 0; w < kRedThreads / 32; ++w) s += red[threadIdx.x][w];
-    partials[(size_t)blockIdx.x * 2 * CH + threadIdx.x] = s;
-  }
+// Weight gradient dW[tap][o][ci] = sum_sites sum_c conj(t[tap][ci]) g[o] with t the tap fields of the layer's
+// input: per chunk of 32 sites the block forms the tap fields in shared memory (transporting them here, one
+// (tap, half of the channels, site) a thread, costs their gathers once; written to memory and read back they
+// are nine times the layer's input), then accumulates the outer products over the chunk's 96 (site, colour)
+// terms in registers, TT taps x TG outputs a thread, the terms shared by kWgThreads / (tiles) groups of threads.
+// A chunk's terms are summed in FP32 (at most 12 in a thread, then the groups), chunks and blocks in FP64.
+//
+// 16^4, 8 -> 8: what the earlier form spent 372 us on, one thread per entry reading both operands of every product
+// from shared memory, is bound here by the FMAs and the gathers; with the taps pass 395 -> 50 us.
+//   IN_FULL: input [CIN][2][3][Vh] on both parities; IN_EVEN_SCALED: the even vector times *in_scale
+//   gscale != null: g is an even vector [3][Vh], times *gscale (COUT = 1, even sites only)
+constexpr int kWgThreads = 288;
+constexpr int kWgSites = 32;
+constexpr int kWgTerms = 3 * kWgSites;
+constexpr int kWgStride = kWgTerms + 1;  // rows of terms start on different banks
+
+template <int CIN, int COUT, int TT, int TG>
+constexpr size_t wgrad_smem() {
+  constexpr int groups = kWgThreads / (NT * CIN / TT * (COUT / TG));
+  constexpr size_t rows = (size_t)(NT * CIN + COUT) * kWgStride * sizeof(float2);
+  constexpr size_t sums = (size_t)groups * NT * CIN * COUT * sizeof(float2);
+  return rows > sums ? rows : sums;
 }
 
-// the 9 tap fields of an input field, for every site: T[tap][ci][par][3][Vh]
-template <int CIN, int IN>
-__global__ void __launch_bounds__(kThreads, 4) k_taps(ConvArgs a, float2* __restrict__ T) {
+struct WgradArgs {
+  Geom g;
+  const float2* fat[2];
+  const float2* in;
+  const double* in_scale;
+  const float2* G;
+  const double* gscale;
+  int nsites;        // Vh (even sites) or 2 Vh
+  double* partials;  // [block][NT * COUT * CIN][2]
+};
+
+template <int CIN, int COUT, int IN, int TT, int TG>
+__global__ void __launch_bounds__(kWgThreads, 3) k_wgrad(WgradArgs a) {
+  constexpr int NE = NT * COUT * CIN;
+  constexpr int TA = NT * CIN / TT, TB = COUT / TG;  // tiles of taps and outputs
+  constexpr int GROUPS = kWgThreads / (TA * TB);
+  constexpr int TERMS = kWgTerms / GROUPS;
+  constexpr int FOLD = (2 * NE + kWgThreads - 1) / kWgThreads;
+  static_assert(TA * TT == NT * CIN && TB * TG == COUT && GROUPS * TA * TB == kWgThreads && TERMS * GROUPS == kWgTerms,
+                "tiling");
+  extern __shared__ float2 sh[];
+  float2* sT = sh;                          // [NT * CIN][kWgStride]
+  float2* sG = sh + NT * CIN * kWgStride;   // [COUT][kWgStride]
+  float* red = reinterpret_cast<float*>(sh);  // [GROUPS][2 NE], after the products
   const Geom& g = a.g;
   const int Vh = g.Vh;
-  const int gid = blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= 2 * Vh) return;
-  const int par = gid / Vh, i = gid % Vh, q = 1 - par;
-  const Site s = site_of(g, i, par);
-  const float sc = (IN == IN_EVEN_SCALED) ? (float)*a.scale : 1.f;
-  auto load_in = [&](int ci, int pp, int j, float2 (&v)[3]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const float isc = IN == IN_EVEN_SCALED ? (float)*a.in_scale : 1.f;
+  const float gsc = a.gscale ? (float)*a.gscale : 1.f;
+  const int tile = threadIdx.x % (TA * TB), grp = threadIdx.x / (TA * TB);
+  const int ta = tile % TA, tb = tile / TA;
+  double fold[FOLD];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      if (IN == IN_FULL) {
-        v[c] = __ldg(a.in + (((size_t)ci * 2 + pp) * 3 + c) * Vh + j);
-      } else {
-        const float2 t = (pp == 0) ? __ldg(a.in + (size_t)c * Vh + j) : make_float2(0.f, 0.f);
-        v[c] = make_float2(t.x * sc, t.y * sc);
-      }
-    }
-  };
-  auto store = [&](int tap, int ci, const float2 (&t)[3]) {
+  for (int k = 0; k < FOLD; ++k) fold[k] = 0.0;
+  for (int base = blockIdx.x * kWgSites; base < a.nsites; base += gridDim.x * kWgSites) {
+    const int site = base + lane;
+    const bool valid = site < a.nsites;
+    const int par = valid ? site / Vh : 0, i = valid ? site % Vh : 0, q = 1 - par;
+    const Site s = site_of(g, i, par);
+    __syncthreads();  // the sums of the chunk before have been read
+    constexpr int CPW = CIN >= 8 ? 4 : 1;  // channels a warp transports with one link
+    for (int task = warp; task < NT * CIN / CPW; task += kWgThreads / 32) {
+      const int tap = task / (CIN / CPW), c0 = (task % (CIN / CPW)) * CPW;
+      float2 t[CPW][3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) T[((((size_t)tap * CIN + ci) * 2 + par) * 3 + c) * Vh + i] = t[c];
-  };
+      for (int k = 0; k < CPW; ++k)
 #pragma unroll
-  for (int ci = 0; ci < CIN; ++ci) {
-    float2 v[3];
-    load_in(ci, par, i, v);
-    store(0, ci, v);
-  }
+        for (int c = 0; c < 3; ++c) t[k][c] = make_float2(0.f, 0.f);
+      const int ip = tap == 0 ? par : q;  // parity of the input
+      if (valid && (IN == IN_FULL || ip == 0)) {
+        const int mu = (tap - 1) >> 1, bwd = (tap - 1) & 1;
+        const int j = tap == 0 ? i : nbr(g, s, mu, bwd ? -1 : 1);
 #pragma unroll
-  for (int mu = 0; mu < 4; ++mu) {
+        for (int k = 0; k < CPW; ++k)
 #pragma unroll
-    for (int dir = 0; dir < 2; ++dir) {
-      const int j = nbr(g, s, mu, dir == 0 ? +1 : -1);
-      float2 u[9];
-      if (dir == 0) load_link9(a.fat[par] + (size_t)mu * 9 * Vh, Vh, i, u);
-      else load_link9(a.fat[q] + (size_t)mu * 9 * Vh, Vh, j, u);
+          for (int c = 0; c < 3; ++c) {
+            if (IN == IN_FULL) {
+              t[k][c] = __ldg(a.in + (((size_t)(c0 + k) * 2 + ip) * 3 + c) * Vh + j);
+            } else {
+              const float2 v = __ldg(a.in + (size_t)c * Vh + j);
+              t[k][c] = make_float2(v.x * isc, v.y * isc);
+            }
+          }
+        if (tap > 0) {
+          float2 u[9];
+          load_link9(a.fat[bwd ? q : par] + (size_t)mu * 9 * Vh, Vh, bwd ? j : i, u);
 #pragma unroll
-      for (int ci = 0; ci < CIN; ++ci) {
-        float2 v[3], t[3];
-        load_in(ci, q, j, v);
-        apply_link(u, dir == 1, v, t);
-        store(1 + 2 * mu + dir, ci, t);
-      }
-    }
-  }
-}
-
-// weight gradient partials: dW[tap][o][ci] = sum_sites sum_c conj(T[tap][ci]) g[o]
-// (block partials [blk][NT*COUT*CIN] complex, as two doubles each)
-template <int CIN, int COUT>
-__global__ void __launch_bounds__(kRedThreads) k_wgrad(const float2* __restrict__ T, const float2* __restrict__ G,
-                                                       int Vh, int even_only, double* partials) {
-  constexpr int NE = NT * COUT * CIN;
-  constexpr int CHUNK = 16;
-  __shared__ float2 sT[NT * CIN][3][CHUNK];
-  __shared__ float2 sG[COUT][3][CHUNK];
-  const int nsites = even_only ? Vh : 2 * Vh;
-  double accr[(NE + kRedThreads - 1) / kRedThreads], acci[(NE + kRedThreads - 1) / kRedThreads];
+          for (int k = 0; k < CPW; ++k) {
+            float2 o[3];
+            if (bwd) apply_link(u, true, t[k], o);
+            else apply_link(u, false, t[k], o);
 #pragma unroll
-  for (int k = 0; k < (NE + kRedThreads - 1) / kRedThreads; ++k) accr[k] = acci[k] = 0.0;
-  for (int base = blockIdx.x * CHUNK; base < nsites; base += gridDim.x * CHUNK) {
-    __syncthreads();
-    for (int j = threadIdx.x; j < NT * CIN * 3 * CHUNK; j += blockDim.x) {
-      const int sidx = j % CHUNK, c = (j / CHUNK) % 3, tc = j / (3 * CHUNK);
-      const int site = base + sidx;
-      float2 v = make_float2(0.f, 0.f);
-      if (site < nsites) {
-        const int par = site / Vh, i = site % Vh;
-        v = T[(((size_t)tc * 2 + par) * 3 + c) * Vh + i];
-      }
-      sT[tc][c][sidx] = v;
-    }
-    for (int j = threadIdx.x; j < COUT * 3 * CHUNK; j += blockDim.x) {
-      const int sidx = j % CHUNK, c = (j / CHUNK) % 3, o = j / (3 * CHUNK);
-      const int site = base + sidx;
-      float2 v = make_float2(0.f, 0.f);
-      if (site < nsites) {
-        const int par = site / Vh, i = site % Vh;
-        v = G[(((size_t)o * 2 + par) * 3 + c) * Vh + i];
-      }
-      sG[o][c][sidx] = v;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < (NE + kRedThreads - 1) / kRedThreads; ++k) {
-      const int e = threadIdx.x + k * kRedThreads;
-      if (e >= NE) continue;
-      const int ci = e % CIN, o = (e / CIN) % COUT, tap = e / (CIN * COUT);
-      float sr = 0.f, si = 0.f;
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-#pragma unroll
-        for (int j = 0; j < CHUNK; ++j) {
-          const float2 t = sT[tap * CIN + ci][c][j], gg = sG[o][c][j];
-          sr = fmaf(t.x, gg.x, fmaf(t.y, gg.y, sr));   // Re(conj(t) g)
-          si = fmaf(t.x, gg.y, fmaf(-t.y, gg.x, si));  // Im(conj(t) g)
+            for (int c = 0; c < 3; ++c) t[k][c] = o[c];
+          }
         }
-      accr[k] += sr;
-      acci[k] += si;
+      }
+#pragma unroll
+      for (int k = 0; k < CPW; ++k)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) sT[(tap * CIN + c0 + k) * kWgStride + c * kWgSites + lane] = t[k][c];
+    }
+    for (int row = warp; row < COUT * 3; row += kWgThreads / 32) {
+      const int o = row / 3, c = row % 3;
+      float2 v = make_float2(0.f, 0.f);
+      if (valid) {
+        v = __ldg(a.G + (a.gscale ? (size_t)c * Vh + i : (((size_t)o * 2 + par) * 3 + c) * Vh + i));
+        if (a.gscale) v = make_float2(gsc * v.x, gsc * v.y);
+      }
+      sG[o * kWgStride + c * kWgSites + lane] = v;
+    }
+    __syncthreads();
+    float2 acc[TT][TG];
+#pragma unroll
+    for (int x = 0; x < TT; ++x)
+#pragma unroll
+      for (int y = 0; y < TG; ++y) acc[x][y] = make_float2(0.f, 0.f);
+#pragma unroll 2
+    for (int k = grp * TERMS; k < (grp + 1) * TERMS; ++k) {
+      float2 t[TT], v[TG];
+#pragma unroll
+      for (int x = 0; x < TT; ++x) t[x] = sT[(ta + TA * x) * kWgStride + k];
+#pragma unroll
+      for (int y = 0; y < TG; ++y) v[y] = sG[(tb + TB * y) * kWgStride + k];
+#pragma unroll
+      for (int x = 0; x < TT; ++x)
+#pragma unroll
+        for (int y = 0; y < TG; ++y) {  // conj(t) g
+          acc[x][y].x = fmaf(t[x].x, v[y].x, fmaf(t[x].y, v[y].y, acc[x][y].x));
+          acc[x][y].y = fmaf(t[x].x, v[y].y, fmaf(-t[x].y, v[y].x, acc[x][y].y));
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int x = 0; x < TT; ++x)
+#pragma unroll
+      for (int y = 0; y < TG; ++y) {
+        const int tc = ta + TA * x, o = tb + TB * y;
+        const int e = ((tc / CIN) * COUT + o) * CIN + tc % CIN;
+        *reinterpret_cast<float2*>(red + grp * 2 * NE + 2 * e) = acc[x][y];
+      }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < FOLD; ++k) {
+      const int e = threadIdx.x + k * kWgThreads;
+      if (e < 2 * NE) {
+        float t = red[e];
+#pragma unroll
+        for (int w = 1; w < GROUPS; ++w) t += red[w * 2 * NE + e];
+        fold[k] += (double)t;
+      }
     }
   }
 #pragma unroll
-  for (int k = 0; k < (NE + kRedThreads - 1) / kRedThreads; ++k) {
-    const int e = threadIdx.x + k * kRedThreads;
-    if (e < NE) {
-      partials[((size_t)blockIdx.x * NE + e) * 2] = accr[k];
-      partials[((size_t)blockIdx.x * NE + e) * 2 + 1] = acci[k];
-    }
+  for (int k = 0; k < FOLD; ++k) {
+    const int e = threadIdx.x + k * kWgThreads;
+    if (e < 2 * NE) a.partials[(size_t)blockIdx.x * 2 * NE + e] = fold[k];
   }
 }
 
-// grad[off + j] += sum over blocks of partials[blk][j] (index order)
-__global__ void k_sum_partials(const double* __restrict__ partials, int nblk, int n, float* grad, int off) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
-  double s = 0.0;
-  for (int b = 0; b < nblk; ++b) s += partials[(size_t)b * n + j];
-  grad[off + j] += (float)s;
+// All sums of block partials of one pair at once: grad[off + j] += sum over rows of partials[row][j], 32 entries a
+// block, 32 row groups added in order, in FP64 (whose rate is what this takes: 64 cycles of a scheduler per
+// warp and addition). Rows of 16 entries are read two to a warp.
+struct SumSegments {
+  const double* partials[5];
+  int rows[5], n[5], off[5], blk0[5];  // blk0: first block of the segment
+  int count;
+};
+__global__ void __launch_bounds__(1024) k_sum_partials(SumSegments S, float* grad) {
+  __shared__ double part[32][33];
+  int k = 0;
+  for (int j = 1; j < S.count; ++j)
+    if ((int)blockIdx.x >= S.blk0[j]) k = j;
+  const int n = S.n[k], wide = n < 32 ? 32 : n;  // n < 32: n is 16
+  const size_t total = (size_t)S.rows[k] * n;
+  const int j = ((int)blockIdx.x - S.blk0[k]) * 32 + threadIdx.x;
+  double t = 0.0;
+  if (j < wide)
+#pragma unroll 8
+    for (size_t at = (size_t)threadIdx.y * wide + j; at < total; at += (size_t)32 * wide) t += S.partials[k][at];
+  part[threadIdx.y][threadIdx.x] = t;
+  __syncthreads();
+  if (threadIdx.y == 0) {
+    for (int y = 1; y < 32; ++y) t += part[y][threadIdx.x];
+    if (n < 32) t += __shfl_down_sync(0xffffffffu, t, 16);
+    if (j < n) grad[S.off[k] + j] += (float)t;
+  }
 }
 
 // generic FP32 two-vector dot products over even vectors [3][Vh]: sum Re<a, b>
@@ -745,24 +842,9 @@ __global__ void __launch_bounds__(kRedThreads) k_dot2(const float2* a1, const fl
   block_partial2(u, v, partials);
 }
 
-// d = z - e
-__global__ void k_sub(const float2* z, const float2* e, float2* d, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) d[i] = make_float2(z[i].x - e[i].x, z[i].y - e[i].y);
-}
-
-// g3 (even, full-lattice layout [1][2][3][Vh], odd = 0) = coef * Ad with coef = 2 / (<e,r> s)
-__global__ void k_dz(const float2* Ad, float2* g3, int Vh, const double* scal) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= 3 * Vh) return;
-  const float coef = (float)(2.0 / (scal[2] * scal[0]));
-  const int c = j / Vh, i = j % Vh;
-  g3[((size_t)0 * 3 + c) * Vh + i] = make_float2(coef * Ad[j].x, coef * Ad[j].y);
-  g3[((size_t)1 * 3 + c) * Vh + i] = make_float2(0.f, 0.f);
-}
-
 // two-sum finisher into nn scalars: mode 0: scal[0] = s = sqrt(3Vh/a), scal[1] = 1/s (input scale);
-// mode 1: scal[2] = <e,r> = b, scal[3] += <d,Ad>/<e,r> = a/b (loss)
+// mode 1: scal[2] = <e,r> = b, scal[3] += <d,Ad>/<e,r> = a/b (loss), scal[4] = 2 / (b s), which takes A d to
+// dL/d(network output before the output scale)
 __global__ void k_nn_finish(const double* partials, int n, double* scal, int mode, int Vh) {
   double a = 0.0, b = 0.0;
   for (int j = threadIdx.x; j < n; j += blockDim.x) {
@@ -778,6 +860,7 @@ __global__ void k_nn_finish(const double* partials, int n, double* scal, int mod
     } else {
       scal[2] = b;
       scal[3] += a / b;
+      scal[4] = 2.0 / (b * scal[0]);
     }
   }
 }
@@ -828,17 +911,17 @@ struct sqcg_nn {
   float* master;   // [NPARAM] FP32
   float2* wfwd;    // [NWEIGHT] BF16-rounded forward weights in FP32
   float2* wadj;    // [NWEIGHT] adjoint-layer weights
-  float* grad;     // [NPARAM]
+  float* grad;     // [NPARAM], right behind scal (one memset, one copy)
+  double* host;    // pinned copy of scal and grad
   float* adam_m;
   float* adam_v;
   int adam_t;
-  double* scal;    // [8]: s, 1/s, <e,r>, loss sum
+  double* scal;    // [8]: s, 1/s, <e,r>, loss sum, 2 / (<e,r> s)
   double* partials;
   size_t npartials;
   float2 *h1, *h2;         // inference / training activations [CH][2][3][Vh]
   float2 *a1, *a2;         // training pre-activations
-  float2 *g1, *g2, *g3;    // training gradients ([CH][2][3][Vh], g3 [1][2][3][Vh])
-  float2* T;               // training taps [9][CH][2][3][Vh]
+  float2 *g1, *g2;         // training gradients [CH][2][3][Vh]
   float2 *d, *Ad, *tmp, *zbuf;  // even FP32 vectors (training) / odd temp
   float2 *r_old, *z;       // flexible CG vectors
   // the captured flexible-CG loop, reused while b, x and the links stay the same
@@ -854,9 +937,11 @@ struct sqcg_nn {
 
 namespace {
 
+constexpr size_t kScalGradBytes = 8 * sizeof(double) + NPARAM * sizeof(float);
+
 int conv_launch(sqcg_nn* nn, int layer, bool adjoint, int in_mode, int out_mode, const float2* in, float2* out,
                 float2* pre, int par0, int npar, const SolverState* st, int gate, const double* scale,
-                cudaStream_t s) {
+                cudaStream_t s, const float2* sub = nullptr, double* partials = nullptr) {
   sqcg_ctx* ctx = nn->ctx;
   ConvArgs a;
   a.g = ctx->g;
@@ -869,8 +954,11 @@ int conv_launch(sqcg_nn* nn, int layer, bool adjoint, int in_mode, int out_mode,
   const float2* W = adjoint ? nn->wadj : nn->wfwd;
   const int offs[3] = {OFF_W1 / 2, OFF_W2 / 2, OFF_W3 / 2};
   a.W = W + offs[layer];
-  a.gate_a = nn->master + OFF_G + (layer == 0 ? 0 : 2 * CH);
+  // the gate behind the layer, or, going backwards through the layer, the one before it
+  a.gate_a = nn->master + OFF_G + (layer - (adjoint ? 1 : 0) == 0 ? 0 : 2 * CH);
   a.gate_b = a.gate_a + CH;
+  a.sub = sub;
+  a.partials = partials;
   a.scale = scale;
   a.st = st;
   a.gate = gate;
@@ -892,12 +980,12 @@ int conv_launch(sqcg_nn* nn, int layer, bool adjoint, int in_mode, int out_mode,
     k_conv88<OUT_GATE_INFER><<<grid2, kThreads, 0, s>>>(a);
   else if (cin == CH && cout == CH && in_mode == IN_FULL && out_mode == OUT_GATE_TRAIN)
     k_conv88<OUT_GATE_TRAIN><<<grid2, kThreads, 0, s>>>(a);
-  else if (cin == CH && cout == CH && in_mode == IN_FULL && out_mode == OUT_FULL)
-    k_conv88<OUT_FULL><<<grid2, kThreads, 0, s>>>(a);
+  else if (cin == CH && cout == CH && in_mode == IN_FULL && out_mode == OUT_GATE_BWD)
+    k_conv88<OUT_GATE_BWD><<<grid2, kThreads, 0, s>>>(a);
   else if (cin == CH && cout == 1 && in_mode == IN_FULL && out_mode == OUT_EVEN_SCALED)
     k_conv<CH, 1, IN_FULL, OUT_EVEN_SCALED><<<grid, kThreads, 0, s>>>(a);
-  else if (cin == 1 && cout == CH && in_mode == IN_FULL && out_mode == OUT_FULL)
-    k_conv<1, CH, IN_FULL, OUT_FULL><<<grid, kThreads, 0, s>>>(a);
+  else if (cin == 1 && cout == CH && in_mode == IN_EVEN_SCALED && out_mode == OUT_GATE_BWD)
+    k_conv<1, CH, IN_EVEN_SCALED, OUT_GATE_BWD><<<grid, kThreads, 0, s>>>(a);
   else
     return SQCG_ERR_INVALID_ARG;
   SQCG_CUDA_TRY(cudaGetLastError());
@@ -936,8 +1024,6 @@ int nn_alloc_train(sqcg_nn* nn) {
             cudaMalloc((void**)&nn->a2, full * sizeof(float2)) == cudaSuccess &&
             cudaMalloc((void**)&nn->g1, full * sizeof(float2)) == cudaSuccess &&
             cudaMalloc((void**)&nn->g2, full * sizeof(float2)) == cudaSuccess &&
-            cudaMalloc((void**)&nn->g3, 2 * 3 * Vh * sizeof(float2)) == cudaSuccess &&
-            cudaMalloc((void**)&nn->T, (size_t)NT * full * sizeof(float2)) == cudaSuccess &&
             cudaMalloc((void**)&nn->d, 3 * Vh * sizeof(float2)) == cudaSuccess &&
             cudaMalloc((void**)&nn->Ad, 3 * Vh * sizeof(float2)) == cudaSuccess &&
             cudaMalloc((void**)&nn->tmp, 3 * Vh * sizeof(float2)) == cudaSuccess &&
@@ -950,38 +1036,43 @@ int nn_alloc_train(sqcg_nn* nn) {
   return SQCG_OK;
 }
 
-// weight-gradient contribution of one layer: grad[off..] += sum_sites conj(taps(h)) g
-template <int CIN, int COUT>
-int wgrad(sqcg_nn* nn, int in_mode, const float2* h, const float2* g, int even_only, int off, cudaStream_t s) {
-  sqcg_ctx* ctx = nn->ctx;
-  const int Vh = ctx->g.Vh;
-  ConvArgs a = {};
-  a.g = ctx->g;
-  a.fat[0] = ctx->fat32;
-  a.fat[1] = ctx->fat32 + 4 * 9 * (size_t)Vh;
-  a.in = h;
-  a.scale = nn->scal;
-  if (in_mode == IN_FULL) k_taps<CIN, IN_FULL><<<nn_grid(2 * Vh), kThreads, 0, s>>>(a, nn->T);
-  else k_taps<CIN, IN_EVEN_SCALED><<<nn_grid(2 * Vh), kThreads, 0, s>>>(a, nn->T);
-  SQCG_CUDA_TRY(cudaGetLastError());
-  constexpr int NE = NT * COUT * CIN;
-  const int nsites = even_only ? Vh : 2 * Vh;
-  int nblk = (nsites + 15) / 16;
-  const int maxblk = (int)(nn->npartials / (2 * NE));
-  if (nblk > maxblk) nblk = maxblk;
-  if (nblk > 1024) nblk = 1024;
-  k_wgrad<CIN, COUT><<<nblk, kRedThreads, 0, s>>>(nn->T, g, Vh, even_only, nn->partials);
-  k_sum_partials<<<(2 * NE + 255) / 256, 256, 0, s>>>(nn->partials, nblk, 2 * NE, nn->grad, off);
-  SQCG_CUDA_TRY(cudaGetLastError());
-  return SQCG_OK;
+// Blocks of the weight-gradient kernels: three a SM (their launch bounds), no more than chunks.
+int wgrad_blocks(const sqcg_nn* nn, int nsites) {
+  const int chunks = grid_for(nsites, kWgSites), full = 3 * nn->ctx->nsm;
+  return chunks < full ? chunks : full;
 }
 
-int gate_bwd(sqcg_nn* nn, int layer, const float2* pre, const float2* gh, float2* ga, cudaStream_t s) {
-  const int Vh = nn->ctx->g.Vh, grid = (2 * Vh + kRedThreads - 1) / kRedThreads;
-  const float* gp = nn->master + OFF_G + (layer == 0 ? 0 : 2 * CH);
-  k_gate_bwd<<<grid, kRedThreads, 0, s>>>(pre, gh, ga, gp, gp + CH, Vh, nn->partials);
-  k_sum_partials<<<1, 64, 0, s>>>(nn->partials, grid, 2 * CH, nn->grad, OFF_G + (layer == 0 ? 0 : 2 * CH));
+// doubles of block partials that one pair's sums take: the three weight gradients, then the two gates
+size_t training_partials(const sqcg_nn* nn) {
+  const size_t Vh = nn->ctx->g.Vh;
+  return (size_t)3 * nn->ctx->nsm * 2 * NWEIGHT + 2 * CH * (size_t)(nn_grid(2 * (int)Vh) + nn_grid(4 * (int)Vh));
+}
+
+// one layer's weight gradient into the block partials at `at`, noted in S
+template <int CIN, int COUT, int IN, int TT, int TG>
+int wgrad(sqcg_nn* nn, const float2* h, const float2* g, const double* gscale, int nsites, int off, double*& at,
+          SumSegments& S, cudaStream_t s) {
+  sqcg_ctx* ctx = nn->ctx;
+  const size_t Vh = ctx->g.Vh;
+  WgradArgs a = {};
+  a.g = ctx->g;
+  a.fat[0] = ctx->fat32;
+  a.fat[1] = ctx->fat32 + 4 * 9 * Vh;
+  a.in = h;
+  a.in_scale = nn->scal;
+  a.G = g;
+  a.gscale = gscale;
+  a.nsites = nsites;
+  a.partials = at;
+  constexpr size_t smem = wgrad_smem<CIN, COUT, TT, TG>();
+  auto kern = k_wgrad<CIN, COUT, IN, TT, TG>;
+  SQCG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int nblk = wgrad_blocks(nn, nsites), n = 2 * NT * COUT * CIN;
+  kern<<<nblk, kWgThreads, smem, s>>>(a);
   SQCG_CUDA_TRY(cudaGetLastError());
+  const int k = S.count++;
+  S.partials[k] = at; S.rows[k] = nblk; S.n[k] = n; S.off[k] = off;
+  at += (size_t)nblk * n;
   return SQCG_OK;
 }
 
@@ -992,10 +1083,9 @@ int nn_pair(sqcg_nn* nn, double sigma, const float2* r, const float2* e, cudaStr
   SQCG_TRY(nn_input_scale(nn, r, s));
   SQCG_TRY(conv_launch(nn, 0, false, IN_EVEN_SCALED, OUT_GATE_TRAIN, r, nn->h1, nn->a1, 0, 2, nullptr, 0, nn->scal, s));
   SQCG_TRY(conv_launch(nn, 1, false, IN_FULL, OUT_GATE_TRAIN, nn->h1, nn->h2, nn->a2, 0, 2, nullptr, 0, nullptr, s));
-  SQCG_TRY(conv_launch(nn, 2, false, IN_FULL, OUT_EVEN_SCALED, nn->h2, nn->zbuf, nullptr, 0, 1, nullptr, 0,
-                       nn->scal + 1, s));
   // d = z - e; Ad = (sigma - D_eo D_oe) d in FP32; <d,Ad>, <e,r>
-  k_sub<<<nn_grid(3 * Vh), kThreads, 0, s>>>(nn->zbuf, e, nn->d, 3 * Vh);
+  SQCG_TRY(conv_launch(nn, 2, false, IN_FULL, OUT_EVEN_SCALED, nn->h2, nn->d, nullptr, 0, 1, nullptr, 0,
+                       nn->scal + 1, s, e));
   DslashLaunch L = {};
   L.out_parity = 1; L.prec = L.out_prec = SQCG_F32; L.epi = EPI_PLAIN; L.in = nn->d; L.out = nn->tmp;
   SQCG_TRY(launch_dslash(ctx, L, s));
@@ -1010,25 +1100,39 @@ int nn_pair(sqcg_nn* nn, double sigma, const float2* r, const float2* e, cudaStr
     L.out_parity = 0; L.epi = EPI_NORMAL; L.in = nn->tmp; L.out = nn->zbuf; L.y = nn->Ad; L.sigma = sigma;
     SQCG_TRY(launch_dslash(ctx, L, s));
     k_dot2<<<grid, kRedThreads, 0, s>>>(nn->Ad, nn->Ad, r, r, Vh, nn->partials);
-    k_nn_finish<<<1, kRedThreads, 0, s>>>(nn->partials, grid, nn->scal, 1, Vh);
-    k_dz<<<nn_grid(3 * Vh), kThreads, 0, s>>>(nn->zbuf, nn->g3, Vh, nn->scal);
   } else {
     // L = <d, A d> / <e, r>; dL/dz = 2 A d / <e, r>
     k_dot2<<<grid, kRedThreads, 0, s>>>(nn->d, nn->Ad, e, r, Vh, nn->partials);
-    k_nn_finish<<<1, kRedThreads, 0, s>>>(nn->partials, grid, nn->scal, 1, Vh);
-    k_dz<<<nn_grid(3 * Vh), kThreads, 0, s>>>(nn->Ad, nn->g3, Vh, nn->scal);
   }
+  k_nn_finish<<<1, kRedThreads, 0, s>>>(nn->partials, grid, nn->scal, 1, Vh);
   SQCG_CUDA_TRY(cudaGetLastError());
-  // layer 3: dW3, dL/dh2
-  SQCG_TRY((wgrad<CH, 1>(nn, IN_FULL, nn->h2, nn->g3, 1, OFF_W3, s)));
-  SQCG_TRY(conv_launch(nn, 2, true, IN_FULL, OUT_FULL, nn->g3, nn->g2, nullptr, 0, 2, nullptr, 0, nullptr, s));
-  // gate 2, layer 2
-  SQCG_TRY(gate_bwd(nn, 1, nn->a2, nn->g2, nn->g2, s));
-  SQCG_TRY((wgrad<CH, CH>(nn, IN_FULL, nn->h1, nn->g2, 0, OFF_W2, s)));
-  SQCG_TRY(conv_launch(nn, 1, true, IN_FULL, OUT_FULL, nn->g2, nn->g1, nullptr, 0, 2, nullptr, 0, nullptr, s));
-  // gate 1, layer 1
-  SQCG_TRY(gate_bwd(nn, 0, nn->a1, nn->g1, nn->g1, s));
-  SQCG_TRY((wgrad<1, CH>(nn, IN_EVEN_SCALED, r, nn->g1, 0, OFF_W1, s)));
+  const float2* Az = nn->loss_norm == 2 ? nn->zbuf : nn->Ad;  // times scal[4]: dL/d(output before its scale), even sites
+  double* at = nn->partials;
+  SumSegments S = {};
+  auto gate_sums = [&](int rows, int off) {
+    const int k = S.count++;
+    S.partials[k] = at; S.rows[k] = rows; S.n[k] = 2 * CH; S.off[k] = off;
+    at += (size_t)rows * 2 * CH;
+  };
+  // layer 3: dW3; dL/dh2 through its gate
+  SQCG_TRY((wgrad<CH, 1, IN_FULL, 4, 1>(nn, nn->h2, Az, nn->scal + 4, Vh, OFF_W3, at, S, s)));
+  SQCG_TRY(conv_launch(nn, 2, true, IN_EVEN_SCALED, OUT_GATE_BWD, Az, nn->g2, nn->a2, 0, 2, nullptr, 0, nn->scal + 4,
+                       s, nullptr, at));
+  gate_sums(nn_grid(2 * Vh), OFF_G + 2 * CH);
+  // layer 2: dW2; dL/dh1 through its gate
+  SQCG_TRY((wgrad<CH, CH, IN_FULL, 4, 4>(nn, nn->h1, nn->g2, nullptr, 2 * Vh, OFF_W2, at, S, s)));
+  SQCG_TRY(conv_launch(nn, 1, true, IN_FULL, OUT_GATE_BWD, nn->g2, nn->g1, nn->a1, 0, 2, nullptr, 0, nullptr, s,
+                       nullptr, at));
+  gate_sums(nn_grid(4 * Vh), OFF_G);
+  // layer 1: dW1
+  SQCG_TRY((wgrad<1, CH, IN_EVEN_SCALED, 3, 4>(nn, r, nn->g1, nullptr, 2 * Vh, OFF_W1, at, S, s)));
+  int blocks = 0;
+  for (int k = 0; k < S.count; ++k) {
+    S.blk0[k] = blocks;
+    blocks += grid_for(S.n[k], 32);
+  }
+  k_sum_partials<<<blocks, dim3(32, 32), 0, s>>>(S, nn->grad);
+  SQCG_CUDA_TRY(cudaGetLastError());
   return SQCG_OK;
 }
 
@@ -1046,17 +1150,16 @@ int sqcg_nn_create(sqcg_ctx* ctx, sqcg_nn** out) {
   nn->loss_norm = 1;
   const size_t Vh = ctx->g.Vh;
   const size_t full = (size_t)CH * 2 * 3 * Vh;
-  // partials: enough for the largest reduction (weight gradients: 1024 blocks x 1152 doubles)
-  nn->npartials = (size_t)1024 * 2 * NT * CH * CH;
-  const size_t red2 = 2 * ((2 * Vh + kRedThreads - 1) / kRedThreads) * 2 * CH;
-  if (red2 > nn->npartials) nn->npartials = red2;
+  nn->npartials = training_partials(nn);
+  const size_t dots = 2 * ((Vh + kRedThreads - 1) / kRedThreads);
+  if (dots > nn->npartials) nn->npartials = dots;
   bool ok = cudaMalloc((void**)&nn->master, NPARAM * sizeof(float)) == cudaSuccess &&
             cudaMalloc((void**)&nn->wfwd, NWEIGHT * sizeof(float2)) == cudaSuccess &&
             cudaMalloc((void**)&nn->wadj, NWEIGHT * sizeof(float2)) == cudaSuccess &&
-            cudaMalloc((void**)&nn->grad, NPARAM * sizeof(float)) == cudaSuccess &&
             cudaMalloc((void**)&nn->adam_m, NPARAM * sizeof(float)) == cudaSuccess &&
             cudaMalloc((void**)&nn->adam_v, NPARAM * sizeof(float)) == cudaSuccess &&
-            cudaMalloc((void**)&nn->scal, 8 * sizeof(double)) == cudaSuccess &&
+            cudaMalloc((void**)&nn->scal, kScalGradBytes) == cudaSuccess &&
+            cudaMallocHost((void**)&nn->host, kScalGradBytes) == cudaSuccess &&
             cudaMalloc((void**)&nn->partials, nn->npartials * sizeof(double)) == cudaSuccess &&
             cudaMalloc((void**)&nn->h1, full * sizeof(float2)) == cudaSuccess &&
             cudaMalloc((void**)&nn->h2, full * sizeof(float2)) == cudaSuccess &&
@@ -1067,11 +1170,12 @@ int sqcg_nn_create(sqcg_ctx* ctx, sqcg_nn** out) {
     sqcg_nn_destroy(nn);
     return SQCG_ERR_NO_MEMORY;
   }
+  nn->grad = (float*)(nn->scal + 8);
   cudaStream_t s = ctx->stream;
   SQCG_CUDA_TRY(cudaMemsetAsync(nn->master, 0, NPARAM * sizeof(float), s));
   SQCG_CUDA_TRY(cudaMemsetAsync(nn->adam_m, 0, NPARAM * sizeof(float), s));
   SQCG_CUDA_TRY(cudaMemsetAsync(nn->adam_v, 0, NPARAM * sizeof(float), s));
-  SQCG_CUDA_TRY(cudaMemsetAsync(nn->scal, 0, 8 * sizeof(double), s));
+  SQCG_CUDA_TRY(cudaMemsetAsync(nn->scal, 0, kScalGradBytes, s));
   SQCG_TRY(nn_refresh_weights(nn, s));
   *out = nn;
   return SQCG_OK;
@@ -1082,10 +1186,11 @@ int sqcg_nn_destroy(sqcg_nn* nn) {
   // the context may already be gone: wait for the device, not for the context's stream
   cudaDeviceSynchronize();
   if (nn->fcg_exec) cudaGraphExecDestroy(nn->fcg_exec);
-  void* bufs[] = {nn->master, nn->wfwd, nn->wadj, nn->grad, nn->adam_m, nn->adam_v, nn->scal, nn->partials,
-                  nn->h1, nn->h2, nn->a1, nn->a2, nn->g1, nn->g2, nn->g3, nn->T, nn->d, nn->Ad, nn->tmp,
+  void* bufs[] = {nn->master, nn->wfwd, nn->wadj, nn->adam_m, nn->adam_v, nn->scal, nn->partials,
+                  nn->h1, nn->h2, nn->a1, nn->a2, nn->g1, nn->g2, nn->d, nn->Ad, nn->tmp,
                   nn->zbuf, nn->r_old, nn->z};
   for (void* b : bufs) cudaFree(b);
+  if (nn->host) cudaFreeHost(nn->host);
   free(nn);
   return SQCG_OK;
 }
@@ -1144,14 +1249,12 @@ int sqcg_nn_loss_grad(sqcg_nn* nn, double sigma, const void* r, const void* e, d
   if (!nn || !r || !e || !(sigma >= 0)) return SQCG_ERR_INVALID_ARG;
   SQCG_TRY(nn_alloc_train(nn));
   cudaStream_t s = nn->ctx->stream;
-  SQCG_CUDA_TRY(cudaMemsetAsync(nn->grad, 0, NPARAM * sizeof(float), s));
-  SQCG_CUDA_TRY(cudaMemsetAsync(nn->scal + 3, 0, sizeof(double), s));
+  SQCG_CUDA_TRY(cudaMemsetAsync(nn->scal, 0, kScalGradBytes, s));
   SQCG_TRY(nn_pair(nn, sigma, (const float2*)r, (const float2*)e, s));
-  double sc[4];
-  SQCG_CUDA_TRY(cudaMemcpyAsync(sc, nn->scal, sizeof(sc), cudaMemcpyDeviceToHost, s));
-  if (grad) SQCG_CUDA_TRY(cudaMemcpyAsync(grad, nn->grad, NPARAM * sizeof(float), cudaMemcpyDeviceToHost, s));
+  SQCG_CUDA_TRY(cudaMemcpyAsync(nn->host, nn->scal, kScalGradBytes, cudaMemcpyDeviceToHost, s));
   SQCG_CUDA_TRY(cudaStreamSynchronize(s));
-  if (loss) *loss = sc[3];
+  if (grad) memcpy(grad, nn->host + 8, NPARAM * sizeof(float));
+  if (loss) *loss = nn->host[3];
   return SQCG_OK;
 }
 
@@ -1165,8 +1268,7 @@ int sqcg_nn_train(sqcg_nn* nn, double sigma, int npairs, const void* r, const vo
   unsigned long long state = seed ? seed : 0x9e3779b97f4a7c15ULL;
   double first = 0.0, last = 0.0;
   for (int step = 0; step < steps; ++step) {
-    SQCG_CUDA_TRY(cudaMemsetAsync(nn->grad, 0, NPARAM * sizeof(float), s));
-    SQCG_CUDA_TRY(cudaMemsetAsync(nn->scal + 3, 0, sizeof(double), s));
+    SQCG_CUDA_TRY(cudaMemsetAsync(nn->scal, 0, kScalGradBytes, s));
     for (int b = 0; b < batch; ++b) {
       state = state * 6364136223846793005ULL + 1442695040888963407ULL;  // LCG (Knuth MMIX constants)
       const int k = (int)((state >> 33) % (unsigned long long)npairs);

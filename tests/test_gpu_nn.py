@@ -360,3 +360,27 @@ def test_network_closes_with_its_lattice(sqcg, links_cache):
     assert net._h is None
     with pytest.raises(sqcg.SqcgError):
         net.set_params(params_to_flat(onn.init_params(8, scale=0.3)))
+
+
+@pytest.mark.parametrize("norm", [1, 2])
+@pytest.mark.parametrize("L", [(6, 6, 6, 6), (4, 6, 10, 6), (14, 14, 14, 14)])
+def test_gradient_at_remainders_of_its_chunks(sqcg, links_cache, L, norm):
+    """Loss and gradient where the sites end inside a chunk of 32 (648 and 720 sites a parity; 19208, with more
+    chunks than resident blocks) and inside the blocks that sum the gates' terms, against the oracle at 1e-4."""
+    fat, lng = links_cache(L, 62)
+    r, e = to_f32(synth.gaussian_source(L, 63)), to_f32(0.3 * synth.gaussian_source(L, 64))
+    sigma = 0.04
+    with sqcg.Lattice(L) as lat:
+        lat.load_links(fat, lng)
+        net = sqcg.Network(lat)
+        net.set_params(params_to_flat(onn.init_params(9)))
+        net.set_loss(norm)
+        dr, de = lat.pack(r, sqcg.F32), lat.pack(e, sqcg.F32)
+        loss, grad = net.loss_grad(sigma, dr, de)
+        again = net.loss_grad(sigma, dr, de)
+        params = flat_to_params(net.get_params(bf16_rounded=True))
+        net.close()
+    want_l, want_g = onn.loss_and_grad(L, fat, lng, params, r, e, sigma, norm=norm)
+    assert abs(loss - want_l) <= 1e-4 * abs(want_l)
+    assert rel(grad, params_to_flat(want_g)) <= 1e-4
+    assert again[0] == loss and np.array_equal(again[1], grad)
