@@ -6,8 +6,8 @@
 // warp loads instead.
 #include <cmath>
 #include <complex>
-#include <vector>
 
+#include "ff_arith.cuh"
 #include "sqcg_internal.cuh"
 
 namespace {
@@ -23,38 +23,98 @@ __device__ __forceinline__ void coords_of(const Geom& g, long n, int& x, int& y,
   t = (int)(n / g.Lz);
 }
 
-// one thread per (mu, site): raw[n][mu][9] -> out64[par][mu][e][n/2] (e < 9) and
-// out32[par][mu][e][n/2] (e < nelem32: 9, or 6 for the 12-real form)
-__global__ void k_pack_links(const double2* __restrict__ raw, Geom g, int fold, int hop, int nelem32,
-                             double2* __restrict__ out64, float2* __restrict__ out32) {
-  const long V = 2L * g.Vh;
-  const long tid = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= 4 * V) return;
-  const int mu = (int)(tid / V);
-  const long n = tid % V;
+// raw[n][mu][9] (host link order) -> out64[par][mu][e][n/2] (e < 9), out32[par][mu][e][n/2] (e < nelem32: 9, or 6
+// for the 12-real form) and the float-float copy outff, phases folded. A block takes 32 consecutive sites: their
+// 18 KB are contiguous in raw, go through shared memory, and leave as runs of 16 sites per parity, direction
+// and element. Bound by the FP64 pipe, which the conversions to FP32 run on (16^4: 29 us a field; the first form,
+// with a thread reading its link's 144 bytes at a stride of 144 and a second pass for outff, took 61).
+constexpr int kPackSites = 32, kPackThreads = 128;
+__global__ void __launch_bounds__(kPackThreads) k_pack_links(const double2* __restrict__ raw, Geom g, int fold, int hop,
+                                                             int nelem32, double2* __restrict__ out64,
+                                                             float2* __restrict__ out32, float4* __restrict__ outff) {
+  __shared__ double2 sm[kPackSites][37];  // 36 elements a site, padded against bank conflicts
+  const long V = 2L * g.Vh, n0 = (long)blockIdx.x * kPackSites;
+  const int ns = V - n0 < kPackSites ? (int)(V - n0) : kPackSites;
+  for (int j = threadIdx.x; j < ns * 36; j += kPackThreads) sm[j / 36][j % 36] = raw[n0 * 36 + j];
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int p = lane >> 4;  // parity; the half index of the site is ih
+  const long ih = (n0 >> 1) + (lane & 15);
+  if (2 * (lane & 15) >= ns) return;
   int x, y, z, t;
-  coords_of(g, n, x, y, z, t);
-  const int par = (x + y + z + t) & 1;
-  const long ih = n >> 1;
+  coords_of(g, 2 * ih, x, y, z, t);
+  const int odd = (y + z + t + p) & 1;  // 2 ih has x even
+  x += odd;
+  const int local = 2 * (lane & 15) + odd;
+  for (int k = warp; k < 36; k += kPackThreads / 32) {
+    const int mu = k / 9, e = k % 9;
+    bool neg = false;
+    if (fold) {
+      const int c = (mu == 0) ? 0 : (mu == 1) ? x : (mu == 2) ? x + y : x + y + z;
+      neg = c & 1;
+      if (mu == 3 && g.apbc && t + hop >= g.Lt) neg = !neg;
+    }
+    double2 v = sm[local][k];
+    if (neg) v = make_double2(-v.x, -v.y);
+    const size_t at64 = (((size_t)p * 4 + mu) * 9 + e) * g.Vh + ih;
+    const float4 f = split_ff(v);
+    out64[at64] = v;
+    outff[at64] = f;
+    if (e < nelem32) out32[(((size_t)p * 4 + mu) * nelem32 + e) * g.Vh + ih] = make_float2(f.x, f.z);
+  }
+}
+
+// Is every long link s W with W in SU(3) and s the one real scale s0, to 1e-12? With the phases folded by the
+// caller, s carries eta_mu(n) and the boundary sign, which are divided out before it is compared. *bad is set
+// where not. One thread a link, the block's links staged through shared memory.
+constexpr int kCheckThreads = 128;
+__global__ void __launch_bounds__(kCheckThreads) k_recon_check(const double2* __restrict__ raw, Geom g, int folded,
+                                                               double s0, int* __restrict__ bad) {
+  __shared__ double2 sm[kCheckThreads * 9];
+  const long nlinks = 8L * g.Vh, l0 = (long)blockIdx.x * kCheckThreads;
+  const int nl = nlinks - l0 < kCheckThreads ? (int)(nlinks - l0) : kCheckThreads;
+  for (int j = threadIdx.x; j < nl * 9; j += kCheckThreads) sm[j] = raw[l0 * 9 + j];
+  __syncthreads();
+  if ((int)threadIdx.x >= nl) return;
+  double2 U[9];
+#pragma unroll
+  for (int e = 0; e < 9; ++e) U[e] = sm[threadIdx.x * 9 + e];
+  auto mul = [](double2 a, double2 b) { return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); };
+  double2 det = make_double2(0.0, 0.0);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const double2 m1 = mul(U[3 + (j + 1) % 3], U[6 + (j + 2) % 3]), m2 = mul(U[3 + (j + 2) % 3], U[6 + (j + 1) % 3]);
+    const double2 d = mul(U[j], make_double2(m1.x - m2.x, m1.y - m2.y));
+    det.x += d.x;
+    det.y += d.y;
+  }
+  const double s = cbrt(det.x), s2 = s * s;
+  bool ok = fabs(s) > 0.0 && isfinite(s) && fabs(det.y) <= 1e-12 * fabs(s2 * s);
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = a; b < 3; ++b) {
+      double re = (a == b) ? -s2 : 0.0, im = 0.0;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const double2 u = U[a * 3 + c], v = U[b * 3 + c];
+        re += u.x * v.x + u.y * v.y;
+        im += u.y * v.x - u.x * v.y;
+      }
+      ok = ok && re * re + im * im <= 1e-24 * s2 * s2;  // false for a NaN
+    }
   double f = 1.0;
-  if (fold) {
-    int e = 0;
-    if (mu == 1) e = x;
-    if (mu == 2) e = x + y;
-    if (mu == 3) e = x + y + z;
+  if (folded) {
+    const long l = l0 + threadIdx.x;
+    const int mu = (int)(l & 3);
+    int x, y, z, t;
+    coords_of(g, l >> 2, x, y, z, t);
+    const int e = (mu == 0) ? 0 : (mu == 1) ? x : (mu == 2) ? x + y : x + y + z;
     if (e & 1) f = -f;
-    if (mu == 3 && g.apbc && t + hop >= g.Lt) f = -f;
+    if (mu == 3 && g.apbc && t + 3 >= g.Lt) f = -f;
   }
-  const double2* src = raw + (n * 4 + mu) * 9;
-  const size_t base64 = ((size_t)par * 4 + mu) * 9 * g.Vh;
-  const size_t base32 = ((size_t)par * 4 + mu) * nelem32 * g.Vh;
-  for (int e = 0; e < 9; ++e) {
-    const double2 u = src[e];
-    const double2 v = make_double2(f * u.x, f * u.y);
-    out64[base64 + (size_t)e * g.Vh + ih] = v;
-    if (e < nelem32)
-      out32[base32 + (size_t)e * g.Vh + ih] = make_float2(__double2float_rn(v.x), __double2float_rn(v.y));
-  }
+  ok = ok && fabs(s * f - s0) <= 1e-12 * fabs(s0);
+  if (!ok) *bad = 1;
 }
 
 // host parity order [Vh][3] complex double -> device [3][Vh] (FP64 or FP32)
@@ -77,12 +137,7 @@ __global__ void k_aos_to_soa_ff(const double2* __restrict__ aos, float4* __restr
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= Vh) return;
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const double2 v = aos[(size_t)i * 3 + c];
-    const float rh = __double2float_rn(v.x), ih = __double2float_rn(v.y);
-    soa[(size_t)c * Vh + i] =
-        make_float4(rh, __double2float_rn(v.x - (double)rh), ih, __double2float_rn(v.y - (double)ih));
-  }
+  for (int c = 0; c < 3; ++c) soa[(size_t)c * Vh + i] = split_ff(aos[(size_t)i * 3 + c]);
 }
 
 __global__ void k_soa_ff_to_aos(const float4* __restrict__ soa, double2* __restrict__ aos, int Vh) {
@@ -148,57 +203,45 @@ __global__ void k_pack_backward(const double2* __restrict__ fwd64, Geom g, int d
     }
 }
 
-typedef std::complex<double> cd;
+// The scale of the first long link (site 0, direction x: its phase and boundary sign are 1): cbrt(Re det).
+double first_link_scale(const double* p) {
+  typedef std::complex<double> cd;
+  cd U[3][3];
+  for (int a = 0; a < 3; ++a)
+    for (int b = 0; b < 3; ++b) U[a][b] = cd(p[(a * 3 + b) * 2], p[(a * 3 + b) * 2 + 1]);
+  const cd det = U[0][0] * (U[1][1] * U[2][2] - U[1][2] * U[2][1]) -
+                 U[0][1] * (U[1][0] * U[2][2] - U[1][2] * U[2][0]) +
+                 U[0][2] * (U[1][0] * U[2][1] - U[1][1] * U[2][0]);
+  return std::cbrt(det.real());
+}
 
-// 12-real eligibility: every long link is s * W, W in SU(3), |s| global.
-// With the phases folded by the caller, s carries eta_mu(n) and the boundary
-// sign; they are divided out before the scale is compared.
-bool recon_check(const sqcg_ctx* ctx, const double* lng, double* s0_out) {
-  const int* L = ctx->L;
-  const long V = (long)L[0] * L[1] * L[2] * L[3];
-  const bool folded = (ctx->flags & SQCG_PHASES_FOLDED) != 0;
-  double s0 = 0.0;
-  for (long n = 0; n < V; ++n) {
-    long m = n;
-    const int x = (int)(m % L[0]); m /= L[0];
-    const int y = (int)(m % L[1]); m /= L[1];
-    const int z = (int)(m % L[2]);
-    const int t = (int)(m / L[2]);
-    for (int mu = 0; mu < 4; ++mu) {
-      const double* p = lng + ((size_t)n * 4 + mu) * 18;
-      cd U[3][3];
-      for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) U[a][b] = cd(p[(a * 3 + b) * 2], p[(a * 3 + b) * 2 + 1]);
-      const cd det = U[0][0] * (U[1][1] * U[2][2] - U[1][2] * U[2][1]) -
-                     U[0][1] * (U[1][0] * U[2][2] - U[1][2] * U[2][0]) +
-                     U[0][2] * (U[1][0] * U[2][1] - U[1][1] * U[2][0]);
-      const double s = std::cbrt(det.real());
-      if (!(std::fabs(s) > 0.0) || !std::isfinite(s)) return false;
-      const double s3 = std::fabs(s * s * s);
-      if (std::abs(det.imag()) > 1e-12 * s3) return false;
-      for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) {
-          cd uu = 0;
-          for (int c = 0; c < 3; ++c) uu += U[a][c] * std::conj(U[b][c]);
-          if (a == b) uu -= s * s;
-          if (std::abs(uu) > 1e-12 * s * s) return false;
-        }
-      double f = 1.0;
-      if (folded) {
-        int e = 0;
-        if (mu == 1) e = x;
-        if (mu == 2) e = x + y;
-        if (mu == 3) e = x + y + z;
-        if (e & 1) f = -f;
-        if (mu == 3 && (ctx->flags & SQCG_ANTIPERIODIC_T) && t + 3 >= L[3]) f = -f;
-      }
-      const double s_unfolded = s * f;
-      if (n == 0 && mu == 0) s0 = s_unfolded;
-      else if (std::fabs(s_unfolded - s0) > 1e-12 * std::fabs(s0)) return false;
-    }
+// 12-real eligibility of long links in device memory (host link order); first: its first link in host memory
+int recon_check(sqcg_ctx* ctx, const double2* lng, const double* first, double* s0_out) {
+  const double s0 = first_link_scale(first);
+  if (!(std::fabs(s0) > 0.0) || !std::isfinite(s0)) return SQCG_ERR_RECON_REJECTED;
+  int* bad = nullptr;
+  if (cudaMalloc((void**)&bad, sizeof(int)) != cudaSuccess) {
+    cudaGetLastError();
+    return SQCG_ERR_NO_MEMORY;
+  }
+  cudaStream_t s = ctx->stream;
+  int h = 0;
+  const long nlinks = 8L * ctx->g.Vh;
+  cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int), s);
+  if (e == cudaSuccess) {
+    k_recon_check<<<(unsigned)((nlinks + kCheckThreads - 1) / kCheckThreads), kCheckThreads, 0, s>>>(
+        lng, ctx->g, (ctx->flags & SQCG_PHASES_FOLDED) ? 1 : 0, s0, bad);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, bad, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  cudaFree(bad);
+  if (e != cudaSuccess) {
+    sqcg_set_last_cuda_error(e, "long-link check", __FILE__, __LINE__);
+    return SQCG_ERR_CUDA;
   }
   *s0_out = s0;
-  return true;
+  return h ? SQCG_ERR_RECON_REJECTED : SQCG_OK;
 }
 
 int ensure_stage(sqcg_ctx* ctx, size_t bytes) {
@@ -218,32 +261,10 @@ int ensure_stage(sqcg_ctx* ctx, size_t bytes) {
 
 namespace {
 
-// fat, lng: host order [V][4][3][3] complex, in host memory or (on_device) in device memory
-int load_links(sqcg_ctx* ctx, const double* fat, const double* lng, int opts, bool on_device) {
-  if (!fat || !lng) return SQCG_ERR_INVALID_ARG;
-  if (opts & ~(SQCG_RECON12_LONG | SQCG_EIGHT_WAY)) return SQCG_ERR_INVALID_ARG;
-  const bool recon = (opts & SQCG_RECON12_LONG) != 0;
-  const bool eightway = (opts & SQCG_EIGHT_WAY) != 0;
-  double s0 = 1.0;
-  if (recon) {
-    if (on_device) {  // the eligibility test runs on the host
-      std::vector<double> h((size_t)2 * ctx->g.Vh * 4 * 18);
-      SQCG_CUDA_TRY(cudaMemcpy(h.data(), lng, h.size() * sizeof(double), cudaMemcpyDeviceToHost));
-      if (!recon_check(ctx, h.data(), &s0)) return SQCG_ERR_RECON_REJECTED;
-    } else if (!recon_check(ctx, lng, &s0)) {
-      return SQCG_ERR_RECON_REJECTED;
-    }
-  }
+// staging of host links up to this size stays with the context, larger staging lives for the call
+constexpr size_t kKeptStage = (size_t)64 << 20;
 
-  const size_t Vh = ctx->g.Vh, V = 2 * Vh;
-  // the 12-real form is used for the FP32 copy only: on this GPU the FP64 Dslash is
-  // bound by FP64 arithmetic, which rebuilding the third row would only add to
-  const int nl32 = recon ? 6 : 9;
-  const size_t nfat = 2 * 4 * 9 * Vh, nlng64 = 2 * 4 * 9 * Vh, nlng32 = 2 * 4 * (size_t)nl32 * Vh;
-  cudaStream_t s = ctx->stream;
-
-  // drop earlier links
-  SQCG_CUDA_TRY(cudaStreamSynchronize(s));
+void free_links(sqcg_ctx* ctx) {
   cudaFree(ctx->fat64); cudaFree(ctx->lng64); cudaFree(ctx->fat32); cudaFree(ctx->lng32);
   cudaFree(ctx->fatb32); cudaFree(ctx->lngb32);
   cudaFree(ctx->fatff); cudaFree(ctx->lngff);
@@ -251,71 +272,113 @@ int load_links(sqcg_ctx* ctx, const double* fat, const double* lng, int opts, bo
   ctx->fat32 = ctx->lng32 = nullptr;
   ctx->fatb32 = ctx->lngb32 = nullptr;
   ctx->fatff = ctx->lngff = nullptr;
+}
+
+// Device link arrays for 12-real or full long links, with the backward arrays of the 8-way form or without; those
+// of the links before are kept where they are the same (an allocation of this size takes 0.1 ms and more).
+int ensure_links(sqcg_ctx* ctx, int nl32, bool eightway) {
+  const size_t Vh = ctx->g.Vh, n9 = 2 * 4 * 9 * Vh, nl = 2 * 4 * (size_t)nl32 * Vh;
+  if (ctx->fat64 && ctx->link_nl32 != nl32) free_links(ctx);
+  if (!eightway) {
+    cudaFree(ctx->fatb32); cudaFree(ctx->lngb32);
+    ctx->fatb32 = ctx->lngb32 = nullptr;
+  }
+  auto want = [](auto** p, size_t bytes) { return *p || cudaMalloc((void**)p, bytes) == cudaSuccess; };
+  const bool ok = want(&ctx->fat64, n9 * sizeof(double2)) && want(&ctx->lng64, n9 * sizeof(double2)) &&
+                  want(&ctx->fat32, n9 * sizeof(float2)) && want(&ctx->lng32, nl * sizeof(float2)) &&
+                  want(&ctx->fatff, n9 * sizeof(float4)) && want(&ctx->lngff, n9 * sizeof(float4)) &&
+                  (!eightway || (want(&ctx->fatb32, n9 * sizeof(float2)) && want(&ctx->lngb32, nl * sizeof(float2))));
+  if (!ok) {
+    cudaGetLastError();
+    free_links(ctx);
+    return SQCG_ERR_NO_MEMORY;
+  }
+  ctx->link_nl32 = nl32;
+  return SQCG_OK;
+}
+
+// fat, lng: host order [V][4][3][3] complex, in host memory or (on_device) in device memory
+int load_links(sqcg_ctx* ctx, const double* fat, const double* lng, int opts, bool on_device) {
+  if (!fat || !lng) return SQCG_ERR_INVALID_ARG;
+  if (opts & ~(SQCG_RECON12_LONG | SQCG_EIGHT_WAY)) return SQCG_ERR_INVALID_ARG;
+  const bool recon = (opts & SQCG_RECON12_LONG) != 0;
+  const bool eightway = (opts & SQCG_EIGHT_WAY) != 0;
+  cudaStream_t s = ctx->stream;
+  const size_t V = 2 * (size_t)ctx->g.Vh, bytes = V * 4 * 9 * sizeof(double2);
+
+  // host links are staged one field at a time, the long ones first: a rejection of the 12-real form leaves
+  // the earlier links as they are
+  void* own = nullptr;
+  void* raw = nullptr;
+  if (!on_device) {
+    if (bytes <= kKeptStage) {
+      SQCG_TRY(ensure_stage(ctx, bytes));
+      raw = ctx->stage;
+    } else if (cudaMalloc(&own, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      return SQCG_ERR_NO_MEMORY;
+    } else {
+      raw = own;
+    }
+  }
+  double s0 = 1.0;
+  int rc = SQCG_OK;
+  const double2* src = (const double2*)lng;
+  if (!on_device) {
+    if (cudaMemcpyAsync(raw, lng, bytes, cudaMemcpyHostToDevice, s) != cudaSuccess) rc = SQCG_ERR_CUDA;
+    src = (const double2*)raw;
+  }
+  if (rc == SQCG_OK && recon) {
+    double first[18];
+    const double* f = lng;
+    if (on_device) {
+      if (cudaMemcpyAsync(first, lng, sizeof(first), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+          cudaStreamSynchronize(s) != cudaSuccess)
+        rc = SQCG_ERR_CUDA;
+      f = first;
+    }
+    if (rc == SQCG_OK) rc = recon_check(ctx, src, f, &s0);
+  }
+  if (rc != SQCG_OK) {
+    if (rc == SQCG_ERR_CUDA) sqcg_set_last_cuda_error(cudaGetLastError(), "load_links", __FILE__, __LINE__);
+    cudaFree(own);
+    return rc;
+  }
+
+  // the 12-real form is used for the FP32 copy only: on this GPU the FP64 Dslash is
+  // bound by FP64 arithmetic, which rebuilding the third row would only add to
+  const int nl32 = recon ? 6 : 9;
+  // drop earlier links
+  if (cudaStreamSynchronize(s) != cudaSuccess) rc = SQCG_ERR_CUDA;
   ctx->eightway = false;
   ctx->have_links = false;
   free_graphs(ctx);
   free_batch_plan(ctx);
-
-  void* raw = nullptr;
-  bool ok = cudaMalloc((void**)&ctx->fat64, nfat * sizeof(double2)) == cudaSuccess &&
-            cudaMalloc((void**)&ctx->lng64, nlng64 * sizeof(double2)) == cudaSuccess &&
-            cudaMalloc((void**)&ctx->fat32, nfat * sizeof(float2)) == cudaSuccess &&
-            cudaMalloc((void**)&ctx->lng32, nlng32 * sizeof(float2)) == cudaSuccess &&
-            cudaMalloc((void**)&ctx->fatff, nfat * sizeof(float4)) == cudaSuccess &&
-            cudaMalloc((void**)&ctx->lngff, nlng64 * sizeof(float4)) == cudaSuccess &&
-            (on_device || cudaMalloc(&raw, V * 4 * 9 * sizeof(double2)) == cudaSuccess);
-  if (!ok) {
-    cudaGetLastError();
-    cudaFree(raw);
-    cudaFree(ctx->fat64); cudaFree(ctx->lng64); cudaFree(ctx->fat32); cudaFree(ctx->lng32);
-    cudaFree(ctx->fatff); cudaFree(ctx->lngff);
-    ctx->fat64 = ctx->lng64 = nullptr;
-    ctx->fat32 = ctx->lng32 = nullptr;
-    ctx->fatff = ctx->lngff = nullptr;
-    return SQCG_ERR_NO_MEMORY;
-  }
+  if (rc == SQCG_OK) rc = ensure_links(ctx, nl32, eightway);
   const int fold = (ctx->flags & SQCG_PHASES_FOLDED) ? 0 : 1;
-  const long nthreads = 4 * (long)V;
-  const int grid = (int)((nthreads + kThreads - 1) / kThreads);
-  int rc = SQCG_OK;
-  do {
-    const double2* src = (const double2*)fat;
-    if (!on_device) {
-      if (cudaMemcpyAsync(raw, fat, V * 4 * 9 * sizeof(double2), cudaMemcpyHostToDevice, s) != cudaSuccess) { rc = SQCG_ERR_CUDA; break; }
-      src = (const double2*)raw;
-    }
-    k_pack_links<<<grid, kThreads, 0, s>>>(src, ctx->g, fold, 1, 9, ctx->fat64, ctx->fat32);
-    if (cudaGetLastError() != cudaSuccess) { rc = SQCG_ERR_CUDA; break; }
-    src = (const double2*)lng;
-    if (!on_device) {
-      // the fat pass must finish reading the staging buffer before it is overwritten (same stream)
-      if (cudaMemcpyAsync(raw, lng, V * 4 * 9 * sizeof(double2), cudaMemcpyHostToDevice, s) != cudaSuccess) { rc = SQCG_ERR_CUDA; break; }
-      src = (const double2*)raw;
-    }
-    k_pack_links<<<grid, kThreads, 0, s>>>(src, ctx->g, fold, 3, nl32, ctx->lng64, ctx->lng32);
-    if (cudaGetLastError() != cudaSuccess) { rc = SQCG_ERR_CUDA; break; }
-    // the float-float copy of the folded FP64 links (reliable-update arithmetic)
-    if (launch_split_ff(ctx->fat64, ctx->fatff, nfat, s) != SQCG_OK) { rc = SQCG_ERR_CUDA; break; }
-    if (launch_split_ff(ctx->lng64, ctx->lngff, nlng64, s) != SQCG_OK) { rc = SQCG_ERR_CUDA; break; }
-    if (cudaStreamSynchronize(s) != cudaSuccess) { rc = SQCG_ERR_CUDA; break; }
-  } while (0);
-  cudaFree(raw);
-  if (rc == SQCG_OK && eightway) {
-    if (cudaMalloc((void**)&ctx->fatb32, nfat * sizeof(float2)) != cudaSuccess ||
-        cudaMalloc((void**)&ctx->lngb32, nlng32 * sizeof(float2)) != cudaSuccess) {
-      cudaGetLastError();
-      cudaFree(ctx->fatb32); cudaFree(ctx->lngb32);
-      ctx->fatb32 = ctx->lngb32 = nullptr;
-      return SQCG_ERR_NO_MEMORY;
-    }
-    k_pack_backward<<<grid, kThreads, 0, s>>>(ctx->fat64, ctx->g, 1, 9, ctx->fatb32);
-    k_pack_backward<<<grid, kThreads, 0, s>>>(ctx->lng64, ctx->g, 3, nl32, ctx->lngb32);
-    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) rc = SQCG_ERR_CUDA;
+  const unsigned grid = (unsigned)((V + kPackSites - 1) / kPackSites);
+  if (rc == SQCG_OK) {
+    k_pack_links<<<grid, kPackThreads, 0, s>>>(src, ctx->g, fold, 3, nl32, ctx->lng64, ctx->lng32, ctx->lngff);
+    src = (const double2*)fat;
+    // the long pass must finish reading the staging buffer before it is overwritten (same stream)
+    if (cudaGetLastError() != cudaSuccess ||
+        (!on_device && cudaMemcpyAsync(raw, fat, bytes, cudaMemcpyHostToDevice, s) != cudaSuccess))
+      rc = SQCG_ERR_CUDA;
+    if (!on_device) src = (const double2*)raw;
   }
-  if (rc != SQCG_OK) {
-    sqcg_set_last_cuda_error(cudaGetLastError(), "load_links", __FILE__, __LINE__);
-    return rc;
+  if (rc == SQCG_OK) {
+    k_pack_links<<<grid, kPackThreads, 0, s>>>(src, ctx->g, fold, 1, 9, ctx->fat64, ctx->fat32, ctx->fatff);
+    if (eightway) {
+      const unsigned gb = (unsigned)((4 * V + kThreads - 1) / kThreads);
+      k_pack_backward<<<gb, kThreads, 0, s>>>(ctx->fat64, ctx->g, 1, 9, ctx->fatb32);
+      k_pack_backward<<<gb, kThreads, 0, s>>>(ctx->lng64, ctx->g, 3, nl32, ctx->lngb32);
+    }
+    if (cudaGetLastError() != cudaSuccess) rc = SQCG_ERR_CUDA;
   }
+  if (cudaStreamSynchronize(s) != cudaSuccess) rc = SQCG_ERR_CUDA;
+  if (rc == SQCG_ERR_CUDA) sqcg_set_last_cuda_error(cudaGetLastError(), "load_links", __FILE__, __LINE__);
+  cudaFree(own);
+  if (rc != SQCG_OK) return rc;
   ctx->eightway = eightway;
   ctx->recon = recon;
   ctx->long_scale = s0;

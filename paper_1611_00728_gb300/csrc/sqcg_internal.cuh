@@ -181,7 +181,9 @@ struct sqcg_ctx {
   float2* fatb32;
   float2* lngb32;
 
-  // host-copy staging for pack/unpack
+  int link_nl32;  // elements of an FP32 long link in the arrays above (9 or 6)
+
+  // host-copy staging for pack/unpack and for the links of smaller lattices
   void* stage;
   size_t stage_bytes;
 

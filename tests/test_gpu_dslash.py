@@ -245,3 +245,57 @@ def test_split_dslash_remainders(sqcg, links_cache, L, recon, eight):
             if prec != 2:
                 lat.normal_op(0.04, d_in, out, prec)
                 assert rel(lat.unpack(out, prec), want_a) <= bar, prec
+
+
+@pytest.mark.parametrize("where", [(0, 0), (1, 2), (-1, 3)])
+@pytest.mark.parametrize("folded", [False, True])
+def test_recon12_check_finds_one_link(sqcg, links_cache, where, folded):
+    """The 12-real eligibility test sees a change of 1e-10 (its line is 1e-12) in any one long link: of its scale,
+    of its determinant's phase, of one element. A refusal leaves the links before it in use; a change of 1e-14
+    passes. 648 sites a parity: the last block of the check is partly filled."""
+    L = (6, 6, 6, 6)
+    fat, lng = links_cache(L, 1005)
+    psi = synth.gaussian_source(L, 2005)
+    want = oracle.dslash(L, fat, lng, psi, 0)
+    if folded:
+        fat, lng = fold_phases(L, fat, 1, True), fold_phases(L, lng, 3, True)
+
+    def changed(kind, eps):
+        out = lng.copy()
+        u = out[where[0], where[1]]
+        if kind == "scale":
+            u *= 1 + eps
+        elif kind == "phase":
+            u *= np.exp(1j * eps)
+        else:
+            u[1, 2] += eps * np.abs(u).max()
+        return out
+
+    with sqcg.Lattice(L, phases_folded=folded) as lat:
+        lat.load_links(fat, lng, recon12=True)
+        out = lat.new_spinor(1)
+        for kind in ("scale", "phase", "element"):
+            with pytest.raises(sqcg.SqcgError) as err:
+                lat.load_links(fat, changed(kind, 1e-10), recon12=True)
+            assert err.value.name == "RECON_REJECTED"
+            lat.dslash(0, lat.pack(psi, 1), out, 1)
+            assert rel(lat.unpack(out, 1), want) <= TOL[1]
+            lat.load_links(fat, changed(kind, 1e-14), recon12=True)
+
+
+def test_links_reloaded_in_other_forms(sqcg, links_cache):
+    """Links loaded again and again into one context, with other values and in every storage form (arrays of the same
+    size are used again), on a lattice whose last 32-site block is half filled."""
+    L = (6, 6, 6, 6)
+    psi = synth.gaussian_source(L, 2006)
+    with sqcg.Lattice(L) as lat:
+        for k, (recon, eight) in enumerate([(False, False), (True, False), (True, True), (False, True), (True, False),
+                                            (True, False), (False, False)]):
+            fat, lng = links_cache(L, 1005 + k % 2)
+            lat.load_links(fat, lng, recon12=recon, eight_way=eight)
+            for prec, bar in ((0, 1e-12), (1, 1e-5), (2, 1e-12)):
+                out = lat.new_spinor(prec)
+                for par in (0, 1):
+                    lat.dslash(par, lat.pack(psi, prec), out, prec)
+                    want = oracle.dslash(L, fat, lng, psi, par)
+                    assert rel(lat.unpack(out, prec), want) <= bar, (k, prec, par)
