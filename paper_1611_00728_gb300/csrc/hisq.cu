@@ -12,13 +12,14 @@
 //
 // One smearing level is three kernels over full-lattice structure-of-arrays
 // fields [field][element][V] (site fastest, coalesced):
-//   A: S^s_{mu nu}(n), the single-sign 3-staples (24 fields), and their sums
-//      S3_{mu nu} = S^+ + S^- (12 fields);
+//   A: S^s_{mu nu}(n), the single-sign 3-staples (24 fields; only where the level
+//      has a Lepage term), and their sums S3_{mu nu} = S^+ + S^- (12 fields);
 //   B: Z_{mu nu}(n) = c5 (S3_{mu rho} + S3_{mu sig})(n)
 //                    + c7 (wrap_rho S3_{mu sig} + wrap_sig S3_{mu rho})(n),
-//      with S3 = S^+ + S^- and {rho, sig} the two directions other than mu, nu;
-//   C: F_mu(n) = c1 U_mu(n) + sum_{nu,s} [ c3 S^s_{mu nu}(n)
-//                + wrap^s_nu( Z_{mu nu} + cL S^s_{mu nu} )(n) ],
+//      {rho, sig} the two directions other than mu, nu; with a Lepage term
+//      Y^s = Z + cL S^s, which takes the place of S^s;
+//   C: F_mu(n) = c1 U_mu(n) + sum_nu [ c3 S3_{mu nu}(n) + sum_s wrap^s_nu(Y^s_{mu nu})(n) ]
+//      (Y^s = Z without a Lepage term),
 // where wrap^+_d X (n) = U_d(n) X(n+d) U_d(n+mu)^+ and
 //       wrap^-_d X (n) = U_d(n-d)^+ X(n-d) U_d(n-d+mu).
 // Expanding C gives every 5-link staple (outer nu, inner rho) with c5, every
@@ -28,12 +29,24 @@
 //
 // Arithmetic: on this GPU an FP64 FMA issues at 1/64 of the FP32 rate, and the FP64 version of these
 // kernels ran with the FP64 pipe 90-97% busy. The staple products therefore run in float-float
-// arithmetic: every real is an unevaluated sum hi + lo of two floats (48-bit significand), a complex
-// number a float4 (re_hi, re_lo, im_hi, im_lo) of the same 16 bytes as a double2, and each product
-// is accumulated by error-free transformations on the FP32 pipe (ff_arith.cuh: TwoProduct with an
-// FMA, Dekker 1971; TwoSum, Knuth). The fields in the workspace are float-float; the thin links are
-// split at the first kernel, the U(3) projection runs in FP64 on the joined values (its Newton
-// steps need division and square roots), and the outputs are joined back to FP64.
+// arithmetic: every real is an unevaluated sum hi + lo of two floats (48-bit significand), and products
+// accumulate by error-free transformations on the FP32 pipe. The fields in the workspace hold a complex
+// number as the pairs (re_hi, im_hi) and (re_lo, im_lo), 16 bytes like a double2: re and im go through the
+// same operations, so every step is one packed two-lane FP32 instruction (sm_100 and later):
+//   TwoProduct(a, b) = (p, e): p = fl(a b), e = fma(a, b, -p)   exact (Dekker 1971, with an FMA)
+//   TwoSum(s, p) = (s', t): s' = fl(s + p), v = s' - s, t = (s - (s' - v)) + (p - v)   exact (Knuth, TAOCP
+//                  vol. 2, 4.2.2)
+// with e, t and the cross terms a_lo b and a b_lo in the low word. (Summing with s' = fma(a, b, s) instead saves three
+// instructions in twelve but is not exact where s and a b cancel: their difference can need more than 24 bits.)
+// The thin links are split at the first kernel, the U(3) projection divides in FP64, and the outputs are
+// joined back to FP64.
+//
+// A thread computes one row of a matrix: row i of a product needs row i of the left factor only, and both
+// products of a wrap keep their rows. With whole matrices in a thread these kernels took 168-232 registers, so that
+// 12-24% of the warp slots hid the latency of the accumulation chains (FMA pipe 52-60% busy). A block is 64 sites
+// x 3 rows, so the right factors that three threads read come from L1 for two of them. 24^3 x 32: 12.8 -> 9.9 ms,
+// the packed instructions (two pipe slots each) filling 72% of the FMA pipe; kernel A 1.33 -> 1.06 ms, B 2.63 -> 2.12,
+// C 1.66 -> 1.14 (level 1), at 5, 4 and 4 blocks a SM (one fewer each: 10.9 ms; five for all: 10.0).
 #include <math.h>
 #include <string.h>
 
@@ -49,24 +62,351 @@ struct Lat {
   long V;
 };
 
-// ---- float-float 3x3 complex matrices (the staple products) ----
+// ---- packed float-float complex numbers ----
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 pk(float x, float y) {
+  f32x2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+  return d;
+}
+__device__ __forceinline__ float2 upk(f32x2 a) {
+  float2 d;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(a));
+  return d;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
+struct __align__(16) C2 {  // complex: (re, im) high and low words
+  f32x2 h, l;
+};
+__device__ __forceinline__ C2 czero() { return {0ull, 0ull}; }
+__device__ __forceinline__ C2 cswap(C2 a) {  // (im, re)
+  const float2 h = upk(a.h), l = upk(a.l);
+  return {pk(h.y, h.x), pk(l.y, l.x)};
+}
+__device__ __forceinline__ C2 from_double(double2 v) {
+  const float4 f = split_ff(v);
+  return {pk(f.x, f.z), pk(f.y, f.w)};
+}
+__device__ __forceinline__ double2 to_double(C2 a) {
+  const float2 h = upk(a.h), l = upk(a.l);
+  return make_double2((double)h.x + (double)l.x, (double)h.y + (double)l.y);
+}
+
+// fl(a b). Written as an FMA with zero: the assembler joins a packed multiply and the addition that takes its
+// result into one FMA, whatever rounding they name, and the error terms below would be those of another sum.
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) { return fma2(a, b, 0ull); }
+
+// acc += a b lane by lane, a = (ah, al), na = -ah, b = (bh, bl); the low word is not renormalised in between
+__device__ __forceinline__ void acc2(C2& acc, f32x2 ah, f32x2 na, f32x2 al, C2 b) {
+  const f32x2 np = mul2(na, b.h);  // -p
+  const f32x2 e = fma2(ah, b.l, fma2(al, b.h, fma2(ah, b.h, np)));
+  const f32x2 s = sub2(acc.h, np);
+  const f32x2 v = sub2(s, acc.h);
+  const f32x2 t = sub2(sub2(acc.h, sub2(s, v)), add2(np, v));
+  acc.l = add2(acc.l, add2(t, e));
+  acc.h = s;
+}
+// acc = a b
+__device__ __forceinline__ void first2(C2& acc, f32x2 ah, f32x2 na, f32x2 al, C2 b) {
+  acc.h = mul2(ah, b.h);
+  acc.l = fma2(ah, b.l, fma2(al, b.h, fma2(ah, b.h, mul2(na, b.h))));
+}
+__device__ __forceinline__ void cnorm(C2& a) {
+  const f32x2 s = add2(a.h, a.l);
+  a.l = sub2(a.l, sub2(s, a.h));
+  a.h = s;
+}
+// a += b, renormalised
+__device__ __forceinline__ void cadd(C2& a, C2 b) {
+  const f32x2 s = add2(a.h, b.h);
+  const f32x2 v = sub2(s, a.h);
+  f32x2 e = add2(sub2(a.h, sub2(s, v)), sub2(b.h, v));
+  e = add2(e, add2(a.l, b.l));
+  a.h = add2(s, e);
+  a.l = sub2(e, sub2(a.h, s));
+}
+
+// The left operand of products, its components spread over the lanes with the signs of the form:
+// PLAIN a b, CONJ_L a^* b, CONJ_R a b^*
+enum Form { PLAIN = 0, CONJ_L = 1, CONJ_R = 2 };
+struct Left {
+  f32x2 rh, nrh, rl, ih, nih, il;  // nrh = -rh, nih = -ih
+};
+template <Form F>
+__device__ __forceinline__ Left left(C2 a) {
+  const float2 h = upk(a.h), l = upk(a.l);
+  if (F == PLAIN)
+    return {pk(h.x, h.x), pk(-h.x, -h.x), pk(l.x, l.x), pk(-h.y, h.y), pk(h.y, -h.y), pk(-l.y, l.y)};
+  if (F == CONJ_L)
+    return {pk(h.x, h.x), pk(-h.x, -h.x), pk(l.x, l.x), pk(h.y, -h.y), pk(-h.y, h.y), pk(l.y, -l.y)};
+  return {pk(h.x, -h.x), pk(-h.x, h.x), pk(l.x, -l.x), pk(h.y, h.y), pk(-h.y, -h.y), pk(l.y, l.y)};
+}
+template <bool FIRST = false>
+__device__ __forceinline__ void cmac(C2& acc, const Left& a, C2 b) {
+  if (FIRST) first2(acc, a.rh, a.nrh, a.rl, b);
+  else acc2(acc, a.rh, a.nrh, a.rl, b);
+  acc2(acc, a.ih, a.nih, a.il, cswap(b));
+}
+// acc += c a for a float-float real c
+__device__ __forceinline__ void caxpy(C2& acc, float2 c, C2 a) {
+  acc2(acc, pk(c.x, c.x), pk(-c.x, -c.x), pk(c.y, c.y), a);
+  cnorm(acc);
+}
+
+struct R3 {  // a row
+  C2 e[3];
+};
+__device__ __forceinline__ R3 rzero() {
+  R3 r;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) r.e[j] = czero();
+  return r;
+}
+
+// element k of field f at site n: fields [f][e][V]
+__device__ __forceinline__ C2 ld(const C2* __restrict__ f, long V, long n, int e) {
+  const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(f + (size_t)e * V + n));
+  return {v.x, v.y};
+}
+__device__ __forceinline__ const C2* field(const C2* base, int k, long V) { return base + (size_t)k * 9 * V; }
+__device__ __forceinline__ R3 ld_row(const C2* __restrict__ f, long V, long n, int i) {
+  R3 r;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) r.e[j] = ld(f, V, n, 3 * i + j);
+  return r;
+}
+__device__ __forceinline__ void st_row(C2* f, long V, long n, int i, const R3& r) {
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+    *reinterpret_cast<ulonglong2*>(f + (size_t)(3 * i + j) * V + n) = make_ulonglong2(r.e[j].h, r.e[j].l);
+}
+
+// acc += row i of A X (FIRST: acc = ...): a[k] = A_ik
+template <Form F, bool FIRST = false>
+__device__ __forceinline__ void row_mul(R3& acc, const R3& a, const C2* __restrict__ X, long V, long n) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const Left l = left<F>(a.e[k]);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      if (FIRST && k == 0) cmac<true>(acc.e[j], l, ld(X, V, n, 3 * k + j));
+      else cmac(acc.e[j], l, ld(X, V, n, 3 * k + j));
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 3; ++j) cnorm(acc.e[j]);
+}
+// acc += (row a) B^+
+__device__ __forceinline__ void row_mul_dag(R3& acc, const R3& a, const C2* __restrict__ B, long V, long n) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const Left l = left<CONJ_R>(a.e[k]);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) cmac(acc.e[j], l, ld(B, V, n, 3 * j + k));
+  }
+#pragma unroll
+  for (int j = 0; j < 3; ++j) cnorm(acc.e[j]);
+}
+
+// A direction at a site: index offset of the neighbour k steps on (periodic, |k| < L)
+struct Dir {
+  int c, L;
+  long st;
+  __device__ __forceinline__ long off(int k) const {
+    const int x = c + k;
+    return (x >= L ? k - L : x < 0 ? k + L : k) * st;
+  }
+};
+__device__ __forceinline__ Dir dir_of(const Lat& g, long n, int d) {
+  const long st = d == 0 ? 1 : d == 1 ? g.L[0] : d == 2 ? (long)g.L[0] * g.L[1] : (long)g.L[0] * g.L[1] * g.L[2];
+  const int L = d == 0 ? g.L[0] : d == 1 ? g.L[1] : d == 2 ? g.L[2] : g.L[3];
+  return {(int)((n / st) % L), L, st};
+}
+// the i-th direction other than mu (increasing order), and the inverse
+__device__ __forceinline__ int other(int mu, int i) { return i + (i >= mu ? 1 : 0); }
+__device__ __forceinline__ int other_index(int mu, int d) { return d - (d > mu ? 1 : 0); }
+// staple fields: single-sign S^s_{mu d} at (mu*3 + index of d)*2 + s, their sum S3_{mu d} at 24 + mu*3 + index
+constexpr int kNumS = 36;
+__device__ __forceinline__ int s3_field(int mu, int d) { return 24 + mu * 3 + other_index(mu, d); }
+
+// acc += row i of wrap^s_d X at n, X a field in direction mu
+__device__ __forceinline__ void wrap_row(R3& acc, const C2* __restrict__ U, long V, long n, const Dir& dmu, const Dir& dd,
+                                         int d, int s, const C2* __restrict__ X, int i) {
+  const C2* Ud = field(U, d, V);
+  if (s == 0) {
+    R3 m;
+    row_mul<PLAIN, true>(m, ld_row(Ud, V, n, i), X, V, n + dd.off(1));
+    row_mul_dag(acc, m, Ud, V, n + dmu.off(1));
+  } else {
+    const long y = n + dd.off(-1);
+    R3 a, m;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) a.e[k] = ld(Ud, V, y, 3 * k + i);
+    row_mul<CONJ_L, true>(m, a, X, V, y);
+    row_mul<PLAIN>(acc, m, Ud, V, y + dmu.off(1));
+  }
+}
+
+// threads of the staple kernels: sites x rows
+constexpr int kSites = 64;
+
+// host AoS [V][4][9] (FP64) -> [mu][e][V] (float-float)
+__global__ void __launch_bounds__(kThreads) k_links_to_fields(Lat g, const double2* __restrict__ aos,
+                                                              C2* __restrict__ U) {
+  const long n = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (n >= g.V) return;
+  const int mu = blockIdx.y;
+#pragma unroll
+  for (int e = 0; e < 9; ++e) {
+    const C2 v = from_double(aos[((size_t)n * 4 + mu) * 9 + e]);
+    *reinterpret_cast<ulonglong2*>(U + ((size_t)mu * 9 + e) * g.V + n) = make_ulonglong2(v.h, v.l);
+  }
+}
+
+// A: 3-staples S^+_{mu nu}, S^-_{mu nu} (s = 0 forward, 1 backward; written if `signs`) and S3_{mu nu} = S^+ + S^-
+__global__ void __launch_bounds__(3 * kSites, 5) k_staple3(Lat g, const C2* __restrict__ U, C2* __restrict__ S, int signs) {
+  const long n = (long)blockIdx.x * kSites + threadIdx.x, V = g.V;
+  if (n >= V) return;
+  const int i = threadIdx.y;
+  const int f = blockIdx.y;  // mu*3 + nu index
+  const int mu = f / 3, nu = other(mu, f % 3);
+  const Dir dmu = dir_of(g, n, mu), dnu = dir_of(g, n, nu);
+  const C2* X = field(U, mu, V);
+  R3 sp = rzero(), sm = rzero();
+  wrap_row(sp, U, V, n, dmu, dnu, nu, 0, X, i);
+  wrap_row(sm, U, V, n, dmu, dnu, nu, 1, X, i);
+  if (signs) {
+    st_row(S + (size_t)(2 * f) * 9 * V, V, n, i, sp);
+    st_row(S + (size_t)(2 * f + 1) * 9 * V, V, n, i, sm);
+  }
+#pragma unroll
+  for (int j = 0; j < 3; ++j) cadd(sm.e[j], sp.e[j]);
+  st_row(S + (size_t)(24 + f) * 9 * V, V, n, i, sm);
+}
+
+// B: Z_{mu nu} = c5 (S3_{mu rho} + S3_{mu sig}) + c7 (wrap_rho S3_{mu sig} + wrap_sig S3_{mu rho})
+// (c5, c7 as float-float pairs; a zero coefficient skips its term); cL = 0: written to Z, else
+// Y^s = Z + cL S^s in place of S^s
+__global__ void __launch_bounds__(3 * kSites, 4) k_staple57(Lat g, const C2* __restrict__ U, C2* S, float2 c5, float2 c7,
+                                                         float2 cL, C2* __restrict__ Z) {
+  const long n = (long)blockIdx.x * kSites + threadIdx.x, V = g.V;
+  if (n >= V) return;
+  const int i = threadIdx.y;
+  const int f = blockIdx.y;  // mu*3 + nu index
+  const int mu = f / 3, nu = other(mu, f % 3);
+  int rho = 0;
+  while (rho == mu || rho == nu) ++rho;
+  const int sig = 6 - mu - nu - rho;
+  const C2* S3r = field(S, s3_field(mu, rho), V);
+  const C2* S3s = field(S, s3_field(mu, sig), V);
+  R3 z = rzero();
+  if (c5.x != 0.f) {
+    R3 t = ld_row(S3r, V, n, i);
+    const R3 u = ld_row(S3s, V, n, i);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      cadd(t.e[j], u.e[j]);
+      caxpy(z.e[j], c5, t.e[j]);
+    }
+  }
+  if (c7.x != 0.f) {
+    const Dir dmu = dir_of(g, n, mu);
+    R3 w = rzero();
+#pragma unroll 1
+    for (int q = 0; q < 2; ++q) {
+      const int d = q == 0 ? rho : sig;
+      const Dir dd = dir_of(g, n, d);
+      const C2* X = q == 0 ? S3s : S3r;
+      wrap_row(w, U, V, n, dmu, dd, d, 0, X, i);
+      wrap_row(w, U, V, n, dmu, dd, d, 1, X, i);
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) caxpy(z.e[j], c7, w.e[j]);
+  }
+  if (cL.x == 0.f) {
+    st_row(Z + (size_t)f * 9 * V, V, n, i, z);
+    return;
+  }
+#pragma unroll 1
+  for (int s = 0; s < 2; ++s) {
+    C2* Y = S + (size_t)(2 * f + s) * 9 * V;
+    R3 y = z;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(Y + (size_t)(3 * i + j) * V + n);
+      caxpy(y.e[j], cL, C2{v.x, v.y});
+    }
+    st_row(Y, V, n, i, y);
+  }
+}
+
+// C: F_mu = c1 U_mu + sum_nu [ c3 S3_{mu nu} + sum_s wrap^s_nu Y^s_{mu nu} ], Y^s at Y + (f per_sign + s (per_sign - 1))
+// fields for f = mu*3 + nu index: Z with per_sign = 1, the fields in place of S^s with 2; none if Y is null.
+// out: float-float structure of arrays [mu][e][V], or FP64 in the host order [V][4][9] when aos != 0
+__global__ void __launch_bounds__(3 * kSites, 4) k_smear_links(Lat g, const C2* __restrict__ U, const C2* __restrict__ S,
+                                                            const C2* __restrict__ Y, int per_sign, float2 c1, float2 c3,
+                                                            int aos, void* __restrict__ out) {
+  const long n = (long)blockIdx.x * kSites + threadIdx.x, V = g.V;
+  if (n >= V) return;
+  const int i = threadIdx.y, mu = blockIdx.y;
+  const Dir dmu = dir_of(g, n, mu);
+  R3 F = rzero();
+  {
+    const R3 u = ld_row(field(U, mu, V), V, n, i);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) caxpy(F.e[j], c1, u.e[j]);
+  }
+#pragma unroll 1
+  for (int q = 0; q < 3; ++q) {
+    const int nu = other(mu, q), f = mu * 3 + q;
+    if (c3.x != 0.f) {  // both signs: S3_{mu nu}
+      const R3 t = ld_row(field(S, 24 + f, V), V, n, i);
+#pragma unroll
+      for (int j = 0; j < 3; ++j) caxpy(F.e[j], c3, t.e[j]);
+    }
+    if (Y) {
+      const Dir dnu = dir_of(g, n, nu);
+      const C2* Yf = field(Y, f * per_sign, V);
+      wrap_row(F, U, V, n, dmu, dnu, nu, 0, Yf, i);
+      wrap_row(F, U, V, n, dmu, dnu, nu, 1, field(Yf, per_sign - 1, V), i);
+    }
+  }
+  if (aos) {
+    double2* p = static_cast<double2*>(out) + ((size_t)n * 4 + mu) * 9 + 3 * i;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) p[j] = to_double(F.e[j]);
+  } else {
+    st_row(static_cast<C2*>(out) + (size_t)mu * 9 * V, V, n, i, F);
+  }
+}
+
+// ---- float-float 3x3 complex matrices with a thread each (the projection) ----
 struct F3 {
   float4 e[9];
 };
-
-// acc += a b, acc += a conj(b), acc += conj(a) b (float-float complex; the low words are not
-// renormalised in between: fnorm after a few terms)
+// acc += a b, acc += conj(a) b (float-float complex; the low words are not renormalised in between: fnorm
+// after a few terms)
 __device__ __forceinline__ void fcfma(float4& acc, float4 a, float4 b) {
   ff_acc(acc.x, acc.y, a.x, a.y, b.x, b.y);
   ff_acc(acc.x, acc.y, -a.z, -a.w, b.z, b.w);
   ff_acc(acc.z, acc.w, a.x, a.y, b.z, b.w);
   ff_acc(acc.z, acc.w, a.z, a.w, b.x, b.y);
-}
-__device__ __forceinline__ void fcfma_cb(float4& acc, float4 a, float4 b) {
-  ff_acc(acc.x, acc.y, a.x, a.y, b.x, b.y);
-  ff_acc(acc.x, acc.y, a.z, a.w, b.z, b.w);
-  ff_acc(acc.z, acc.w, a.z, a.w, b.x, b.y);
-  ff_acc(acc.z, acc.w, -a.x, -a.y, b.z, b.w);
 }
 __device__ __forceinline__ void fcfma_ca(float4& acc, float4 a, float4 b) {
   ff_acc(acc.x, acc.y, a.x, a.y, b.x, b.y);
@@ -77,269 +417,6 @@ __device__ __forceinline__ void fcfma_ca(float4& acc, float4 a, float4 b) {
 __device__ __forceinline__ void fnorm(float4& v) {
   ff_norm(v.x, v.y);
   ff_norm(v.z, v.w);
-}
-__device__ __forceinline__ F3 fzero() {
-  F3 m;
-#pragma unroll
-  for (int e = 0; e < 9; ++e) m.e[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-  return m;
-}
-
-__device__ __forceinline__ F3 fmm(const F3& A, const F3& B) {  // A B
-  F3 C;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) fcfma(s, A.e[i * 3 + k], B.e[k * 3 + j]);
-      fnorm(s);
-      C.e[i * 3 + j] = s;
-    }
-  return C;
-}
-__device__ __forceinline__ F3 fmm_nd(const F3& A, const F3& B) {  // A B^+
-  F3 C;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) fcfma_cb(s, A.e[i * 3 + k], B.e[j * 3 + k]);
-      fnorm(s);
-      C.e[i * 3 + j] = s;
-    }
-  return C;
-}
-__device__ __forceinline__ F3 fmm_dn(const F3& A, const F3& B) {  // A^+ B
-  F3 C;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) fcfma_ca(s, A.e[k * 3 + i], B.e[k * 3 + j]);
-      fnorm(s);
-      C.e[i * 3 + j] = s;
-    }
-  return C;
-}
-// C += A B and C += A B^+, renormalised after the three terms of each element
-__device__ __forceinline__ void fmm_acc(F3& C, const F3& A, const F3& B) {
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-#pragma unroll
-      for (int k = 0; k < 3; ++k) fcfma(C.e[i * 3 + j], A.e[i * 3 + k], B.e[k * 3 + j]);
-      fnorm(C.e[i * 3 + j]);
-    }
-}
-__device__ __forceinline__ void fmm_nd_acc(F3& C, const F3& A, const F3& B) {
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-#pragma unroll
-      for (int k = 0; k < 3; ++k) fcfma_cb(C.e[i * 3 + j], A.e[i * 3 + k], B.e[j * 3 + k]);
-      fnorm(C.e[i * 3 + j]);
-    }
-}
-// Y += a X for a float-float real a = (ah, al)
-__device__ __forceinline__ void faxpy(F3& Y, float2 a, const F3& X) {
-#pragma unroll
-  for (int e = 0; e < 9; ++e) {
-    ff_acc(Y.e[e].x, Y.e[e].y, a.x, a.y, X.e[e].x, X.e[e].y);
-    ff_acc(Y.e[e].z, Y.e[e].w, a.x, a.y, X.e[e].z, X.e[e].w);
-    fnorm(Y.e[e]);
-  }
-}
-// Y += X (float-float: TwoSum of the high words, low words added to the error, renormalised)
-__device__ __forceinline__ void ff_add(float& h, float& l, float bh, float bl) {
-  const float s = __fadd_rn(h, bh);
-  const float v = __fsub_rn(s, h);
-  float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, v)), __fsub_rn(bh, v));
-  e = __fadd_rn(e, __fadd_rn(l, bl));
-  h = __fadd_rn(s, e);
-  l = __fsub_rn(e, __fsub_rn(h, s));
-}
-__device__ __forceinline__ void faddto(F3& Y, const F3& X) {
-#pragma unroll
-  for (int e = 0; e < 9; ++e) {
-    ff_add(Y.e[e].x, Y.e[e].y, X.e[e].x, X.e[e].y);
-    ff_add(Y.e[e].z, Y.e[e].w, X.e[e].z, X.e[e].w);
-  }
-}
-
-// field k of a structure-of-arrays float-float buffer: elements [k][e][V]
-__device__ __forceinline__ F3 fld(const float4* __restrict__ f, int k, long V, long n) {
-  F3 m;
-  const float4* p = f + (size_t)k * 9 * V + n;
-#pragma unroll
-  for (int e = 0; e < 9; ++e) m.e[e] = __ldg(p + (size_t)e * V);
-  return m;
-}
-__device__ __forceinline__ void fst(float4* __restrict__ f, int k, long V, long n, const F3& m) {
-  float4* p = f + (size_t)k * 9 * V + n;
-#pragma unroll
-  for (int e = 0; e < 9; ++e) p[(size_t)e * V] = m.e[e];
-}
-
-__device__ __forceinline__ void coords(const Lat& g, long n, int c[4]) {
-  c[0] = (int)(n % g.L[0]);
-  n /= g.L[0];
-  c[1] = (int)(n % g.L[1]);
-  n /= g.L[1];
-  c[2] = (int)(n % g.L[2]);
-  c[3] = (int)(n / g.L[2]);
-}
-// lex index of c + k1 e_d1 + k2 e_d2 (periodic; |k| <= 3 < L)
-__device__ __forceinline__ long nb(const Lat& g, const int c[4], int d1, int k1, int d2 = 0, int k2 = 0) {
-  int cc[4] = {c[0], c[1], c[2], c[3]};
-  cc[d1] += k1;
-  cc[d2] += k2;
-#pragma unroll
-  for (int d = 0; d < 4; ++d) {
-    if (cc[d] < 0) cc[d] += g.L[d];
-    if (cc[d] >= g.L[d]) cc[d] -= g.L[d];
-  }
-  return cc[0] + (long)g.L[0] * (cc[1] + (long)g.L[1] * (cc[2] + (long)g.L[2] * cc[3]));
-}
-// the i-th direction other than mu (increasing order), and the inverse
-__device__ __forceinline__ int other(int mu, int i) { return i + (i >= mu ? 1 : 0); }
-__device__ __forceinline__ int other_index(int mu, int d) { return d - (d > mu ? 1 : 0); }
-// staple fields: single-sign S^s_{mu d} at (mu*3 + index of d)*2 + s, their sum S3_{mu d} at 24 + mu*3 + index
-constexpr int kNumS = 36;
-__device__ __forceinline__ int s3_field(int mu, int d) { return 24 + mu * 3 + other_index(mu, d); }
-
-// wrap^s_d X (n) for the direction-mu field X given at the displaced site
-__device__ __forceinline__ F3 wrap(const Lat& g, const float4* __restrict__ U, const int c[4], long n, int mu, int d,
-                                   int s, const F3& Xd) {
-  if (s == 0) {
-    const F3 a = fld(U, d, g.V, n);
-    const F3 b = fld(U, d, g.V, nb(g, c, mu, 1));
-    return fmm_nd(fmm(a, Xd), b);
-  }
-  const F3 a = fld(U, d, g.V, nb(g, c, d, -1));
-  const F3 b = fld(U, d, g.V, nb(g, c, d, -1, mu, 1));
-  return fmm(fmm_dn(a, Xd), b);
-}
-
-// acc += wrap^s_d X (n)
-__device__ __forceinline__ void wrap_acc(F3& acc, const Lat& g, const float4* __restrict__ U, const int c[4], long n,
-                                         int mu, int d, int s, const F3& Xd) {
-  if (s == 0) {
-    const F3 a = fld(U, d, g.V, n);
-    const F3 b = fld(U, d, g.V, nb(g, c, mu, 1));
-    fmm_nd_acc(acc, fmm(a, Xd), b);
-    return;
-  }
-  const F3 a = fld(U, d, g.V, nb(g, c, d, -1));
-  const F3 b = fld(U, d, g.V, nb(g, c, d, -1, mu, 1));
-  fmm_acc(acc, fmm_dn(a, Xd), b);
-}
-
-// host AoS [V][4][9] (FP64) -> [mu][e][V] (float-float)
-__global__ void __launch_bounds__(kThreads) k_links_to_fields(Lat g, const double2* __restrict__ aos,
-                                                              float4* __restrict__ U) {
-  const long n = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= g.V) return;
-  const int mu = blockIdx.y;
-#pragma unroll
-  for (int e = 0; e < 9; ++e) U[((size_t)mu * 9 + e) * g.V + n] = split_ff(aos[((size_t)n * 4 + mu) * 9 + e]);
-}
-
-// A: 3-staples S^+_{mu nu}, S^-_{mu nu} (s = 0 forward, 1 backward) and S3_{mu nu} = S^+ + S^-
-__global__ void __launch_bounds__(kThreads) k_staple3(Lat g, const float4* __restrict__ U, float4* __restrict__ S) {
-  const long n = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= g.V) return;
-  const int f = blockIdx.y;  // mu*3 + nu index
-  const int mu = f / 3, nu = other(mu, f % 3);
-  int c[4];
-  coords(g, n, c);
-  const F3 sp = wrap(g, U, c, n, mu, nu, 0, fld(U, mu, g.V, nb(g, c, nu, 1)));
-  fst(S, 2 * f, g.V, n, sp);
-  F3 sm = wrap(g, U, c, n, mu, nu, 1, fld(U, mu, g.V, nb(g, c, nu, -1)));
-  fst(S, 2 * f + 1, g.V, n, sm);
-  faddto(sm, sp);
-  fst(S, 24 + f, g.V, n, sm);
-}
-
-// B: Z_{mu nu} = c5 (S3_{mu rho} + S3_{mu sig}) + c7 (wrap_rho S3_{mu sig} + wrap_sig S3_{mu rho})
-// (c5, c7 as float-float pairs; a zero coefficient skips its term)
-__global__ void __launch_bounds__(kThreads) k_staple57(Lat g, const float4* __restrict__ U,
-                                                       const float4* __restrict__ S, float2 c5, float2 c7,
-                                                       float4* __restrict__ Z) {
-  const long n = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= g.V) return;
-  const int f = blockIdx.y;  // mu*3 + nu index
-  const int mu = f / 3, nu = other(mu, f % 3);
-  int rs[2], k = 0;
-  for (int d = 0; d < 4; ++d)
-    if (d != mu && d != nu) rs[k++] = d;
-  int c[4];
-  coords(g, n, c);
-  F3 z = fzero();
-  if (c5.x != 0.f) {
-    F3 t = fld(S, s3_field(mu, rs[0]), g.V, n);
-    faddto(t, fld(S, s3_field(mu, rs[1]), g.V, n));
-    faxpy(z, c5, t);
-  }
-  if (c7.x != 0.f) {
-    F3 w = fzero();
-    for (int q = 0; q < 2; ++q) {
-      const int d = rs[q], inner = rs[1 - q];
-      for (int s = 0; s < 2; ++s) {
-        const F3 x = fld(S, s3_field(mu, inner), g.V, nb(g, c, d, s == 0 ? 1 : -1));
-        wrap_acc(w, g, U, c, n, mu, d, s, x);
-      }
-    }
-    faxpy(z, c7, w);
-  }
-  fst(Z, f, g.V, n, z);
-}
-
-// C: F_mu = c1 U_mu + sum_{nu,s} [ c3 S^s_{mu nu} + wrap^s_nu (Z_{mu nu} + cL S^s_{mu nu}) ]
-// out: float-float structure of arrays [mu][e][V], or FP64 in the host order [V][4][9] when aos != 0
-__global__ void __launch_bounds__(kThreads) k_smear_links(Lat g, const float4* __restrict__ U,
-                                                          const float4* __restrict__ S,
-                                                          const float4* __restrict__ Z, float2 c1, float2 c3,
-                                                          float2 cL, int use_z, int aos, void* __restrict__ out) {
-  const long n = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= g.V) return;
-  const int mu = blockIdx.y;
-  int c[4];
-  coords(g, n, c);
-  F3 F = fzero();
-  faxpy(F, c1, fld(U, mu, g.V, n));
-  for (int i = 0; i < 3; ++i) {
-    const int nu = other(mu, i);
-    if (c3.x != 0.f) faxpy(F, c3, fld(S, 24 + mu * 3 + i, g.V, n));  // both signs: S3_{mu nu}
-    for (int s = 0; s < 2; ++s) {
-      const int fs = (mu * 3 + i) * 2 + s;
-      if (!use_z && cL.x == 0.f) continue;
-      const long y = nb(g, c, nu, s == 0 ? 1 : -1);
-      F3 x;
-      if (use_z) {
-        x = fld(Z, mu * 3 + i, g.V, y);
-        if (cL.x != 0.f) faxpy(x, cL, fld(S, fs, g.V, y));
-      } else {
-        x = fzero();
-        faxpy(x, cL, fld(S, fs, g.V, y));
-      }
-      wrap_acc(F, g, U, c, n, mu, nu, s, x);
-    }
-  }
-  if (aos) {
-    double2* p = static_cast<double2*>(out) + ((size_t)n * 4 + mu) * 9;
-#pragma unroll
-    for (int e = 0; e < 9; ++e) p[e] = join_ff(F.e[e]);
-  } else {
-    fst(static_cast<float4*>(out), mu, g.V, n, F);
-  }
 }
 
 // U(3) projection W = V (V^+ V)^(-1/2): the unitary polar factor of V, by Newton's
@@ -355,11 +432,17 @@ constexpr int kMaxPolar = 40;
 
 __device__ __forceinline__ float4 fneg(float4 a) { return make_float4(-a.x, -a.y, -a.z, -a.w); }
 
-__global__ void __launch_bounds__(kThreads) k_u3_project(Lat g, float4* __restrict__ F, int* __restrict__ err) {
+__global__ void __launch_bounds__(kThreads) k_u3_project(Lat g, C2* __restrict__ F, int* __restrict__ err) {
   const long n = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= g.V) return;
   const int mu = blockIdx.y;
-  F3 X = fld(F, mu, g.V, n);
+  F3 X;
+#pragma unroll
+  for (int e = 0; e < 9; ++e) {
+    const C2 v = ld(field(F, mu, g.V), g.V, n, e);
+    const float2 h = upk(v.h), l = upk(v.l);
+    X.e[e] = make_float4(h.x, l.x, h.y, l.y);
+  }
   bool ok = false;
   for (int it = 0; it < kMaxPolar; ++it) {
     // cofactors C_ij = X_{i1 j1} X_{i2 j2} - X_{i1 j2} X_{i2 j1} and det = sum_j X_0j C_0j
@@ -419,26 +502,28 @@ __global__ void __launch_bounds__(kThreads) k_u3_project(Lat g, float4* __restri
     atomicExch(err, 1);
     return;
   }
-  fst(F, mu, g.V, n, X);
+#pragma unroll
+  for (int e = 0; e < 9; ++e)
+    *reinterpret_cast<ulonglong2*>(F + ((size_t)mu * 9 + e) * g.V + n) =
+        make_ulonglong2(pk(X.e[e].x, X.e[e].z), pk(X.e[e].y, X.e[e].w));
 }
 
 // long_mu(n) = naik W_mu(n) W_mu(n+mu) W_mu(n+2mu), written in FP64 in host order [V][4][9]
-__global__ void __launch_bounds__(kThreads) k_naik(Lat g, const float4* __restrict__ W, double naik,
-                                                   double2* __restrict__ out) {
-  const long n = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= g.V) return;
-  const int mu = blockIdx.y;
-  int c[4];
-  coords(g, n, c);
-  const F3 a = fld(W, mu, g.V, n);
-  const F3 b = fld(W, mu, g.V, nb(g, c, mu, 1));
-  const F3 d = fld(W, mu, g.V, nb(g, c, mu, 2));
-  const F3 p = fmm(fmm(a, b), d);
-  double2* o = out + ((size_t)n * 4 + mu) * 9;
+__global__ void __launch_bounds__(3 * kSites) k_naik(Lat g, const C2* __restrict__ W, double naik,
+                                                     double2* __restrict__ out) {
+  const long n = (long)blockIdx.x * kSites + threadIdx.x, V = g.V;
+  if (n >= V) return;
+  const int i = threadIdx.y, mu = blockIdx.y;
+  const Dir dmu = dir_of(g, n, mu);
+  const C2* Wm = field(W, mu, V);
+  R3 m, p;
+  row_mul<PLAIN, true>(m, ld_row(Wm, V, n, i), Wm, V, n + dmu.off(1));
+  row_mul<PLAIN, true>(p, m, Wm, V, n + dmu.off(2));
+  double2* o = out + ((size_t)n * 4 + mu) * 9 + 3 * i;
 #pragma unroll
-  for (int e = 0; e < 9; ++e) {
-    const double2 v = join_ff(p.e[e]);
-    o[e] = make_double2(naik * v.x, naik * v.y);
+  for (int j = 0; j < 3; ++j) {
+    const double2 v = to_double(p.e[j]);
+    o[j] = make_double2(naik * v.x, naik * v.y);
   }
 }
 
@@ -473,17 +558,19 @@ float2 ff_coeff(double c) {
 }
 
 // one smearing level: U (float-float fields) -> out (float-float fields, or FP64 host order when aos)
-int smear_level(const Lat& g, const float4* U, float4* S, float4* Z, const sqcg_smear_level& c, int aos, void* out,
-                cudaStream_t s) {
-  const dim3 blk(kThreads);
-  const unsigned gx = (unsigned)((g.V + kThreads - 1) / kThreads);
-  const bool need_s = c.three_staple != 0.0 || c.five_staple != 0.0 || c.seven_staple != 0.0 || c.lepage != 0.0;
-  const bool use_z = c.five_staple != 0.0 || c.seven_staple != 0.0;
-  if (need_s) k_staple3<<<dim3(gx, 12), blk, 0, s>>>(g, U, S);
-  if (use_z)
-    k_staple57<<<dim3(gx, 12), blk, 0, s>>>(g, U, S, ff_coeff(c.five_staple), ff_coeff(c.seven_staple), Z);
-  k_smear_links<<<dim3(gx, 4), blk, 0, s>>>(g, U, S, Z, ff_coeff(c.one_link), ff_coeff(c.three_staple),
-                                             ff_coeff(c.lepage), use_z ? 1 : 0, aos, out);
+int smear_level(const Lat& g, const C2* U, C2* S, C2* Z, const sqcg_smear_level& c, int aos, void* out, cudaStream_t s) {
+  const dim3 blk(kSites, 3);
+  const unsigned gx = (unsigned)((g.V + kSites - 1) / kSites);
+  const bool lepage = ff_coeff(c.lepage).x != 0.f;
+  const bool staples57 = ff_coeff(c.five_staple).x != 0.f || ff_coeff(c.seven_staple).x != 0.f;
+  const bool need_s = lepage || staples57 || ff_coeff(c.three_staple).x != 0.f;
+  if (need_s) k_staple3<<<dim3(gx, 12), blk, 0, s>>>(g, U, S, lepage ? 1 : 0);
+  if (lepage || staples57)
+    k_staple57<<<dim3(gx, 12), blk, 0, s>>>(g, U, S, ff_coeff(c.five_staple), ff_coeff(c.seven_staple),
+                                            ff_coeff(c.lepage), Z);
+  const C2* Y = lepage ? S : staples57 ? Z : nullptr;
+  k_smear_links<<<dim3(gx, 4), blk, 0, s>>>(g, U, S, Y, lepage ? 2 : 1, ff_coeff(c.one_link), ff_coeff(c.three_staple),
+                                            aos, out);
   return cudaGetLastError() == cudaSuccess ? SQCG_OK : SQCG_ERR_CUDA;
 }
 
@@ -508,10 +595,10 @@ extern "C" int sqcg_hisq_smear(const int dims[4], const void* thin, void* fat, v
   if (!finite_level(c.level1) || !finite_level(c.level2) || !isfinite(c.naik)) return SQCG_ERR_INVALID_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   const size_t nf = 9 * (size_t)g.V;
-  float4* U = (float4*)workspace;  // float-float fields, 16 bytes per complex element
-  float4* S = U + 4 * nf;
-  float4* Z = S + kNumS * nf;
-  float4* W = Z + 12 * nf;
+  C2* U = (C2*)workspace;  // float-float fields, 16 bytes per complex element
+  C2* S = U + 4 * nf;
+  C2* Z = S + kNumS * nf;
+  C2* W = Z + 12 * nf;
   int* err = (int*)(W + 4 * nf);
   const unsigned gx = (unsigned)((g.V + kThreads - 1) / kThreads);
   SQCG_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), s));
@@ -521,7 +608,7 @@ extern "C" int sqcg_hisq_smear(const int dims[4], const void* thin, void* fat, v
   k_u3_project<<<dim3(gx, 4), kThreads, 0, s>>>(g, W, err);
   SQCG_CUDA_TRY(cudaGetLastError());
   SQCG_TRY(smear_level(g, W, S, Z, c.level2, 1, fat, s));
-  k_naik<<<dim3(gx, 4), kThreads, 0, s>>>(g, W, c.naik, (double2*)lng);
+  k_naik<<<dim3((unsigned)((g.V + kSites - 1) / kSites), 4), dim3(kSites, 3), 0, s>>>(g, W, c.naik, (double2*)lng);
   SQCG_CUDA_TRY(cudaGetLastError());
   int h_err = 0;
   SQCG_CUDA_TRY(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, s));

@@ -153,3 +153,19 @@ def test_hisq_errors(sqcg):
         sqcg.hisq_smear(L, d, f, l, small)
     assert e.value.name == "INVALID_ARG"
     assert sqcg.hisq_workspace_bytes((4, 4, 4, 5)) == 0
+
+
+@pytest.mark.parametrize("l1", [{"one_link": 0.4, "three_staple": 0.05, "five_staple": 0.01, "seven_staple": 0.002,
+                                 "lepage": 0.03},
+                                {"one_link": 0.5, "lepage": 0.04}, {"one_link": 0.6}])
+def test_hisq_at_a_remainder_of_its_blocks(sqcg, l1):
+    """1296 sites: the last 64-site block holds 16. Each way a level can run: with the Lepage term in the place of the
+    single-sign staples, Lepage alone (no 5- and 7-link staples), the link alone; level 2 with all terms."""
+    L = (6, 6, 6, 6)
+    thin = synth.thin_links(L, 1400, width=0.3)
+    l2 = {"one_link": 1.0, "three_staple": 1 / 16, "five_staple": 1 / 64, "seven_staple": 1 / 384, "lepage": -1 / 8}
+    want_f, want_l = hisq.hisq_links(L, thin, level1=l1, level2=l2, naik_coeff=-1 / 24)
+    with sqcg.Lattice(L) as lat:
+        fat, lng = lat.hisq_load_links(thin, coeffs=sqcg.hisq_coeffs(l1, l2, -1 / 24), return_links=True)
+    assert maxrel(fat, want_f) <= TOL
+    assert maxrel(lng, want_l) <= TOL
