@@ -128,6 +128,18 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// Two FP64 sums over SUB consecutive lanes (SUB <= 32) with the additions of one: the lower half of the lanes goes
+// on with a, the upper half with b. Totals: a in the first lane, b in lane SUB / 2. (An FP64 addition holds its
+// scheduler for 64 cycles on this GPU, whatever the lanes in it.)
+template <int SUB>
+__device__ __forceinline__ double sum2(double a, double b) {
+  const bool upper = (threadIdx.x + threadIdx.y * blockDim.x) & (SUB / 2);
+  double v = (upper ? b : a) + __shfl_xor_sync(0xffffffffu, upper ? a : b, SUB / 2);
+#pragma unroll
+  for (int o = SUB / 4; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o, SUB / 2);
+  return v;
+}
+
 // decode a tile into (lattice, RHS block, site block); RHS blocks fastest
 __device__ __forceinline__ int find_lat(const LatDev* lats, int nlat, int tile, bool fp64) {
   int k = 0;
@@ -215,14 +227,61 @@ __device__ void rhs_block_partial(double (&v)[WT], const LatDev& L, int wbase, i
   }
 }
 
+// Which RHS blocks need the reliable update -> IF condition; run by a whole block, a thread per RHS block.
+__device__ void update_control(BatchState* st, const LatDev* lats, int nlat, int W) {
+  int any = 0;
+  for (int b = threadIdx.x; b < st->nblk; b += blockDim.x) {
+    int k = 0;
+    for (int j = 1; j < nlat; ++j)
+      if (b >= lats[j].rb0) k = j;
+    const LatDev& L = lats[k];
+    const int w0 = (b - L.rb0) * W;
+    int u = 0;
+    for (int w = w0; w < min(w0 + W, L.nrhs); ++w) u |= *(volatile int*)&st->r[L.rhs0 + w].need_update;
+    st->blk_update[b] = u;
+    any |= u;
+  }
+  any = __syncthreads_or(any);
+  if (threadIdx.x == 0) {
+    st->if_runs += any ? 1 : 0;
+    if (st->use_graph) cudaGraphSetConditional((cudaGraphConditionalHandle)st->h_if, any ? 1u : 0u);
+  }
+}
+
+// Active RHS blocks, loop count and the WHILE condition; run by one block beside the p update, which reads the
+// same flags: a block that stops being active has no active right-hand side either way.
+__device__ void loop_control(BatchState* st, const LatDev* lats, int nlat, int W) {
+  int any = 0;
+  for (int b = threadIdx.x; b < st->nblk; b += blockDim.x) {
+    int k = 0;
+    for (int j = 1; j < nlat; ++j)
+      if (b >= lats[j].rb0) k = j;
+    const LatDev& L = lats[k];
+    const int w0 = (b - L.rb0) * W;
+    int u = 0;
+    for (int w = w0; w < min(w0 + W, L.nrhs); ++w) u |= st->r[L.rhs0 + w].active;
+    st->blk_active[b] = u;
+    any |= u;
+  }
+  any = __syncthreads_or(any);
+  if (threadIdx.x == 0) {
+    st->loop_count += 1;
+    const int go = any && st->loop_count < st->loop_limit;  // at the bound the host gives the others their status
+    if (st->use_graph) cudaGraphSetConditional((cudaGraphConditionalHandle)st->h_while, go ? 1u : 0u);
+  }
+}
+
 // Second stage: one block per RHS adds its partials in site-block order and
-// runs the per-RHS scalar step (deterministic). blas: the partials come from
+// runs the per-RHS scalar step (deterministic); after the update's step the last block to finish also decides on
+// the reliable update. blas: the partials come from
 // the BLAS tiling (nsb_b site blocks) rather than the Dslash tiling (nsb).
 constexpr int kBatchFinishThreads = 1024;
 
 __global__ void __launch_bounds__(kBatchFinishThreads) k_batch_finish(BatchState* st, const LatDev* lats, int nlat,
                                                                       const double* partials, int max_nsb, int fin,
-                                                                      int blas) {
+                                                                      int blas, int W) {
+  pdl_wait();
+  pdl_launch_dependents();
   const int g = blockIdx.x;
   int k = 0;
   for (int j = 1; j < nlat; ++j)
@@ -243,7 +302,20 @@ __global__ void __launch_bounds__(kBatchFinishThreads) k_batch_finish(BatchState
   }
   for (; j < n; j += B) s0 += pp[j];
   const double s = block_sum((s0 + s1) + (s2 + s3));
-  if (threadIdx.x == 0) rhs_finish(st->r[g], st, fin, s);
+  __shared__ int last;
+  if (threadIdx.x == 0) {
+    rhs_finish(st->r[g], st, fin, s);
+    last = 0;
+    if (fin == BFIN_UPDATE) {
+      __threadfence();
+      last = atomicAdd(&st->arrived, 1u) == gridDim.x - 1;
+    }
+  }
+  __syncthreads();
+  if (fin != BFIN_UPDATE || !last) return;
+  __threadfence();
+  if (threadIdx.x == 0) st->arrived = 0u;
+  update_control(st, lats, nlat, W);
 }
 
 // ---------------------------------------------------------------------------
@@ -516,7 +588,10 @@ __global__ void __launch_bounds__(128, 6) k_mrhs_dslash_ff(MArgs a) {
   const int k = have_tile ? find_lat(a.lats, a.nlat, tile, true) : 0;
   const LatDev& L = a.lats[k];
   const int local = tile - L.tile640;
-  const int rb = have_tile ? local % L.nrb64 : 0, sb = have_tile ? local / L.nrb64 : 0;
+  // site blocks fastest: the slices of a CTA have the same right-hand sides, so in an update of a few of them whole
+  // CTAs have nothing to do (with RHS blocks fastest two thirds of every CTA idled in an 11-RHS solve: 421 us a pass
+  // for one right-hand side at 32^4, 254 now)
+  const int rb = have_tile ? local / L.nsb : 0, sb = have_tile ? local % L.nsb : 0;
   const int wbase = rb * WT;
   const int nw_tile = have_tile ? min(WT, L.nrhs - wbase) : 0;
   const int w0 = wbase;
@@ -632,18 +707,17 @@ __global__ void k_mrhs_flush_x(const LatDev* lats, int nlat, const BatchState* s
   const int w = g - L.rhs0;
   if (w >= L.nrhs) return;
   if (gated && !(st->r[g].need_update && st->r[g].active)) return;
-  const int Vh = L.g.Vh;
-  const size_t n = (size_t)3 * Vh, off = (size_t)w * n;
-  for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += (size_t)gridDim.x * blockDim.x) {
-    const int c = (int)(idx / Vh), i = (int)(idx % Vh);
+  const int Vh = L.g.Vh, c = blockIdx.z;
+  const size_t off = ((size_t)w * 3 + c) * Vh;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Vh; i += gridDim.x * blockDim.x) {
     float2* hp = L.xh + pv(w, c, i, Vh);
     const float2 h = *hp;
-    double2 v = L.x[off + idx];
+    double2 v = L.x[off + i];
     v.x += (double)h.x;
     v.y += (double)h.y;
-    L.x[off + idx] = v;
+    L.x[off + i] = v;
     *hp = make_float2(0.f, 0.f);
-    if (split) L.xff[off + idx] = split_ff(v);
+    if (split) L.xff[off + i] = split_ff(v);
   }
 }
 
@@ -657,12 +731,17 @@ __device__ void rhs_block_partial_m(double (&v)[WT], const LatDev& L, int wbase,
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
   const int lane = tid & 31;
   const int nchunk = blockDim.x / SUB;
-#pragma unroll
-  for (int w = 0; w < WT; ++w) {
-    double t = v[w];
+  if constexpr (WT == 1) {
+    double t = v[0];
 #pragma unroll
     for (int o = SUB / 2; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o, SUB);
-    if ((lane & (SUB - 1)) == 0) red[ay * WT + w][ax / SUB] = t;
+    if ((lane & (SUB - 1)) == 0) red[ay][ax / SUB] = t;
+  } else {
+#pragma unroll
+    for (int w = 0; w < WT; w += 2) {
+      const double t = sum2<SUB>(v[w], v[w + 1]);
+      if ((lane & (SUB / 2 - 1)) == 0) red[ay * WT + w + ((lane & (SUB / 2)) ? 1 : 0)][ax / SUB] = t;
+    }
   }
   __syncthreads();
   if (tid < nw_tile) {
@@ -733,7 +812,14 @@ __global__ void __launch_bounds__(kMaxThreads) k_mrhs_dslash_smem(MArgs a) {
   const int wbase = rb * Wtile;
   const int nw_tile = min(Wtile, L.nrhs - wbase);
   const int blk = L.rb0 + rb;
-  if (a.gate == GATE_ITER && !a.st->blk_active[blk]) return;
+  // launched while the kernel before it drains (programmatic dependent launch), the block stages its links first:
+  // nothing but the vectors and the state depends on that kernel. A right-hand side never becomes active again
+  // within a solve, so an inactive block seen early is one.
+  pdl_launch_dependents();
+  if (a.gate == GATE_ITER && !a.st->blk_active[blk]) {
+    pdl_wait();
+    return;
+  }
   const Geom& g = L.g;
   const int Vh = g.Vh;
   const int par = a.par, q = 1 - par;
@@ -781,6 +867,7 @@ __global__ void __launch_bounds__(kMaxThreads) k_mrhs_dslash_smem(MArgs a) {
       for (int e = 0; e < 9; ++e) sU[(h * 9 + e) * TX + threadIdx.x] = u[e];
     }
   }
+  pdl_wait();
   __syncthreads();
   // ---- apply to this thread's right-hand sides: thread (site ax, group ay) ----
   int ax = threadIdx.x, ay = threadIdx.y;
@@ -791,7 +878,13 @@ __global__ void __launch_bounds__(kMaxThreads) k_mrhs_dslash_smem(MArgs a) {
     ay = (warp / cpr) * 2 + (lane >> 4);
   }
   const int w0 = wbase + ay * WT;
-  const int nw = max(0, min(WT, L.nrhs - w0));
+  int nw = max(0, min(WT, L.nrhs - w0));
+  if (a.gate == GATE_ITER) {  // a group whose right-hand sides have all finished has nothing to do
+    bool any = false;
+#pragma unroll
+    for (int w = 0; w < WT; ++w) any = any || (w < nw && a.st->r[L.rhs0 + w0 + w].active);
+    if (!any) nw = 0;
+  }
   const int i = sb * TX + ax;
   const bool valid = i < Vh;
   double part[WT];
@@ -916,9 +1009,15 @@ __global__ void __launch_bounds__(kTB) k_mrhs_blas(BArgs a) {
     if ((int)blockIdx.x >= a.lats[j].sbt0) k = j;
   const LatDev& L = a.lats[k];
   const int w0 = 2 * blockIdx.y;
-  if (w0 >= L.nrhs) return;
+  if (w0 >= L.nrhs) {
+    pdl_wait();
+    return;
+  }
   const int nw = min(2, L.nrhs - w0);
   const int sb = blockIdx.x - L.sbt0;
+  pdl_wait();
+  pdl_launch_dependents();
+  if (a.op == B_XPAY && blockIdx.x == 0 && blockIdx.y == 0) loop_control(a.st, a.lats, a.nlat, a.W);
   const bool all = (a.op == B_NORM_B || a.op == B_NORM_X || a.op == B_INIT_B);
   bool act[2];
   double alpha[2], beta[2];
@@ -1007,52 +1106,18 @@ __global__ void __launch_bounds__(kTB) k_mrhs_blas(BArgs a) {
       for (int c = 0; c < 3; ++c) pv_store<2>(L.p, w0, nw, c, i, Vh, pc[c]);
     }
   }
-  if (a.op != B_XPAY) {
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const double t = block_sum(part[u]);
-      if (threadIdx.x == 0 && act[u]) a.partials[(size_t)(L.rhs0 + w0 + u) * a.max_nsb + sb] = t;
+  if (a.op != B_XPAY) {  // both sums of the block: a warp's at its lanes 0 and 16, then the warps' in order
+    __shared__ double red[2][kTB / 32];
+    const double t = sum2<32>(part[0], part[1]);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if ((lane & 15) == 0) red[lane >> 4][warp] = t;
+    __syncthreads();
+    if (threadIdx.x < 2 && act[threadIdx.x]) {
+      double v = 0.0;
+      for (int j = 0; j < kTB / 32; ++j) v += red[threadIdx.x][j];
+      a.partials[(size_t)(L.rhs0 + w0 + threadIdx.x) * a.max_nsb + sb] = v;
     }
   }
-}
-
-// One thread: which RHS blocks need the FP64 reliable update -> IF condition
-__global__ void k_batch_ctl_update(BatchState* st, const LatDev* lats, int nlat, int W) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  int any = 0;
-  for (int k = 0; k < nlat; ++k) {
-    const LatDev& L = lats[k];
-    for (int rb = 0; rb < L.nrb; ++rb) {
-      int u = 0;
-      for (int w = rb * W; w < min((rb + 1) * W, L.nrhs); ++w) u |= st->r[L.rhs0 + w].need_update;
-      st->blk_update[L.rb0 + rb] = u;
-      any |= u;
-    }
-  }
-  st->if_runs += any;
-  if (st->use_graph) cudaGraphSetConditional((cudaGraphConditionalHandle)st->h_if, any ? 1u : 0u);
-}
-
-// One thread: active RHS blocks, loop count and the WHILE condition
-__global__ void k_batch_ctl_loop(BatchState* st, const LatDev* lats, int nlat, int W) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  st->loop_count += 1;
-  int any = 0;
-  for (int k = 0; k < nlat; ++k) {
-    const LatDev& L = lats[k];
-    for (int rb = 0; rb < L.nrb; ++rb) {
-      int a = 0;
-      for (int w = rb * W; w < min((rb + 1) * W, L.nrhs); ++w) a |= st->r[L.rhs0 + w].active;
-      st->blk_active[L.rb0 + rb] = a;
-      any |= a;
-    }
-  }
-  const int go = any && st->loop_count < st->loop_limit;
-  if (!go && any) {  // hard bound reached: stop every RHS that is still running
-    for (int j = 0; j < st->nrhs; ++j)
-      if (st->r[j].active) { st->r[j].active = 0; st->r[j].status = SQCG_ERR_NOT_CONVERGED; }
-  }
-  if (st->use_graph) cudaGraphSetConditional((cudaGraphConditionalHandle)st->h_while, go ? 1u : 0u);
 }
 
 }  // namespace
@@ -1208,7 +1273,8 @@ int launch_mrhs_dslash_w(int WT, int G, int grid, int T, cudaStream_t s, const M
   return SQCG_OK;
 }
 
-int launch_mrhs_blas(const BatchPlan& P, int op, cudaStream_t s) {
+// pdl: the kernel before it on the stream is a kernel (programmatic dependent launch)
+int launch_mrhs_blas(const BatchPlan& P, int op, cudaStream_t s, bool pdl = false) {
   BArgs a;
   a.lats = P.dev; a.nlat = P.nlat; a.op = op; a.st = P.st; a.partials = P.partials; a.max_nsb = P.max_nsb; a.W = P.W;
   int maxr = 0, nsb = 0;
@@ -1216,8 +1282,7 @@ int launch_mrhs_blas(const BatchPlan& P, int op, cudaStream_t s) {
     maxr = P.nrhs[k] > maxr ? P.nrhs[k] : maxr;
     nsb += P.host[k].nsb_b;
   }
-  k_mrhs_blas<<<dim3(nsb, (maxr + 1) / 2), kTB, 0, s>>>(a);
-  SQCG_CUDA_TRY(cudaGetLastError());
+  SQCG_CUDA_TRY(launch_kernel(k_mrhs_blas, dim3(nsb, (maxr + 1) / 2), dim3(kTB), 0, s, pdl && P.ctx[0]->pdl, a));
   return SQCG_OK;
 }
 
@@ -1229,9 +1294,9 @@ MArgs margs(const BatchPlan& P, int par, int in_vec, int epi, int gate, int writ
   return a;
 }
 
-int launch_finish_b(const BatchPlan& P, int fin, int blas, cudaStream_t s) {
-  k_batch_finish<<<P.nrhs_total, kBatchFinishThreads, 0, s>>>(P.st, P.dev, P.nlat, P.partials, P.max_nsb, fin, blas);
-  SQCG_CUDA_TRY(cudaGetLastError());
+int launch_finish_b(const BatchPlan& P, int fin, int blas, cudaStream_t s) {  // always follows a kernel
+  SQCG_CUDA_TRY(launch_kernel(k_batch_finish, dim3(P.nrhs_total), dim3(kBatchFinishThreads), 0, s, P.ctx[0]->pdl != 0, P.st,
+                              P.dev, P.nlat, P.partials, P.max_nsb, fin, blas, P.W));
   return SQCG_OK;
 }
 
@@ -1264,7 +1329,7 @@ int set_carve(int WT, int sub, int carve) {
   return SQCG_OK;
 }
 
-int launch_f32(const BatchPlan& P, int par, int in_vec, int epi, int gate, cudaStream_t s) {
+int launch_f32(const BatchPlan& P, int par, int in_vec, int epi, int gate, cudaStream_t s, bool pdl = false) {
   const int G = P.W / P.WT, T = P.T;
   if (!smem_shape_ok(P.W, P.WT, T, P.sub)) return SQCG_ERR_INVALID_ARG;
   const size_t smem = (size_t)kHops * 9 * T * sizeof(float2);
@@ -1278,8 +1343,7 @@ int launch_f32(const BatchPlan& P, int par, int in_vec, int epi, int gate, cudaS
     attr_set[k] = true;
   }
   const MArgs a = margs(P, par, in_vec, epi, gate, 0);
-  smem_kernel(k)<<<P.ntiles, dim3(T, G), smem, s>>>(a);
-  SQCG_CUDA_TRY(cudaGetLastError());
+  SQCG_CUDA_TRY(launch_kernel(smem_kernel(k), dim3(P.ntiles), dim3(T, G), smem, s, pdl && P.ctx[0]->pdl, a));
   return SQCG_OK;
 }
 
@@ -1293,8 +1357,8 @@ int launch_f64(const BatchPlan& P, int par, int in_vec, int epi, int gate, int w
 int launch_flush_x(const BatchPlan& P, int gated, int split, cudaStream_t s) {
   int max_vh = 0;
   for (int k = 0; k < P.nlat; ++k) max_vh = P.host[k].g.Vh > max_vh ? P.host[k].g.Vh : max_vh;
-  const int gx = (int)(((size_t)3 * max_vh + 255) / 256 < 1024 ? ((size_t)3 * max_vh + 255) / 256 : 1024);
-  k_mrhs_flush_x<<<dim3(gx, P.nrhs_total), 256, 0, s>>>(P.dev, P.nlat, P.st, gated, split);
+  const int full = grid_for(max_vh, 256), gx = full < 1024 ? full : 1024;
+  k_mrhs_flush_x<<<dim3(gx, P.nrhs_total, 3), 256, 0, s>>>(P.dev, P.nlat, P.st, gated, split);
   SQCG_CUDA_TRY(cudaGetLastError());
   return SQCG_OK;
 }
@@ -1520,17 +1584,14 @@ int build_plan(int nctx, sqcg_ctx* const* ctx, const int* nrhs, const void* cons
   return SQCG_OK;
 }
 
-// One iteration in three parts: head (D_oe p; A p + <p,Ap>; x, r update; ctl), the FP64
-// reliable update r = b - A x of the blocks that asked for it, tail (p update; loop ctl)
+// One iteration in three parts: head (D_oe p; A p + <p,Ap>; x, r update, deciding on the reliable update), the
+// reliable update r = b - A x of the blocks that asked for it, tail (p update with the loop control)
 int enqueue_head(BatchPlan& P, cudaStream_t s) {
   SQCG_TRY(launch_f32(P, 1, V_P, M_PLAIN, GATE_ITER, s));
-  SQCG_TRY(launch_f32(P, 0, V_TMP, M_NORMAL_DOT, GATE_ITER, s));
+  SQCG_TRY(launch_f32(P, 0, V_TMP, M_NORMAL_DOT, GATE_ITER, s, true));
   SQCG_TRY(launch_finish_b(P, BFIN_PAP, 0, s));
-  SQCG_TRY(launch_mrhs_blas(P, B_UPDATE, s));
-  SQCG_TRY(launch_finish_b(P, BFIN_UPDATE, 1, s));
-  k_batch_ctl_update<<<1, 32, 0, s>>>(P.st, P.dev, P.nlat, P.W);
-  SQCG_CUDA_TRY(cudaGetLastError());
-  return SQCG_OK;
+  SQCG_TRY(launch_mrhs_blas(P, B_UPDATE, s, true));
+  return launch_finish_b(P, BFIN_UPDATE, 1, s);
 }
 
 int enqueue_reliable(BatchPlan& P, cudaStream_t s) {
@@ -1538,12 +1599,7 @@ int enqueue_reliable(BatchPlan& P, cudaStream_t s) {
   return launch_finish_b(P, BFIN_TRUE, 0, s);
 }
 
-int enqueue_tail(BatchPlan& P, cudaStream_t s) {
-  SQCG_TRY(launch_mrhs_blas(P, B_XPAY, s));
-  k_batch_ctl_loop<<<1, 32, 0, s>>>(P.st, P.dev, P.nlat, P.W);
-  SQCG_CUDA_TRY(cudaGetLastError());
-  return SQCG_OK;
-}
+int enqueue_tail(BatchPlan& P, cudaStream_t s) { return launch_mrhs_blas(P, B_XPAY, s); }
 
 // The same loop launched one kernel at a time (SQCG_LAUNCH_MODE=eager), the host reading the
 // state where the graph's conditional nodes would branch. Kernel-level profilers do not see
@@ -1566,7 +1622,7 @@ int run_eager(BatchPlan& P, cudaStream_t s) {
     SQCG_TRY(read());
     int act = 0;
     for (int j = 0; j < P.nblk; ++j) act |= h->blk_active[j];
-    if (!act || h->loop_count >= h->loop_limit) break;  // the WHILE condition of k_batch_ctl_loop
+    if (!act || h->loop_count >= h->loop_limit) break;  // the WHILE condition of loop_control
   }
   return SQCG_OK;
 }
@@ -1741,7 +1797,15 @@ int batched_solve(int nctx, sqcg_ctx* const* ctx, const int* nrhs, const double*
   if (any) {
     const char* mode = getenv("SQCG_LAUNCH_MODE");
     const bool eager = mode && strcmp(mode, "eager") == 0;
-    if (!eager && !P.exec) SQCG_TRY(capture_plan(P));
+    if (!eager && !P.exec) {
+      int rc = capture_plan(P);
+      if (rc == SQCG_ERR_CUDA && c0->pdl) {  // a driver without programmatic edges in a conditional body (see cg.cu)
+        cudaGetLastError();
+        c0->pdl = 0;
+        rc = capture_plan(P);
+      }
+      SQCG_TRY(rc);
+    }
     for (int k = 0; k < P.nlat; ++k)
       for (int rb = 0; rb < P.host[k].nrb; ++rb) {
         int a = 0;
@@ -1766,13 +1830,13 @@ int batched_solve(int nctx, sqcg_ctx* const* ctx, const int* nrhs, const double*
     // whatever the partial solutions still hold (nothing for an RHS whose last update converged)
     SQCG_TRY(launch_flush_x(P, 0, 0, s));
     SQCG_CUDA_TRY(cudaStreamSynchronize(s));
-    launches += h->loop_count * 8 + h->if_runs * 4 + 1;
+    launches += h->loop_count * 6 + h->if_runs * 4 + 1;
   }
   const double secs = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
   int worst = SQCG_OK;
   for (int j = 0; j < total; ++j) {
     const RhsScalars& r = h->r[j];
-    int st = r.active ? SQCG_ERR_NOT_CONVERGED : r.status;
+    int st = r.active ? SQCG_ERR_NOT_CONVERGED : r.status;  // active: the loop's hard bound ended it
     if (info) {
       info[j].iters = r.iter;
       info[j].reliable_updates = r.updates;

@@ -117,6 +117,7 @@ struct BatchState {
   double delta2;
   int loop_count, loop_limit;
   int if_runs;    // executions of the reliable-update IF body
+  unsigned arrived;  // blocks of the update's finisher that are done (zero between launches)
   int use_graph;  // the control kernels set the graph's conditional handles (0: eager launches)
   unsigned long long h_while, h_if;
   RhsScalars r[SQCG_MAX_BATCH_RHS];

@@ -249,3 +249,29 @@ def test_batched_update_arithmetic_and_initial_guess(sqcg, links_cache, arith):
                 assert abs(res - infos[n][j].true_rel_resid) <= 1e-12, (res, infos[n][j].true_rel_resid)
     for lat in lats:
         lat.close()
+
+
+@pytest.mark.parametrize("nrhs", [1, 3, 13])
+def test_batched_right_hand_sides_that_end_early(sqcg, links_cache, nrhs):
+    """Right-hand sides that start from their solution end at once while others of their pair, block and lattice go
+    on, on lattices whose sites fill no whole number of blocks: every solution on the oracle's FP64 true residual."""
+    specs = [((6, 6, 6, 10), 0.1), ((4, 6, 8, 10), 0.05)]
+    tol = 1e-9
+    lats, bs, xs, srcs, links = [], [], [], [], []
+    for n, (L, m) in enumerate(specs):
+        fat, lng = links_cache(L, 640 + n)
+        lat = sqcg.Lattice(L)
+        lat.load_links(fat, lng, recon12=n == 1)
+        s = [synth.gaussian_source(L, 7700 + 20 * n + j) for j in range(nrhs)]
+        b, x = make_batch(sqcg, lat, s)
+        for j in range(nrhs):
+            if (j + n) % 3 != 1:  # done from the start
+                lat.cg_solve(m, b[j], x[j], tol=tol / 100, max_iter=5000, mode=0)
+        lats.append(lat); bs.append(b); xs.append(x); srcs.append(s); links.append((fat, lng))
+    infos = sqcg.cg_solve_batched(lats, [m for _, m in specs], bs, xs, tol=tol, max_iter=5000)
+    for n, (L, m) in enumerate(specs):
+        for j in range(nrhs):
+            assert infos[n][j].status == 0
+            assert (infos[n][j].iters == 0) == ((j + n) % 3 != 1)
+            assert oracle.true_rel_residual(L, *links[n], 4 * m * m, srcs[n][j], lats[n].unpack(xs[n][j])) <= tol
+        lats[n].close()
