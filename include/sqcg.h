@@ -436,7 +436,9 @@ int sqcg_batched_tuning(const sqcg_ctx* ctx, int* W, int* T);
  * block T, shared-memory carveout in percent (-1 = the driver's default) and
  * warp_sites, the consecutive sites one warp covers: 32 (one RHS group per
  * warp), or 16 (two RHS groups per warp, whose link reads from shared memory
- * are then one broadcast access for both). Any output pointer may be NULL. */
+ * are then one broadcast access for both), or 4 for the kernel that splits the
+ * hops of 32 sites over four warps (WT = W right-hand sides in registers, no
+ * shared-memory links). Any output pointer may be NULL. */
 int sqcg_batched_tuning_ex(const sqcg_ctx* ctx, int* W, int* WT, int* T, int* carve, int* warp_sites);
 
 /* Pin the FP32 Dslash configuration of batched solves planned from now on in
@@ -444,7 +446,8 @@ int sqcg_batched_tuning_ex(const sqcg_ctx* ctx, int* W, int* WT, int* T, int* ca
  * keep theirs); W = 0 returns to autotuning. Requirements: W in {1, 2, 4, 8,
  * 12, 16}; WT in {1, 2, 4}, WT <= W and dividing W; T a multiple of 32 in [32, 128] with
  * T * W / WT <= 512; carve -1 or 0..100; warp_sites 32 (or 0, the same) or 16
- * with W / WT even. SQCG_ERR_INVALID_ARG otherwise (nothing changes).
+ * with W / WT even, or 4 with W = WT in {2, 4}, T = 32 and carve -1.
+ * SQCG_ERR_INVALID_ARG otherwise (nothing changes).
  * Thread-safe. */
 int sqcg_batched_pin_tuning(int W, int WT, int T, int carve, int warp_sites);
 

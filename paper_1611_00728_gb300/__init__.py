@@ -435,7 +435,8 @@ def batched_tuning(lattice) -> tuple[int, int]:
 
 def batched_tuning_ex(lattice) -> dict:
     """The full FP32 Dslash configuration of the last batched solve led by lattice: W, WT (RHS per thread),
-    T, carve (shared-memory carveout in percent, -1 = default) and warp_sites (32 or 16 sites per warp)."""
+    T, carve (shared-memory carveout in percent, -1 = default) and warp_sites (32 or 16 sites per warp; 4: the hops split
+    over four warps)."""
     v = [ctypes.c_int() for _ in range(5)]
     _check(library().sqcg_batched_tuning_ex(lattice._h, *[ctypes.byref(c) for c in v]), "sqcg_batched_tuning_ex")
     return dict(zip(("W", "WT", "T", "carve", "warp_sites"), (c.value for c in v)))

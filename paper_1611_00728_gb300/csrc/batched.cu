@@ -982,6 +982,153 @@ __global__ void __launch_bounds__(kMaxThreads) k_mrhs_dslash_smem(MArgs a) {
     rhs_block_partial_m<WT, SUB>(part, L, wbase, nw_tile, sb, ax, ay, a.partials, a.max_nsb);
 }
 
+// FP32 multi-RHS Dslash for few right-hand sides: a block is 32 sites, warp mu takes the four hops of direction mu and
+// applies each link to the RT right-hand sides of the block from registers, one load of the link per warp (the
+// kernel above stages 16 links a site in shared memory, which keeps few warps resident and pays off only where many
+// groups of right-hand sides read them). The partial sums meet in shared memory; warp w finishes the right-hand sides
+// 2 w and 2 w + 1. Bound by the latency of the gathers: 7 blocks per SM (72 registers; RT = 4 spills 56 bytes) beat 6,
+// 5 and 4 (136 / 156 / 155 / 177 us a pass at 32^4, 12-real, 4 right-hand sides). Against the best shape of the
+// kernel above at 32^4: 108 / 106 / 136 us for 1 / 2 / 4 right-hand sides (326 / 223 / 203), which takes a solve
+// from 131 / 99 / 102 ms to 56 / 57 / 79; for 8 from 164 to 141; for 16 a pass is 471 against 348. RT = 6 and 8 (355
+// and 404 us for 11, against 291) were no gain.
+template <int RT>
+__global__ void __launch_bounds__(128, 7) k_mrhs_dslash_hops(MArgs a) {
+  constexpr int NP = RT / 2;
+  static_assert(RT % 2 == 0 && NP <= 4, "a warp per pair of right-hand sides in the epilogue");
+  __shared__ float4 red[4][NP * 3][32];
+  const int tile = blockIdx.x;
+  const int k = find_lat(a.lats, a.nlat, tile, false);
+  const LatDev& L = a.lats[k];
+  const int local = tile - L.tile0;
+  const int rb = local % L.nrb, sb = local / L.nrb;
+  const int wbase = rb * RT;
+  const int np = min(NP, (L.nrhs - wbase + 1) / 2);  // pairs of this block (the last may be half filled)
+  pdl_launch_dependents();
+  if (a.gate == GATE_ITER && !a.st->blk_active[L.rb0 + rb]) {
+    pdl_wait();
+    return;
+  }
+  const Geom& g = L.g;
+  const int Vh = g.Vh, par = a.par, q = 1 - par;
+  const int lane = threadIdx.x, mu = threadIdx.y;
+  const int i = sb * 32 + lane;
+  const bool valid = i < Vh;
+  const int iv = valid ? i : 0;
+  const SiteXY c = site_of(g, iv, par);
+  const bool recon = L.recon != 0;
+  const int nl = recon ? 6 : 9;
+  float inv0 = L.inv_s0_f;
+  if (recon) {
+    const int ep = mu == 0 ? 0 : mu == 1 ? c.x : mu == 2 ? c.x + c.y : c.x + c.y + c.z;
+    if (ep & 1) inv0 = -inv0;
+  }
+  pdl_wait();
+  const float4* in = reinterpret_cast<const float4*>(a.in_vec == V_P ? L.p : L.tmp) + (size_t)(wbase >> 1) * 3 * Vh;
+  float2 acc[RT][3];
+#pragma unroll
+  for (int w = 0; w < RT; ++w)
+#pragma unroll
+    for (int cc = 0; cc < 3; ++cc) acc[w][cc] = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    const int lng = h >> 1, bwd = h & 1;
+    const int j = nbr_of(g, iv, c, mu, bwd ? (lng ? -3 : -1) : (lng ? 3 : 1));
+    float4 v[NP][3];
+#pragma unroll
+    for (int w = 0; w < NP; ++w)
+#pragma unroll
+      for (int cc = 0; cc < 3; ++cc)
+        if (w < np) v[w][cc] = __ldg(in + ((size_t)w * 3 + cc) * Vh + j);
+    float2 U[9];
+    const float2* base = (lng ? (bwd ? L.lng32[q] : L.lng32[par]) : (bwd ? L.fat32[q] : L.fat32[par])) +
+                         (size_t)mu * (lng ? nl : 9) * Vh + (bwd ? j : iv);
+#pragma unroll
+    for (int e = 0; e < 9; ++e)
+      if (e < 6 || !lng || !recon) U[e] = __ldg(base + (size_t)e * Vh);
+    if (lng && recon) {
+      float inv_s = inv0;
+      if (mu == 3 && g.apbc && (bwd ? (c.t < 3) : (c.t + 3 >= g.Lt))) inv_s = -inv_s;
+#pragma unroll
+      for (int jj = 0; jj < 3; ++jj) {
+        const int kk = (jj + 1) % 3, ll = (jj + 2) % 3;
+        const float2 ak = U[kk], al = U[ll], bk = U[3 + kk], bl = U[3 + ll];
+        const float re = ak.x * bl.x - ak.y * bl.y - (al.x * bk.x - al.y * bk.y);
+        const float im = ak.x * bl.y + ak.y * bl.x - (al.x * bk.y + al.y * bk.x);
+        U[6 + jj] = make_float2(re * inv_s, -im * inv_s);
+      }
+    }
+#pragma unroll
+    for (int w = 0; w < NP; ++w) {
+      if (w >= np) continue;
+#pragma unroll
+      for (int aa = 0; aa < 3; ++aa)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          const float2 u = bwd ? U[b * 3 + aa] : U[aa * 3 + b];
+          const float4 x = v[w][b];
+          float2& p0 = acc[2 * w][aa];
+          float2& p1 = acc[2 * w + 1][aa];
+          if (!bwd) {
+            p0.x = fmaf(-u.y, x.y, fmaf(u.x, x.x, p0.x));
+            p0.y = fmaf(u.y, x.x, fmaf(u.x, x.y, p0.y));
+            p1.x = fmaf(-u.y, x.w, fmaf(u.x, x.z, p1.x));
+            p1.y = fmaf(u.y, x.z, fmaf(u.x, x.w, p1.y));
+          } else {
+            p0.x = fmaf(-u.y, x.y, fmaf(-u.x, x.x, p0.x));
+            p0.y = fmaf(u.y, x.x, fmaf(-u.x, x.y, p0.y));
+            p1.x = fmaf(-u.y, x.w, fmaf(-u.x, x.z, p1.x));
+            p1.y = fmaf(u.y, x.z, fmaf(-u.x, x.w, p1.y));
+          }
+        }
+    }
+  }
+#pragma unroll
+  for (int w = 0; w < NP; ++w)
+#pragma unroll
+    for (int cc = 0; cc < 3; ++cc)
+      red[mu][w * 3 + cc][lane] = make_float4(acc[2 * w][cc].x, acc[2 * w][cc].y, acc[2 * w + 1][cc].x, acc[2 * w + 1][cc].y);
+  __syncthreads();
+  const int w = threadIdx.y;  // this warp's pair
+  if (w >= np) return;
+  const int w0 = wbase + 2 * w, nw = min(2, L.nrhs - w0);
+  double part[2] = {0.0, 0.0};
+  if (valid) {
+    float sig[2] = {0.f, 0.f}, dot[2] = {0.f, 0.f};
+    if (a.epi == M_NORMAL_DOT)
+      for (int u = 0; u < nw; ++u) sig[u] = (float)a.st->r[L.rhs0 + w0 + u].sigma;
+#pragma unroll
+    for (int cc = 0; cc < 3; ++cc) {
+      float4 d = red[0][w * 3 + cc][lane];
+#pragma unroll
+      for (int m = 1; m < 4; ++m) {
+        const float4 x = red[m][w * 3 + cc][lane];
+        d.x += x.x;
+        d.y += x.y;
+        d.z += x.z;
+        d.w += x.w;
+      }
+      float2 o[2] = {make_float2(d.x, d.y), make_float2(d.z, d.w)};
+      if (a.epi == M_PLAIN) {
+        pv_store<2>(L.tmp, w0, nw, cc, i, Vh, o);
+      } else {
+        float2 y[2];
+        pv_load<2>(L.p, w0, nw, cc, i, Vh, y);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          o[u] = make_float2(sig[u] * y[u].x - o[u].x, sig[u] * y[u].y - o[u].y);
+          dot[u] = fmaf(y[u].x, o[u].x, fmaf(y[u].y, o[u].y, dot[u]));
+        }
+        pv_store<2>(L.Ap, w0, nw, cc, i, Vh, o);
+      }
+    }
+    part[0] = (double)dot[0];
+    part[1] = (double)dot[1];
+  }
+  if (a.epi == M_PLAIN) return;
+  const double t = sum2<32>(part[0], part[1]);
+  if ((lane & 15) == 0 && (lane >> 4) < nw) a.partials[(size_t)(L.rhs0 + w0 + (lane >> 4)) * a.max_nsb + sb] = t;
+}
+
 // ---------------------------------------------------------------------------
 // multi-RHS BLAS: x += alpha p, r -= alpha Ap (|r|^2); p = r + beta p; |b|^2
 // ---------------------------------------------------------------------------
@@ -1162,8 +1309,9 @@ struct TuneChoice {
 };
 
 // shape rules of the FP32 Dslash: T a multiple of 32 up to kMaxTSmem, T * W / WT threads at most
-// kMaxThreads, SUB = 16 only with an even number of RHS groups
+// kMaxThreads, SUB = 16 only with an even number of RHS groups; SUB = 4 stands for k_mrhs_dslash_hops
 bool smem_shape_ok(int W, int WT, int T, int sub) {
+  if (sub == 4) return W == WT && (W == 2 || W == 4) && T == 32;  // k_mrhs_dslash_hops
   if (WT < 1 || W % WT) return false;
   const int G = W / WT;
   if (T < 32 || T % 32 || T > kMaxTSmem || T * G > kMaxThreads) return false;
@@ -1318,6 +1466,7 @@ SmemKernel smem_kernel(int idx) {
 // more of the SM's 256 KB to L1, which serves the neighbour gathers, at fewer resident blocks.
 // Set outside graph capture (by the tuner, before the plan's graph is captured).
 int set_carve(int WT, int sub, int carve) {
+  if (sub == 4) return SQCG_OK;
   std::lock_guard<std::recursive_mutex> lock(tune_mutex());
   static int cur[6] = {-2, -2, -2, -2, -2, -2};
   const int k = smem_index(WT, sub);
@@ -1330,6 +1479,10 @@ int set_carve(int WT, int sub, int carve) {
 }
 
 int launch_f32(const BatchPlan& P, int par, int in_vec, int epi, int gate, cudaStream_t s, bool pdl = false) {
+  if (P.sub == 4) {
+    SQCG_CUDA_TRY(launch_kernel(P.W == 2 ? k_mrhs_dslash_hops<2> : k_mrhs_dslash_hops<4>, dim3(P.ntiles), dim3(32, 4), 0, s, pdl && P.ctx[0]->pdl, margs(P, par, in_vec, epi, gate, 0)));
+    return SQCG_OK;
+  }
   const int G = P.W / P.WT, T = P.T;
   if (!smem_shape_ok(P.W, P.WT, T, P.sub)) return SQCG_ERR_INVALID_ARG;
   const size_t smem = (size_t)kHops * 9 * T * sizeof(float2);
@@ -1452,6 +1605,11 @@ int autotune(BatchPlan& P, cudaStream_t s) {
               ms / 5);
     if (ms < best) { best = ms; bestc = {W, WT, T, carve, sub}; }
   };
+  // 0: the hops split over warps (faster up to 8 right-hand sides at 32^4; the timing decides)
+  for (int W : {2, 4}) {
+    if (rc != SQCG_OK || W / 2 >= maxr + (W == 2)) break;
+    trial(W, W, 32, -1, 4);
+  }
   // 1: block shapes at the driver's default carveout
   for (int W : Ws) {
     if (W > 1 && W / 2 >= maxr) break;  // wider blocks than any lattice's RHS count only add idle lanes
@@ -1472,7 +1630,7 @@ int autotune(BatchPlan& P, cudaStream_t s) {
     if (rc != SQCG_OK) break;
   }
   // 2: the best W and WT again with smaller shared-memory carveouts (more L1 for the gathers)
-  if (rc == SQCG_OK) {
+  if (rc == SQCG_OK && bestc.sub != 4) {
     const int W = bestc.W, WT = bestc.WT, G = W / WT, sub = bestc.sub;
     const int carves[] = {25, 50, 75};
     for (int T : Ts) {
@@ -1894,7 +2052,7 @@ extern "C" int sqcg_batched_pin_tuning(int W, int WT, int T, int carve, int warp
   if ((W != 1 && W != 2 && W != 4 && W != 8 && W != 12 && W != 16) || (WT != 1 && WT != 2 && WT != 4) || WT > W)
     return SQCG_ERR_INVALID_ARG;
   if (!smem_shape_ok(W, WT, T, warp_sites)) return SQCG_ERR_INVALID_ARG;
-  if (carve < -1 || carve > 100) return SQCG_ERR_INVALID_ARG;
+  if (carve < -1 || carve > 100 || (warp_sites == 4 && carve != -1)) return SQCG_ERR_INVALID_ARG;
   tune_pin() = {W, WT, T, carve, warp_sites};
   return SQCG_OK;
 }

@@ -275,3 +275,38 @@ def test_batched_right_hand_sides_that_end_early(sqcg, links_cache, nrhs):
             assert (infos[n][j].iters == 0) == ((j + n) % 3 != 1)
             assert oracle.true_rel_residual(L, *links[n], 4 * m * m, srcs[n][j], lats[n].unpack(xs[n][j])) <= tol
         lats[n].close()
+
+
+@pytest.mark.parametrize("W", [2, 4])
+@pytest.mark.parametrize("nrhs", [1, 4, 7])
+@pytest.mark.parametrize("recon", [False, True])
+def test_batched_hops_split_over_warps(sqcg, links_cache, W, nrhs, recon):
+    """The Dslash that splits a site's hops over four warps: half-filled pairs and blocks of right-hand sides, a
+    last block of fewer than 32 sites, full and 12-real links with both temporal boundaries of the long hops. Every
+    solution on the oracle's FP64 true residual, in as many iterations (10% and 5) as the staged Dslash needs: an
+    FP32 operator that is off by more than its rounding sends the reliable updates back to work."""
+    specs = [((6, 6, 6, 10), 0.1), ((4, 6, 8, 8), 0.05)]
+    tol = 1e-9
+    iters = {}
+    for cfg in (dict(W=2, WT=2, T=32, carve=-1, warp_sites=32), dict(W=W, WT=W, T=32, carve=-1, warp_sites=4)):
+        sqcg.pin_batched_tuning(**cfg)
+        try:
+            lats, bs, xs, srcs, links = [], [], [], [], []
+            for n, (L, m) in enumerate(specs):
+                fat, lng = links_cache(L, 660 + n)
+                lat = sqcg.Lattice(L)
+                lat.load_links(fat, lng, recon12=recon)
+                s = [synth.gaussian_source(L, 7800 + 20 * n + j) for j in range(nrhs)]
+                b, x = make_batch(sqcg, lat, s)
+                lats.append(lat); bs.append(b); xs.append(x); srcs.append(s); links.append((fat, lng))
+            infos = sqcg.cg_solve_batched(lats, [m for _, m in specs], bs, xs, tol=tol, max_iter=5000)
+            assert sqcg.batched_tuning_ex(lats[0]) == cfg
+        finally:
+            sqcg.pin_batched_tuning(0)
+        iters[cfg["warp_sites"]] = [i.iters for r in infos for i in r]
+        for n, (L, m) in enumerate(specs):
+            for j in range(nrhs):
+                assert infos[n][j].status == 0
+                assert oracle.true_rel_residual(L, *links[n], 4 * m * m, srcs[n][j], lats[n].unpack(xs[n][j])) <= tol
+            lats[n].close()
+    assert all(a <= 1.1 * b + 5 for a, b in zip(iters[4], iters[32]))
