@@ -789,18 +789,29 @@ __device__ __forceinline__ int nbr_of(const Geom& g, int i, const SiteXY& c, int
 // FP32 multi-RHS Dslash with the links of the tile staged in shared memory.
 // A block covers T = blockDim.x sites and the tile's W = WT * G right-hand sides
 // (G = blockDim.y groups of WT). First the block copies the 16 links of each of
-// its sites (8 fat, 8 long; 12-real long links rebuilt here) from global memory
-// into shared memory, thread (x, y) staging site x for hops y, y + G, ...; then
-// every (site, group) thread applies them to its WT right-hand sides. Each link
+// its sites (8 fat, 8 long) from global memory into shared memory, thread (x, y)
+// staging site x for hops y, y + G, ..., by asynchronous copies that are all in
+// flight together, and beside them its first gather (loads through registers in
+// a loop over the hops took three memory latencies of the 16 us a block lives);
+// 12-real long links get their third rows there. Then every (site, group) thread
+// applies the links to its WT right-hand sides. Each link
 // is read from global memory once per RHS block, whatever W is.
 // SUB = 32: a warp holds 32 consecutive sites of one group. SUB = 16 (G even):
 // a warp holds 16 sites of two groups, so each link element a warp reads from
 // shared memory serves both groups in one access (a broadcast), which halves the
 // shared-memory wavefronts of the link reads; the neighbour gathers are the same.
+// Bound by the L1 pipe (72%: gathers and link reads) and by issue (67%) at 28 warps
+// per SM: at most 64 registers for WT <= 2, so that five blocks of six warps fit.
+// 8 right-hand sides on 16^4 and 24^4: 101 -> 97 us a pass, a solve 78.3 -> 75.1 ms.
+// Neighbour indices and 16-byte link rows in shared memory were slower (105 us).
 constexpr int kHops = 16;
 
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
 template <int WT, int SUB>
-__global__ void __launch_bounds__(kMaxThreads) k_mrhs_dslash_smem(MArgs a) {
+__global__ void __launch_bounds__(kMaxThreads, WT <= 2 ? 2 : 0) k_mrhs_dslash_smem(MArgs a) {
   extern __shared__ float2 sU[];  // [kHops][9][blockDim.x]
   const int tile = blockIdx.x;
   const int k = find_lat(a.lats, a.nlat, tile, false);
@@ -825,51 +836,25 @@ __global__ void __launch_bounds__(kMaxThreads) k_mrhs_dslash_smem(MArgs a) {
   const int par = a.par, q = 1 - par;
   // ---- stage the links: thread (x, y) stages site x for hops h = y, y + G, ... ----
   // hop h = 4 * mu + 2 * (long) + (backward)
+  const bool recon = L.recon != 0;
   {
     const int i = sb * TX + threadIdx.x;
-    const bool valid = i < Vh;
-    const SiteXY c = valid ? site_of(g, i, par) : SiteXY{0, 0, 0, 0, 0};
-    const bool recon = L.recon != 0;
-    const int nl = recon ? 6 : 9;
-    for (int h = threadIdx.y; h < kHops; h += G) {
-      const int mu = h >> 2, lng = (h >> 1) & 1, bwd = h & 1;
-      const int d = lng ? 3 : 1;
-      float2 u[9];
-      if (valid) {
+    if (i < Vh) {
+      const SiteXY c = site_of(g, i, par);
+      const int nl = recon ? 6 : 9;
+      for (int h = threadIdx.y; h < kHops; h += G) {
+        const int mu = h >> 2, lng = (h >> 1) & 1, bwd = h & 1;
+        const int d = lng ? 3 : 1;
         const float2* base = lng ? (bwd ? L.lng32[q] : L.lng32[par]) : (bwd ? L.fat32[q] : L.fat32[par]);
-        base += (size_t)mu * (lng ? nl : 9) * Vh;
-        const int idx = bwd ? nbr_of(g, i, c, mu, -d) : i;
         const int ne = lng ? nl : 9;
+        base += (size_t)mu * ne * Vh + (bwd ? nbr_of(g, i, c, mu, -d) : i);
+        float2* dst = sU + h * 9 * TX + threadIdx.x;
 #pragma unroll
         for (int e = 0; e < 9; ++e)
-          if (e < ne) u[e] = __ldg(base + (size_t)e * Vh + idx);
-        if (lng && recon) {  // third row = conj(row0 x row1) / s, s = s0 * eta_mu * boundary sign
-          int ep = 0;
-          if (mu == 1) ep = c.x;
-          if (mu == 2) ep = c.x + c.y;
-          if (mu == 3) ep = c.x + c.y + c.z;
-          float inv_s = (ep & 1) ? -L.inv_s0_f : L.inv_s0_f;
-          if (mu == 3 && g.apbc && (bwd ? (c.t < 3) : (c.t + 3 >= g.Lt))) inv_s = -inv_s;
-#pragma unroll
-          for (int jj = 0; jj < 3; ++jj) {
-            const int kk = (jj + 1) % 3, ll = (jj + 2) % 3;
-            const float2 ak = u[kk], al = u[ll], bk = u[3 + kk], bl = u[3 + ll];
-            const float re = ak.x * bl.x - ak.y * bl.y - (al.x * bk.x - al.y * bk.y);
-            const float im = ak.x * bl.y + ak.y * bl.x - (al.x * bk.y + al.y * bk.x);
-            u[6 + jj] = make_float2(re * inv_s, -im * inv_s);
-          }
-        }
-      } else {
-#pragma unroll
-        for (int e = 0; e < 9; ++e) u[e] = make_float2(0.f, 0.f);
+          if (e < ne) cp_async8(dst + e * TX, base + (size_t)e * Vh);
       }
-#pragma unroll
-      for (int e = 0; e < 9; ++e) sU[(h * 9 + e) * TX + threadIdx.x] = u[e];
     }
   }
-  pdl_wait();
-  __syncthreads();
-  // ---- apply to this thread's right-hand sides: thread (site ax, group ay) ----
   int ax = threadIdx.x, ay = threadIdx.y;
   if constexpr (SUB == 16) {
     const int tid = threadIdx.x + TX * threadIdx.y;
@@ -879,6 +864,7 @@ __global__ void __launch_bounds__(kMaxThreads) k_mrhs_dslash_smem(MArgs a) {
   }
   const int w0 = wbase + ay * WT;
   int nw = max(0, min(WT, L.nrhs - w0));
+  pdl_wait();
   if (a.gate == GATE_ITER) {  // a group whose right-hand sides have all finished has nothing to do
     bool any = false;
 #pragma unroll
@@ -886,33 +872,59 @@ __global__ void __launch_bounds__(kMaxThreads) k_mrhs_dslash_smem(MArgs a) {
     if (!any) nw = 0;
   }
   const int i = sb * TX + ax;
-  const bool valid = i < Vh;
+  const bool valid = i < Vh, work = valid && nw > 0;
   double part[WT];
 #pragma unroll
   for (int w = 0; w < WT; ++w) part[w] = 0.0;
   const float2* in = (a.in_vec == V_P ? (const float2*)L.p : (const float2*)L.tmp);
-  if (valid && nw > 0) {
-    const SiteXY c = site_of(g, i, par);
+  const SiteXY c = site_of(g, valid ? i : 0, par);
+  // one-hop software pipeline: the next hop's neighbour vectors are in flight while
+  // this hop's products run (the gathers, not the FMAs, set the pace of this kernel)
+  float2 vin[WT][3], vnx[WT][3];
+  auto gather = [&](int h, float2 (&v)[WT][3]) {
+    const int mu = h >> 2, lng = (h >> 1) & 1, bwd = h & 1;
+    const int j = nbr_of(g, i, c, mu, bwd ? (lng ? -3 : -1) : (lng ? 3 : 1));
+#pragma unroll
+    for (int cc = 0; cc < 3; ++cc) {
+      float2 t[WT];
+      pv_load<WT>(in, w0, nw, cc, j, Vh, t);  // one 16-byte gather per RHS pair
+#pragma unroll
+      for (int w = 0; w < WT; ++w) v[w][cc] = t[w];
+    }
+  };
+  if (work) gather(0, vin);
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  if (recon) {  // third rows: conj(row0 x row1) / s, s = s0 * eta_mu * boundary sign, of the thread's own links
+    const int i = sb * TX + threadIdx.x;
+    const SiteXY c = site_of(g, i < Vh ? i : 0, par);
+    for (int h = threadIdx.y; h < kHops; h += G) {
+      const int mu = h >> 2, bwd = h & 1;
+      if (!(h & 2)) continue;
+      float2* u = sU + h * 9 * TX + threadIdx.x;
+      int ep = 0;
+      if (mu == 1) ep = c.x;
+      if (mu == 2) ep = c.x + c.y;
+      if (mu == 3) ep = c.x + c.y + c.z;
+      float inv_s = (ep & 1) ? -L.inv_s0_f : L.inv_s0_f;
+      if (mu == 3 && g.apbc && (bwd ? (c.t < 3) : (c.t + 3 >= g.Lt))) inv_s = -inv_s;
+#pragma unroll
+      for (int jj = 0; jj < 3; ++jj) {
+        const int kk = (jj + 1) % 3, ll = (jj + 2) % 3;
+        const float2 ak = u[kk * TX], al = u[ll * TX], bk = u[(3 + kk) * TX], bl = u[(3 + ll) * TX];
+        const float re = ak.x * bl.x - ak.y * bl.y - (al.x * bk.x - al.y * bk.y);
+        const float im = ak.x * bl.y + ak.y * bl.x - (al.x * bk.y + al.y * bk.x);
+        u[(6 + jj) * TX] = make_float2(re * inv_s, -im * inv_s);
+      }
+    }
+  }
+  __syncthreads();
+  // ---- apply to this thread's right-hand sides: thread (site ax, group ay) ----
+  if (work) {
     float2 acc[WT][3];
 #pragma unroll
     for (int w = 0; w < WT; ++w)
 #pragma unroll
       for (int cc = 0; cc < 3; ++cc) acc[w][cc] = make_float2(0.f, 0.f);
-    // one-hop software pipeline: the next hop's neighbour vectors are in flight while
-    // this hop's products run (the gathers, not the FMAs, set the pace of this kernel)
-    float2 vin[WT][3], vnx[WT][3];
-    auto gather = [&](int h, float2 (&v)[WT][3]) {
-      const int mu = h >> 2, lng = (h >> 1) & 1, bwd = h & 1;
-      const int j = nbr_of(g, i, c, mu, bwd ? (lng ? -3 : -1) : (lng ? 3 : 1));
-#pragma unroll
-      for (int cc = 0; cc < 3; ++cc) {
-        float2 t[WT];
-        pv_load<WT>(in, w0, nw, cc, j, Vh, t);  // one 16-byte gather per RHS pair
-#pragma unroll
-        for (int w = 0; w < WT; ++w) v[w][cc] = t[w];
-      }
-    };
-    gather(0, vin);
 #pragma unroll
     for (int h = 0; h < kHops; ++h) {
       if (h + 1 < kHops) gather(h + 1, vnx);
@@ -1002,7 +1014,7 @@ __global__ void __launch_bounds__(128, 7) k_mrhs_dslash_hops(MArgs a) {
   const int local = tile - L.tile0;
   const int rb = local % L.nrb, sb = local / L.nrb;
   const int wbase = rb * RT;
-  const int np = min(NP, (L.nrhs - wbase + 1) / 2);  // pairs of this block (the last may be half filled)
+  int np = min(NP, (L.nrhs - wbase + 1) / 2);  // pairs of this block (the last may be half filled)
   pdl_launch_dependents();
   if (a.gate == GATE_ITER && !a.st->blk_active[L.rb0 + rb]) {
     pdl_wait();
@@ -1023,6 +1035,9 @@ __global__ void __launch_bounds__(128, 7) k_mrhs_dslash_hops(MArgs a) {
     if (ep & 1) inv0 = -inv0;
   }
   pdl_wait();
+  if (a.gate == GATE_ITER)  // trailing pairs that have finished are left out
+    while (np > 1 && !a.st->r[L.rhs0 + wbase + 2 * np - 2].active &&
+           !(wbase + 2 * np - 1 < L.nrhs && a.st->r[L.rhs0 + wbase + 2 * np - 1].active)) --np;
   const float4* in = reinterpret_cast<const float4*>(a.in_vec == V_P ? L.p : L.tmp) + (size_t)(wbase >> 1) * 3 * Vh;
   float2 acc[RT][3];
 #pragma unroll
