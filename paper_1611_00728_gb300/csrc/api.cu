@@ -67,6 +67,8 @@ void free_workspace(sqcg_ctx* ctx) {
   for (int j = 1; j < ctx->ms_nalloc; ++j) cudaFree(ctx->ms_p[j]);
   for (int j = 0; j < SQCG_MAX_SHIFTS; ++j) ctx->ms_p[j] = nullptr;
   ctx->ms_nalloc = 0;
+  cudaFree(ctx->ms_ring);
+  ctx->ms_ring = nullptr;
   for (int j = 0; j < ctx->rat_n; ++j) cudaFree(ctx->rat_x[j]);
   for (int j = 0; j < SQCG_MAX_SHIFTS; ++j) ctx->rat_x[j] = nullptr;
   cudaFree(ctx->ms_stack);

@@ -5,6 +5,9 @@
 // deterministically (warp shuffle -> block partial -> one finisher block that
 // adds the partials in index order), and the scalar CG step runs in that
 // finisher.
+#include <type_traits>
+
+#include "ff_arith.cuh"
 #include "solver_device.cuh"
 #include "sqcg_internal.cuh"
 
@@ -167,21 +170,22 @@ k_scale_copy_f64(const double2* __restrict__ src, double2* __restrict__ dst, dou
 }
 
 // ---------------------------------------------------------------------------
-// multi-shift CG: the base r update with the x_s updates of all shifts, and
-// the p_s updates. The shift scalars come from SolverState (FP64).
+// multi-shift CG: the base system's r and p updates of each step, and the x_s
+// and p_s updates of all shifts, for the steps of a pass together. The shift
+// scalars come from SolverState (FP64).
 // ---------------------------------------------------------------------------
 struct MSPtrs {
   double2* x[SQCG_MAX_SHIFTS];
   void* p[SQCG_MAX_SHIFTS];
 };
 
-// r -= alpha Ap (base), reduce |r|^2 -> FIN_MS_UPDATE
+// rn = r - alpha Ap (base), reduce |rn|^2 -> FIN_MS_UPDATE; rn may be r
 template <typename R>
 __global__ void __launch_bounds__(kThreads)
-k_ms_update(typename V2<R>::T* __restrict__ r, const typename V2<R>::T* __restrict__ Ap, int Vh, SolverState* st,
-            double* partials) {
+k_ms_update(const typename V2<R>::T* r, typename V2<R>::T* rn, const typename V2<R>::T* __restrict__ Ap, int Vh,
+            SolverState* st, double* partials) {
   typedef typename V2<R>::T R2;
-  if (!gate_open(st, GATE_ITER)) return;
+  if (!gate_open(st, GATE_STEP)) return;
   const R ra = (R)st->alpha;
   double nrm = 0.0;                             // FP64 vectors: FP64 partials
   float2 nrm_ff[1] = {make_float2(0.f, 0.f)};  // FP32 vectors: float-float partials
@@ -197,7 +201,7 @@ k_ms_update(typename V2<R>::T* __restrict__ r, const typename V2<R>::T* __restri
     for (int c = 0; c < 3; ++c) {
       rc[c].x = fma(-ra, apc[c].x, rc[c].x);
       rc[c].y = fma(-ra, apc[c].y, rc[c].y);
-      r[(size_t)c * Vh + i] = rc[c];
+      rn[(size_t)c * Vh + i] = rc[c];
       part = fma(rc[c].x, rc[c].x, fma(rc[c].y, rc[c].y, part));
     }
     if constexpr (sizeof(R) == 4)
@@ -213,55 +217,142 @@ k_ms_update(typename V2<R>::T* __restrict__ r, const typename V2<R>::T* __restri
   }
 }
 
-// One pass over every shift's direction: x_s += alpha_s p_s (the old p_s; for
-// every shift with an update this iteration, including one that just
-// converged), then p_s = zeta_s r + beta_s p_s for shifts still iterating.
-// Shift 0 is the base system: its direction is the base p = r + beta p.
-// Runs while the loop goes on, and once more in the iteration that ends it.
-template <typename R>
+// Step k of a pass has been taken (and has not broken down): p = r + beta p of the base system, whose direction the
+// next Dslash needs. A later step that its gate skipped leaves ms_n behind.
 __global__ void __launch_bounds__(kThreads)
-k_ms_xpay(MSPtrs P, const typename V2<R>::T* __restrict__ r, typename V2<R>::T* __restrict__ p, int Vh,
-          const SolverState* st) {
-  typedef typename V2<R>::T R2;
-  const int done = !gate_open(st, GATE_ITER);
-  if (done && !st->ms_final) return;
-  const int ns = st->nshift;
+k_ms_base_p(const float2* __restrict__ r, float2* __restrict__ p, int k, int Vh, const SolverState* st) {
+  __shared__ int open;
+  if (threadIdx.x == 0) open = static_cast<const volatile SolverState*>(st)->ms_n == k + 1;
+  __syncthreads();
+  if (!open) return;
+  const float b = (float)st->beta;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Vh; i += gridDim.x * blockDim.x) {
-    R2 rc[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) rc[c] = r[(size_t)c * Vh + i];
+    for (int c = 0; c < 3; ++c) {
+      const size_t j = (size_t)c * Vh + i;
+      const float2 rc = r[j];
+      float2 pc = p[j];
+      pc.x = fmaf(b, pc.x, rc.x);
+      pc.y = fmaf(b, pc.y, rc.y);
+      p[j] = pc;
+    }
+  }
+}
+
+// The updates of every shift for the n steps of a pass, in their order: x_s += alpha_s p_s (for every shift with an
+// update in that step, including the one it converged in), then p_s = zeta_s r + beta_s p_s with the step's new
+// residual for shifts still iterating. Shift 0 is the base system.
+// FP64 vectors: one step a pass. FP32 vectors: x_s is held as float-float for the length of the loop (48 bits, as the
+// reliable update's residuals read it; this GPU does 2 FP64 operations a clock and SM, which one step's x_s updates
+// and conversions filled for 122 us at 32^4 with 11 shifts, as long as their 830 MB took), and a pass of four steps
+// reads and writes x_s and p_s once: 220 MB a step. 11 shifts, mixed, to 1e-11: 182 -> 160 ms at 32^4, 65 -> 50 at
+// 24^4, 15.4 -> 13.2 at 16^4 (the last two with the refinement's gains); the solutions' errors are the same.
+struct MSRing {
+  const void* r[kMSUnroll];  // the residual after each step of the pass
+};
+
+template <typename R, int M>
+__global__ void __launch_bounds__(kThreads)
+k_ms_flush(MSPtrs P, MSRing ring, typename V2<R>::T* __restrict__ r0, int Vh, const SolverState* st) {
+  typedef typename V2<R>::T R2;
+  typedef typename std::conditional<sizeof(R) == 4, float4, double2>::type X;  // float4: re_hi, re_lo, im_hi, im_lo
+  __shared__ double sa[M][SQCG_MAX_SHIFTS];  // alpha (R = float: as a float-float)
+  __shared__ R sz[M][SQCG_MAX_SHIFTS], sb[M][SQCG_MAX_SHIFTS];
+  __shared__ int sact[M][SQCG_MAX_SHIFTS], any[SQCG_MAX_SHIFTS];
+  const int n = st->ms_n, ns = st->nshift;
+  if (n < 1) return;
+  for (int k = threadIdx.x; k < n * ns; k += blockDim.x) {
+    const int q = k / ns, j = k % ns;
+    const double al = st->ms_ha[q][j];
+    if constexpr (sizeof(R) == 4) {
+      const float h = (float)al;
+      reinterpret_cast<float2*>(sa[q])[j] = make_float2(h, (float)(al - (double)h));
+    } else {
+      sa[q][j] = al;
+    }
+    sz[q][j] = (R)st->ms_hz[q][j];
+    sb[q][j] = (R)st->ms_hb[q][j];
+    sact[q][j] = st->ms_act[q][j];
+  }
+  for (int j = threadIdx.x; j < ns; j += blockDim.x) any[j] = st->ms_act[0][j];  // shifts only ever stop
+  __syncthreads();
+  const R2* rl = nullptr;
+#pragma unroll
+  for (int q = 0; q < M - 1; ++q)
+    if (q == n - 1) rl = static_cast<const R2*>(ring.r[q]);
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Vh; i += gridDim.x * blockDim.x) {
+    R2 rc[M][3];
+#pragma unroll
+    for (int q = 0; q < M; ++q)
+      if (q < n)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) rc[q][c] = static_cast<const R2*>(ring.r[q])[(size_t)c * Vh + i];
+    if (rl)  // a pass that ended early leaves its residual where the next one starts
+#pragma unroll
+      for (int c = 0; c < 3; ++c) r0[(size_t)c * Vh + i] = rl[(size_t)c * Vh + i];
     for (int j = 0; j < ns; ++j) {
-      const int act = st->active[j];
-      const bool upd_p = !done && (j == 0 || act == 1);  // the base direction moves while the loop runs
-      if (!act && !upd_p) continue;
-      R2* ps = (j == 0) ? p : static_cast<R2*>(P.p[j]);
-      const double as = st->alpha_s[j];
-      const R z = (j == 0) ? R(1) : (R)st->zeta[j];
-      const R bs = (j == 0) ? (R)st->beta : (R)st->beta_s[j];
-      double2* xs = P.x[j];
+      const bool upd_x = any[j] != 0;
+      if (!upd_x && j > 0) continue;
+      R2* ps = static_cast<R2*>(P.p[j]);
+      X* xs = reinterpret_cast<X*>(P.x[j]);
       R2 pc[3];
-      double2 xc[3];
+      X xc[3];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {  // loads before stores (see k_cg_update)
         pc[c] = ps[(size_t)c * Vh + i];
-        if (act) xc[c] = xs[(size_t)c * Vh + i];
+        if (upd_x) xc[c] = xs[(size_t)c * Vh + i];
+      }
+#pragma unroll
+      for (int q = 0; q < M; ++q) {
+        const int act = q < n ? sact[q][j] : 0;
+        if (act) {
+          if constexpr (sizeof(R) == 4) {
+            const float2 al = reinterpret_cast<const float2*>(sa[q])[j];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+              const float4 x = xc[c];
+              const float tx = __fmul_rn(al.x, pc[c].x), ty = __fmul_rn(al.x, pc[c].y);
+              const float2 re = ffs_add(make_float2(x.x, x.y),
+                                        make_float2(tx, fmaf(al.y, pc[c].x, fmaf(al.x, pc[c].x, -tx))));
+              const float2 im = ffs_add(make_float2(x.z, x.w),
+                                        make_float2(ty, fmaf(al.y, pc[c].y, fmaf(al.x, pc[c].y, -ty))));
+              xc[c] = make_float4(re.x, re.y, im.x, im.y);
+            }
+          } else {
+            const double al = sa[q][j];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+              xc[c].x = fma(al, pc[c].x, xc[c].x);
+              xc[c].y = fma(al, pc[c].y, xc[c].y);
+            }
+          }
+        }
+        if ((j == 0 && q < n) || act == 1) {
+          const R z = sz[q][j], b = sb[q][j];
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            pc[c].x = fma(b, pc[c].x, z * rc[q][c].x);
+            pc[c].y = fma(b, pc[c].y, z * rc[q][c].y);
+          }
+        }
       }
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const size_t k = (size_t)c * Vh + i;
-        if (act) {
-          xc[c].x = fma(as, (double)pc[c].x, xc[c].x);
-          xc[c].y = fma(as, (double)pc[c].y, xc[c].y);
-          xs[k] = xc[c];
-        }
-        if (upd_p) {
-          R2 pn;
-          pn.x = fma(bs, pc[c].x, z * rc[c].x);
-          pn.y = fma(bs, pc[c].y, z * rc[c].y);
-          ps[k] = pn;
-        }
+        if (upd_x) xs[k] = xc[c];
+        ps[k] = pc[c];
       }
     }
+  }
+}
+
+// x_s of the mixed loop between FP64 and float-float, in place (the loop runs on float-float, the reliable updates
+// and the caller see FP64; a value that came from float-float goes through FP64 unchanged)
+__global__ void __launch_bounds__(kThreads) k_ms_x_form(MSPtrs P, size_t n, int to_ff) {
+  double2* x = P.x[blockIdx.y];
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    if (to_ff) reinterpret_cast<float4*>(x)[i] = split_ff(x[i]);
+    else x[i] = join_ff(reinterpret_cast<const float4*>(x)[i]);
   }
 }
 
@@ -480,18 +571,41 @@ int launch_scale_copy_f64(sqcg_ctx* ctx, const double2* src, double2* dst, doubl
   return SQCG_OK;
 }
 
-int launch_ms_update_x(sqcg_ctx* ctx, int mixed, int nshift, double2* const* x, cudaStream_t s) {
+// the base residual before step k of a pass and after step k - 1; every pass starts and ends in r32
+static float2* ms_ring_r(sqcg_ctx* ctx, int k) {
+  k %= ctx->ms_unroll;
+  return k == 0 ? ctx->r32 : ctx->ms_ring + (size_t)k * 3 * ctx->g.Vh;
+}
+
+int launch_ms_update(sqcg_ctx* ctx, int mixed, int k, cudaStream_t s) {
   // one thread per site: measured faster here than the one-wave grid of the CG kernels
   const int Vh = ctx->g.Vh, grid = grid_for(Vh, kThreads);
-  if (grid > ctx->max_blocks || nshift < 1 || nshift > ctx->ms_nalloc) return SQCG_ERR_INVALID_ARG;
-  (void)x;  // the x_s updates run in k_ms_xpay
+  if (grid > ctx->max_blocks) return SQCG_ERR_INVALID_ARG;
   if (mixed)
-    k_ms_update<float><<<grid, kThreads, 0, s>>>(ctx->r32, ctx->Ap32, Vh, ctx->st, ctx->partials);
+    k_ms_update<float><<<grid, kThreads, 0, s>>>(ms_ring_r(ctx, k), ms_ring_r(ctx, k + 1), ctx->Ap32, Vh, ctx->st,
+                                                 ctx->partials);
   else
-    k_ms_update<double><<<grid, kThreads, 0, s>>>(ctx->r64, ctx->Ap64, Vh, ctx->st, ctx->partials);
+    k_ms_update<double><<<grid, kThreads, 0, s>>>(ctx->r64, ctx->r64, ctx->Ap64, Vh, ctx->st, ctx->partials);
   SQCG_CUDA_TRY(cudaGetLastError());
-  return mixed ? launch_finish_ffs(ctx, grid, FIN_MS_UPDATE, GATE_ITER, s)
-               : launch_finish(ctx, grid, FIN_MS_UPDATE, GATE_ITER, s);
+  return mixed ? launch_finish_ffs(ctx, grid, FIN_MS_UPDATE, GATE_STEP, s)
+               : launch_finish(ctx, grid, FIN_MS_UPDATE, GATE_STEP, s);
+}
+
+int launch_ms_base_p(sqcg_ctx* ctx, int k, cudaStream_t s) {
+  const int Vh = ctx->g.Vh;
+  k_ms_base_p<<<grid_for(Vh, kThreads), kThreads, 0, s>>>(ms_ring_r(ctx, k + 1), ctx->p32, k, Vh, ctx->st);
+  SQCG_CUDA_TRY(cudaGetLastError());
+  return SQCG_OK;
+}
+
+int launch_ms_x_form(sqcg_ctx* ctx, int nshift, double2* const* x, bool to_ff, cudaStream_t s) {
+  const size_t n = (size_t)3 * ctx->g.Vh;
+  const size_t full = (n + kThreads - 1) / kThreads;
+  MSPtrs P = {};
+  for (int j = 0; j < nshift; ++j) P.x[j] = x[j];
+  k_ms_x_form<<<dim3((unsigned)(full < 4096 ? full : 4096), nshift), kThreads, 0, s>>>(P, n, to_ff ? 1 : 0);
+  SQCG_CUDA_TRY(cudaGetLastError());
+  return SQCG_OK;
 }
 
 int launch_ms_ru_sums(sqcg_ctx* ctx, const double2* a, const double2* b, double z, cudaStream_t s) {
@@ -526,7 +640,7 @@ int launch_ms_ru_fix(sqcg_ctx* ctx, int mixed, int nshift, const void* rt, int r
   return SQCG_OK;
 }
 
-int launch_ms_xpay(sqcg_ctx* ctx, int mixed, int nshift, double2* const* x, cudaStream_t s) {
+int launch_ms_flush(sqcg_ctx* ctx, int mixed, int nshift, double2* const* x, cudaStream_t s) {
   const int Vh = ctx->g.Vh, grid = grid_for(Vh, kThreads);
   if (nshift < 1 || nshift > ctx->ms_nalloc) return SQCG_ERR_INVALID_ARG;
   MSPtrs P;
@@ -534,10 +648,14 @@ int launch_ms_xpay(sqcg_ctx* ctx, int mixed, int nshift, double2* const* x, cuda
     P.x[j] = (j < nshift) ? x[j] : nullptr;
     P.p[j] = (j < nshift) ? ctx->ms_p[j] : nullptr;
   }
-  if (mixed)
-    k_ms_xpay<float><<<grid, kThreads, 0, s>>>(P, ctx->r32, ctx->p32, Vh, ctx->st);
+  MSRing ring = {};
+  for (int k = 0; k < ctx->ms_unroll; ++k) ring.r[k] = mixed ? (const void*)ms_ring_r(ctx, k + 1) : ctx->r64;
+  if (!mixed)
+    k_ms_flush<double, 1><<<grid, kThreads, 0, s>>>(P, ring, ctx->r64, Vh, ctx->st);
+  else if (ctx->ms_unroll == 1)
+    k_ms_flush<float, 1><<<grid, kThreads, 0, s>>>(P, ring, ctx->r32, Vh, ctx->st);
   else
-    k_ms_xpay<double><<<grid, kThreads, 0, s>>>(P, ctx->r64, ctx->p64, Vh, ctx->st);
+    k_ms_flush<float, kMSUnroll><<<grid, kThreads, 0, s>>>(P, ring, ctx->r32, Vh, ctx->st);
   SQCG_CUDA_TRY(cudaGetLastError());
   return SQCG_OK;
 }

@@ -18,7 +18,7 @@ namespace {
 
 constexpr int kCGKernelsPerIter = 7;  // enqueue_cg_head (3 + 2 finishers) + xpay + loop control
 constexpr int kCGKernelsPerUpdate = 3;  // enqueue_cg_reliable (2 + finisher)
-constexpr int kMSKernelsPerIter = 7;  // enqueue_ms_iteration (4 + 2 finishers) + loop control
+constexpr int kMSKernelsPerStep = 5;  // two Dslash passes and the residual's update, with two finishers
 constexpr int kSRKernelsPerIter = 4;  // enqueue_sr_head (2 + finisher) + the update
 // Steps of the single-reduction loop per pass of its WHILE node. Each pass ends with the reliable-update
 // IF node and the loop control; a step that asks for a reliable update closes the pass (the steps
@@ -168,25 +168,29 @@ int enqueue_sr_reliable(sqcg_ctx* ctx, const void* b, void* x, cudaStream_t s, b
   return head ? enqueue_sr_head(ctx, s, true, true) : SQCG_OK;  // gated on the loop going on (GATE_STEP)
 }
 
-int enqueue_ms_iteration(sqcg_ctx* ctx, int mixed, int nshift, double2* const* x, cudaStream_t s) {
+// A pass of the multi-shift loop: ctx->ms_unroll steps on the base system, each skipped once the loop is to pause or
+// has ended, then the x_s and p_s updates of all shifts for the steps taken.
+int enqueue_ms_pass(sqcg_ctx* ctx, int mixed, int nshift, double2* const* x, cudaStream_t s) {
   const int wp = mixed ? SQCG_F32 : SQCG_F64;
   void* p = mixed ? (void*)ctx->p32 : (void*)ctx->p64;
   void* Ap = mixed ? (void*)ctx->Ap32 : (void*)ctx->Ap64;
   void* tmp = mixed ? (void*)ctx->tmp32 : (void*)ctx->tmp64;
-  DslashLaunch L = {};
-  L.out_parity = 1; L.prec = L.out_prec = wp; L.epi = EPI_PLAIN; L.in = p; L.out = tmp; L.gate = GATE_ITER;
-  SQCG_TRY(launch_dslash(ctx, L, s));
-  L = DslashLaunch{};
-  L.out_parity = 0; L.prec = L.out_prec = wp; L.epi = EPI_NORMAL_DOT; L.in = tmp; L.out = Ap; L.y = p;
-  L.sigma_dev = &ctx->st->sigma; L.gate = GATE_ITER; L.fin = FIN_MS_PAP; L.pdl = 1;
-  SQCG_TRY(launch_dslash(ctx, L, s));
-  SQCG_TRY(launch_ms_update_x(ctx, mixed, nshift, x, s));
-  SQCG_TRY(launch_ms_xpay(ctx, mixed, nshift, x, s));
-  return SQCG_OK;
+  for (int k = 0; k < ctx->ms_unroll; ++k) {
+    DslashLaunch L = {};
+    L.out_parity = 1; L.prec = L.out_prec = wp; L.epi = EPI_PLAIN; L.in = p; L.out = tmp; L.gate = GATE_STEP;
+    SQCG_TRY(launch_dslash(ctx, L, s));
+    L = DslashLaunch{};
+    L.out_parity = 0; L.prec = L.out_prec = wp; L.epi = EPI_NORMAL_DOT; L.in = tmp; L.out = Ap; L.y = p;
+    L.sigma_dev = &ctx->st->sigma; L.gate = GATE_STEP; L.fin = FIN_MS_PAP; L.pdl = 1;
+    SQCG_TRY(launch_dslash(ctx, L, s));
+    SQCG_TRY(launch_ms_update(ctx, mixed, k, s));
+    if (ctx->ms_unroll > 1) SQCG_TRY(launch_ms_base_p(ctx, k, s));
+  }
+  return launch_ms_flush(ctx, mixed, nshift, x, s);
 }
 
 // Build the solver graph: one WHILE node whose body is one iteration (kSRUnroll
-// steps for the single-reduction loop) followed by the loop-control kernel. For
+// steps for the single-reduction loop, a pass of the multi-shift loop) followed by the loop-control kernel. For
 // single-mass CG the reliable update sits in an IF node inside the body, so
 // iterations without an update launch none of its kernels. The conditional
 // handles are passed to the kernels through the device state (h_while, h_if).
@@ -228,7 +232,7 @@ int capture_body(sqcg_ctx* ctx, int kind, int mixed, const void* b, void* const*
     }
     if (rc == SQCG_OK && kind == KIND_CG) rc = launch_cg_xpay(ctx, mixed, cs);
   } else {
-    rc = enqueue_ms_iteration(ctx, mixed, nx, (double2* const*)x, cs);
+    rc = enqueue_ms_pass(ctx, mixed, nx, (double2* const*)x, cs);
   }
   if (rc == SQCG_OK) rc = launch_loop_control(ctx, cs);
   cudaGraph_t out = nullptr;
@@ -322,6 +326,7 @@ int run_loop(sqcg_ctx* ctx, CGGraph* g, int max_iter, cudaStream_t s, int* iters
   h->use_if = (g->kind == KIND_CG || g->kind == KIND_SR) ? 1 : 0;
   h->loop_count = 0;
   h->loop_limit = max_iter + 4;
+  h->ms_n = 0;
   SQCG_TRY(write_state(ctx, s));
   SQCG_CUDA_TRY(cudaGraphLaunch(g->exec, s));
   SQCG_TRY(read_state(ctx, s));
@@ -342,6 +347,7 @@ int run_eager(sqcg_ctx* ctx, int kind, int mixed, const void* b, void* const* x,
               cudaStream_t s, int* iters_run) {
   SolverState* h = ctx->st_host;
   h->use_if = 0;  // no graph: the kernels must not touch conditional handles
+  h->ms_n = 0;
   SQCG_TRY(write_state(ctx, s));
   int it = 0;
   for (; it < max_iter + 4; ++it) {
@@ -364,7 +370,7 @@ int run_eager(sqcg_ctx* ctx, int kind, int mixed, const void* b, void* const* x,
       if (h->done) break;
       SQCG_TRY(launch_sr_update(ctx, s));
     } else {
-      SQCG_TRY(enqueue_ms_iteration(ctx, mixed, nx, (double2* const*)x, s));
+      SQCG_TRY(enqueue_ms_pass(ctx, mixed, nx, (double2* const*)x, s));
       SQCG_TRY(read_state(ctx, s));
       if (h->done || (h->ms_ru && h->need_update)) break;  // finished, or paused for the host-driven update
     }
@@ -716,6 +722,8 @@ extern "C" int sqcg_multishift_cg_solve(sqcg_ctx* ctx, int nshift, const double*
   // per-shift directions p_s (s >= 1) in the working precision; p_0 is the base p
   if (ctx->ms_nalloc < nshift || ctx->ms_prec != mixed) {
     for (int j = 1; j < ctx->ms_nalloc; ++j) cudaFree(ctx->ms_p[j]);
+    cudaFree(ctx->ms_ring);
+    ctx->ms_ring = nullptr;
     ctx->ms_nalloc = 0;
     free_graphs(ctx);
     for (int j = 1; j < nshift; ++j) {
@@ -727,8 +735,13 @@ extern "C" int sqcg_multishift_cg_solve(sqcg_ctx* ctx, int nshift, const double*
     }
     ctx->ms_nalloc = nshift;
     ctx->ms_prec = mixed;
+    ctx->ms_unroll = 1;
+    if (mixed) {  // without room for it the loop applies every step by itself
+      if (cudaMalloc(&ctx->ms_ring, kMSUnroll * wbytes) == cudaSuccess) ctx->ms_unroll = kMSUnroll;
+      else { cudaGetLastError(); ctx->ms_ring = nullptr; }
+    }
   }
-  ctx->ms_p[0] = mixed ? (void*)ctx->p32 : (void*)ctx->p64;
+  ctx->ms_p[0] = !mixed ? (void*)ctx->p64 : ctx->ms_unroll > 1 ? (void*)ctx->ms_ring : (void*)ctx->p32;
 
   SolverState* h = ctx->st_host;
   memset(h, 0, sizeof(SolverState));
@@ -738,6 +751,7 @@ extern "C" int sqcg_multishift_cg_solve(sqcg_ctx* ctx, int nshift, const double*
   h->max_iter = max_iter;
   h->mixed = mixed;
   h->nshift = nshift;
+  h->ms_unroll = ctx->ms_unroll;
   h->alpha_prev = 1.0;
   h->beta_prev = 0.0;
   h->ms_ru = ru;
@@ -758,6 +772,12 @@ extern "C" int sqcg_multishift_cg_solve(sqcg_ctx* ctx, int nshift, const double*
   void* r = mixed ? (void*)ctx->r32 : (void*)ctx->r64;
   SQCG_TRY(layout_convert(ctx, SQCG_F64, b, wp, r, s));
   for (int j = 0; j < nshift; ++j) SQCG_TRY(layout_convert(ctx, SQCG_F64, b, wp, ctx->ms_p[j], s));
+  auto base_p = [&]() -> int {  // the base direction is the copy that shift 0's updates start from
+    if (ctx->ms_unroll > 1)
+      SQCG_CUDA_TRY(cudaMemcpyAsync(ctx->p32, ctx->ms_p[0], wbytes, cudaMemcpyDeviceToDevice, s));
+    return SQCG_OK;
+  };
+  SQCG_TRY(base_p());
   SQCG_TRY(read_state(ctx, s));
   if (h->bb == 0.0) {
     SQCG_CUDA_TRY(cudaStreamSynchronize(s));
@@ -784,11 +804,17 @@ extern "C" int sqcg_multishift_cg_solve(sqcg_ctx* ctx, int nshift, const double*
     if (eager) SQCG_TRY(run_eager(ctx, KIND_MS, mixed, b, xs, nshift, max_iter, s, &seg));
     else SQCG_TRY(run_loop(ctx, g, max_iter, s, &seg));
     loops += seg;
+    if (mixed) SQCG_TRY(launch_ms_x_form(ctx, nshift, (double2* const*)xs, false, s));
     if (h->done || !(h->ms_ru && h->need_update)) break;
     SQCG_TRY(ms_shift_aware_update(ctx, mixed, nshift, sig_l, tol_l, perm, b, xs, s, ru_count, &ru_launches,
                                    ru_shifts != 0));
+    SQCG_TRY(base_p());
+    if (mixed) SQCG_TRY(launch_ms_x_form(ctx, nshift, (double2* const*)xs, true, s));
+    ru_launches += mixed ? 2 : 0;
   }
-  int launches = 2 + 1 + nshift + loops * kMSKernelsPerIter + ru_launches;
+  // passes: steps (with the base direction's update where several make a pass), the flush, loop control
+  int launches = 2 + 1 + nshift + (mixed ? 1 : 0) + ru_launches +
+                 loops * (ctx->ms_unroll * (kMSKernelsPerStep + (ctx->ms_unroll > 1 ? 1 : 0)) + 2);
   const int loop_status = h->done ? h->status : SQCG_ERR_NOT_CONVERGED;
   int iters_s[SQCG_MAX_SHIFTS];
   for (int j = 0; j < nshift; ++j) iters_s[j] = h->iters_s[j];

@@ -181,13 +181,14 @@ __device__ inline void solver_finish_ms(SolverState* s, int fin, double v) {
     __syncthreads();  // every thread has read the base scalars before thread 0 writes them
     if (j == 0) {
       s->pAp = v;
+      if (s->ms_n >= s->ms_unroll) s->ms_n = 0;  // a pass starts
       if (bad) finish_breakdown(s);
       else s->alpha = a;
     }
   } else if (fin == FIN_MS_UPDATE) {  // |r_{k+1}|^2, beta_k, beta^s_k, per-shift convergence
     const bool bad = !isfinite(v);
     const double b = v / s->rr;
-    const int it = s->iter + 1;
+    const int it = s->iter + 1, step = s->ms_n;
     int any = 0;
     if (own && !bad && s->active[j] == 1) {
       const double zk = s->zeta[j], znext = s->beta_s[j];
@@ -199,19 +200,26 @@ __device__ inline void solver_finish_ms(SolverState* s, int fin, double v) {
       if (znext * znext * v <= s->stop_rr_s[j]) s->active[j] = 2;
       else any = 1;
     }
+    if (own && !bad) {
+      s->ms_ha[step][j] = s->alpha_s[j];
+      s->ms_hz[step][j] = j == 0 ? 1.0 : s->zeta[j];  // shift 0 is the base system: p = r + beta p
+      s->ms_hb[step][j] = j == 0 ? b : s->beta_s[j];
+      s->ms_act[step][j] = s->active[j];
+    }
     any = __syncthreads_or(any);  // also: every thread has read the base scalars
     if (j == 0) {
       if (bad) {
         finish_breakdown(s);
       } else {
+        s->ms_n = step + 1;
         s->iter = it;
         s->rr_prev = s->rr;
         s->rr = v;
         s->beta = b;
         s->alpha_prev = s->alpha;
         s->beta_prev = b;
-        if (!any) { s->done = 1; s->status = SQCG_OK; s->ms_final = 1; }
-        else if (it >= s->max_iter) { s->done = 1; s->status = SQCG_ERR_NOT_CONVERGED; s->ms_final = 1; }
+        if (!any) { s->done = 1; s->status = SQCG_OK; }
+        else if (it >= s->max_iter) { s->done = 1; s->status = SQCG_ERR_NOT_CONVERGED; }
         else if (s->ms_ru) {  // shift-aware reliable update: the loop pauses after this iteration
           if (v > s->rr_max) s->rr_max = v;
           if (v < s->delta2 * s->rr_max) s->need_update = 1;

@@ -49,6 +49,9 @@ struct LinkField {
 // solver state kept in device memory (scalars never leave the GPU inside a solve)
 // ---------------------------------------------------------------------------
 #define SQCG_MAX_SHIFTS 32
+// Steps of the mixed multi-shift loop per pass of its WHILE node (k_ms_flush): the updates of all shifts, which set
+// the loop's memory traffic, read and write x_s and p_s once for so many steps.
+constexpr int kMSUnroll = 4;
 
 struct SolverState {
   double sigma;    // diagonal term of the Krylov system
@@ -87,7 +90,8 @@ struct SolverState {
 
   // multi-shift CG (Jegerlehner recurrences; shift s uses sigma + dsig[s])
   int nshift;
-  int ms_final;  // the loop has just ended: the fused update still applies the last x_s updates
+  int ms_unroll;  // steps whose x_s and p_s updates are applied together (kMSUnroll, or 1)
+  int ms_n;       // steps of this pass taken so far; their scalars are in ms_h*, ms_act[step][shift]
   int active[SQCG_MAX_SHIFTS];  // 1 iterating, 2 converged with its last x update pending, 0 done
   double dsig[SQCG_MAX_SHIFTS];
   double stop_rr_s[SQCG_MAX_SHIFTS];
@@ -95,6 +99,10 @@ struct SolverState {
   double alpha_s[SQCG_MAX_SHIFTS], beta_s[SQCG_MAX_SHIFTS];
   double alpha_prev, beta_prev;
   int iters_s[SQCG_MAX_SHIFTS];
+  double ms_ha[kMSUnroll][SQCG_MAX_SHIFTS];  // x_s += ha p_s where ms_act is not 0,
+  double ms_hz[kMSUnroll][SQCG_MAX_SHIFTS];  // then p_s = hz r + hb p_s where it is 1
+  double ms_hb[kMSUnroll][SQCG_MAX_SHIFTS];
+  int ms_act[kMSUnroll][SQCG_MAX_SHIFTS];
   int ms_ru;           // shift-aware reliable updates: the loop pauses when need_update is set
   double ms_sums[3];   // the host-driven update's sums (k_ms_ru_sum3)
 };
@@ -206,7 +214,10 @@ struct sqcg_ctx {
   SolverState* st_host;  // pinned host mirror
 
   // multi-shift workspace
-  void* ms_p[SQCG_MAX_SHIFTS];  // per-shift search directions (working precision)
+  void* ms_p[SQCG_MAX_SHIFTS];  // per-shift search directions (working precision); with ms_unroll > 1 ms_p[0] is the
+                                // base direction as of the pass's start
+  float2* ms_ring;  // mixed: ms_p[0], then the residuals of steps 1 .. kMSUnroll - 1 of a pass (step 0's is r32)
+  int ms_unroll;
   void* rat_x[SQCG_MAX_SHIFTS];  // per-shift solutions of sqcg_rational_apply (FP64)
   int rat_n;
   double2* ms_stack;  // batched refinement (FP64): per-shift solutions [nshift][3][Vh], then a copy of b
@@ -315,9 +326,12 @@ int launch_flush_partial_x(sqcg_ctx* ctx, double2* x, int gate, cudaStream_t s);
 int launch_norm2_f64(sqcg_ctx* ctx, const double2* v, int fin, cudaStream_t s);
 int launch_scale_copy_f64(sqcg_ctx* ctx, const double2* src, double2* dst, double a, cudaStream_t s);
 
-int launch_ms_update_x(sqcg_ctx* ctx, int mixed, int nshift, double2* const* x, cudaStream_t s);
-
-int launch_ms_xpay(sqcg_ctx* ctx, int mixed, int nshift, double2* const* x, cudaStream_t s);
+// step k of a pass of the multi-shift loop: r -= alpha Ap with the scalar step; p = r + beta p of the base system
+// (only where ms_unroll > 1); the updates of all shifts for the steps of the pass; x_s between FP64 and float-float
+int launch_ms_update(sqcg_ctx* ctx, int mixed, int k, cudaStream_t s);
+int launch_ms_base_p(sqcg_ctx* ctx, int k, cudaStream_t s);
+int launch_ms_flush(sqcg_ctx* ctx, int mixed, int nshift, double2* const* x, cudaStream_t s);
+int launch_ms_x_form(sqcg_ctx* ctx, int nshift, double2* const* x, bool to_ff, cudaStream_t s);
 // shift-aware reliable update of the multi-shift loop: Re<a, b>, |b - z a|^2 and |a|^2 (FP64 vectors) into
 // st->ms_sums; then r <- rt (FP64, or FP32 in mixed mode) with p_s += zeta_s (rt - r) for every direction
 // still moving

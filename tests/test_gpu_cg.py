@@ -763,3 +763,29 @@ def test_persistent_loop_outside_the_float_float_step(sqcg, links_cache, monkeyp
             out.append((info.iters, lat.unpack(x) / scale))
         assert out[0][0] == out[1][0]
         assert rel(out[1][1], out[0][1]) <= 1e-5  # FP32 vectors, scalars rounded to FP32 from either step
+
+
+@pytest.mark.parametrize("flags", ["", "MS_SHIFT_RU", "MS_NO_RU"])
+@pytest.mark.parametrize("nshift", [1, 5])
+@pytest.mark.parametrize("tol", [0.5, 1e-2, 1e-4, 1e-6])
+def test_multishift_passes_that_end_early(sqcg, links_cache, flags, nshift, tol):
+    """The mixed multi-shift loop applies the shifts' updates for four steps together; loops and pauses that end after
+    any number of steps leave the same solutions: the residuals on the FP64 oracle, and as many iterations as the
+    FP64 mode, which applies each step by itself (10% and 5: a pass with an update missing is all refined again)."""
+    L = (6, 6, 6, 10)
+    fat, lng = links_cache(L, 680)
+    shifts = np.logspace(-2, 0, nshift).tolist()
+    src = synth.gaussian_source(L, 7900)
+    with sqcg.Lattice(L) as lat:
+        lat.load_links(fat, lng)
+        b = lat.pack(src)
+        xs = [lat.new_spinor() for _ in shifts]
+        ref = lat.multishift_cg_solve(shifts, b, xs, tol=tol, mode=sqcg.MODE_F64)
+        mode = sqcg.MODE_MIXED | (getattr(sqcg, flags) if flags else 0)
+        for x in xs:
+            x.normal_()  # overwritten
+        infos = lat.multishift_cg_solve(shifts, b, xs, tol=tol, mode=mode)
+        for j, s in enumerate(shifts):
+            assert infos[j].status == 0
+            assert oracle.true_rel_residual(L, fat, lng, s, src, lat.unpack(xs[j])) <= tol
+            assert infos[j].iters <= 1.1 * ref[j].iters + 5
