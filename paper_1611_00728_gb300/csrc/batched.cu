@@ -128,18 +128,6 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Two FP64 sums over SUB consecutive lanes (SUB <= 32) with the additions of one: the lower half of the lanes goes
-// on with a, the upper half with b. Totals: a in the first lane, b in lane SUB / 2. (An FP64 addition holds its
-// scheduler for 64 cycles on this GPU, whatever the lanes in it.)
-template <int SUB>
-__device__ __forceinline__ double sum2(double a, double b) {
-  const bool upper = (threadIdx.x + threadIdx.y * blockDim.x) & (SUB / 2);
-  double v = (upper ? b : a) + __shfl_xor_sync(0xffffffffu, upper ? a : b, SUB / 2);
-#pragma unroll
-  for (int o = SUB / 4; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o, SUB / 2);
-  return v;
-}
-
 // decode a tile into (lattice, RHS block, site block); RHS blocks fastest
 __device__ __forceinline__ int find_lat(const LatDev* lats, int nlat, int tile, bool fp64) {
   int k = 0;

@@ -442,6 +442,7 @@ __global__ void __launch_bounds__(kFinishThreads) k_finish_ffs(SolverState* st, 
 
 __global__ void __launch_bounds__(kFinishThreads) k_finish2(SolverState* st, const double* partials, int n, int fin,
                                                             int gate) {
+  pdl_wait();
   if (!gate_open(st, gate)) return;
   finish_partials2(st, partials, n, fin);
 }
@@ -501,9 +502,8 @@ int launch_finish_ffs(sqcg_ctx* ctx, int nblocks, int fin, int gate, cudaStream_
   return SQCG_OK;
 }
 
-int launch_finish2(sqcg_ctx* ctx, int nblocks, int fin, int gate, cudaStream_t s) {
-  k_finish2<<<1, kFinishThreads, 0, s>>>(ctx->st, ctx->partials, nblocks, fin, gate);
-  SQCG_CUDA_TRY(cudaGetLastError());
+int launch_finish2(sqcg_ctx* ctx, int nblocks, int fin, int gate, cudaStream_t s, bool pdl) {
+  SQCG_CUDA_TRY(launch_kernel(k_finish2, 1, kFinishThreads, 0, s, pdl, ctx->st, ctx->partials, nblocks, fin, gate));
   return SQCG_OK;
 }
 

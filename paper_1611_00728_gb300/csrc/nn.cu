@@ -142,7 +142,8 @@ struct ConvArgs {
   float2* out;            // OUT_GATE_*: [COUT][2][3][Vh]; OUT_EVEN_SCALED: even vector [3][Vh]
   float2* pre;            // pre-activations [COUT][2][3][Vh]: written by OUT_GATE_TRAIN, read by OUT_GATE_BWD
   const float2* sub;      // OUT_EVEN_SCALED: subtracted from the result (may be null)
-  double* partials;       // OUT_GATE_BWD: [block][2 COUT] sums of dL/dgate_a, dL/dgate_b
+  double* partials;       // OUT_GATE_BWD: [block][2 COUT] sums of dL/dgate_a, dL/dgate_b; with dot_r: see there
+  const float2 *dot_r, *dot_o;  // OUT_EVEN_SCALED, not null: sums of <out, dot_r>, then of <out, dot_o>, by block
   const float2* W;        // [9][COUT][CIN] complex (FP32 copy of BF16 values)
   const float* gate_a;    // [COUT]
   const float* gate_b;
@@ -184,152 +185,165 @@ __device__ __forceinline__ void gate_partials(const float (&red)[2 * CH][SITES +
   if (seg == 0) partials[(size_t)blockIdx.x * 2 * CH + v] = t;
 }
 
-// one lane per site: the layers with one input or one output channel (the 8 -> 8 layer is
-// k_conv88 below)
-template <int CIN, int COUT, int IN, int OUT>
-__global__ void __launch_bounds__(kThreads, 4) k_conv(ConvArgs a) {
+// The layers with one input or one output channel: a block is 32 sites, each warp transports one hop of all of them,
+// so a site's eight gathers are in flight together in eight warps (bound by their latency: one lane a site walked the
+// hops in turn, on two blocks an SM at 16^4). The sums over the taps keep the order of the taps. 8 -> 1 at 24^4 53 -> 43
+// us (ncu; the 163 MB take 24); both, with five and four blocks an SM, take a network application there from 281 to
+// 263 us and one at 16^4 from 75 to 65 (one parity's sites a block in the first layer: 267 and 66).
+
+// 1 -> 8, from the even sites: the odd sites' hops meet in shared memory beside the even sites' own vectors, then warp
+// o mixes output channel o of both. TILES: groups of 32 sites of each parity that a block takes in turn (with gate
+// sums to form: the sums of 128 sites make a row).
+constexpr int kHopThreads = 256;
+
+template <int OUT>
+__global__ void __launch_bounds__(kHopThreads, 5) k_conv_1to8(ConvArgs a) {
+  pdl_wait();
+  pdl_launch_dependents();
   if (a.st && !gate_open(a.st, a.gate)) return;
-  __shared__ float2 W[NT * COUT * CIN];
-  for (int j = threadIdx.x; j < NT * COUT * CIN; j += blockDim.x) W[j] = a.W[j];
-  __syncthreads();
+  constexpr int TILES = OUT == OUT_GATE_BWD ? 2 : 1;
+  __shared__ float2 t[NT][3][32];  // the even site's vector, the odd site's transported ones
+  __shared__ float red[OUT == OUT_GATE_BWD ? 2 * CH : 1][64 * TILES + 1];
   const Geom& g = a.g;
   const int Vh = g.Vh;
-  const int gid = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool valid = gid < a.npar * Vh;
-  if (!valid && OUT != OUT_GATE_BWD) return;  // with sums to form, lanes past the end compute site 0 and add nothing
-  const int sv = valid ? gid : 0;
-  const int par = a.par0 + sv / Vh;
-  const int i = sv % Vh;
-  const int q = 1 - par;
-  const Site s = site_of(g, i, par);
-  const float sc = (IN == IN_EVEN_SCALED) ? (float)*a.scale : 1.f;
-
-  float2 acc[COUT][3];
+  const int lane = threadIdx.x & 31, hop = threadIdx.x >> 5, o = hop;
+  const int mu = hop >> 1, dir = hop & 1;
+#pragma unroll 1
+  for (int k = 0; k < TILES; ++k) {
+    const int gid = (blockIdx.x * TILES + k) * 32 + lane;
+    const bool valid = gid < Vh;
+    const int i = valid ? gid : 0;
+    const float sc = (float)*a.scale;
+    {
+      const int j = nbr(g, site_of(g, i, 1), mu, dir == 0 ? +1 : -1);
+      float2 u[9], v[3], tv[3];
+      if (dir == 0) load_link9(a.fat[1] + (size_t)mu * 9 * Vh, Vh, i, u);  // F_mu(n)
+      else load_link9(a.fat[0] + (size_t)mu * 9 * Vh, Vh, j, u);           // F_mu(n - mu)
 #pragma unroll
-  for (int o = 0; o < COUT; ++o)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) acc[o][c] = make_float2(0.f, 0.f);
-
-  // input channel ci at parity pp, half index j
-  auto load_in = [&](int ci, int pp, int j, float2 (&v)[3]) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      if (IN == IN_FULL) {
-        v[c] = __ldg(a.in + (((size_t)ci * 2 + pp) * 3 + c) * Vh + j);
-      } else {
-        const float2 t = __ldg(a.in + (size_t)c * Vh + j);
-        v[c] = make_float2(t.x * sc, t.y * sc);
+      for (int c = 0; c < 3; ++c) {
+        const float2 x = __ldg(a.in + (size_t)c * Vh + j);
+        v[c] = make_float2(x.x * sc, x.y * sc);
       }
+      if (hop < 3) {
+        const float2 x = __ldg(a.in + (size_t)hop * Vh + i);
+        t[0][hop][lane] = make_float2(x.x * sc, x.y * sc);
+      }
+      apply_link(u, dir == 1, v, tv);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) t[1 + hop][c][lane] = tv[c];
     }
-  };
-  auto mix = [&](int tap, const float2 (&t)[3], int ci) {
+    float2 w[NT];  // this warp's output channel
 #pragma unroll
-    for (int o = 0; o < COUT; ++o) {
-      const float2 w = W[(tap * COUT + o) * CIN + ci];
+    for (int tap = 0; tap < NT; ++tap) w[tap] = __ldg(a.W + tap * CH + o);
+    const float ga = a.gate_a[o], gb = a.gate_b[o];
+    __syncthreads();
 #pragma unroll
-      for (int c = 0; c < 3; ++c) cmac(acc[o][c], w, t[c]);
-    }
-  };
-
-  // self tap (input of the same parity; an even-only input is zero on odd sites)
-  if (IN == IN_FULL || par == 0) {
+    for (int par = 0; par < 2; ++par) {
+      float2 acc[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
-    for (int ci = 0; ci < CIN; ++ci) {
-      float2 v[3];
-      load_in(ci, par, i, v);
-      mix(0, v, ci);
-    }
-  }
-  // hops (input of the other parity); each link is loaded once and applied to every channel
-  if (IN == IN_FULL || q == 0) {
+      for (int tap = par; tap < (par == 0 ? 1 : NT); ++tap)
 #pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
+        for (int c = 0; c < 3; ++c) cmac(acc[c], w[tap], t[tap][c][lane]);
+      const size_t at = ((size_t)o * 2 + par) * 3 * Vh + i;
+      if constexpr (OUT == OUT_GATE_BWD) {
+        float2 h[3];
+        float da, db;
 #pragma unroll
-      for (int dir = 0; dir < 2; ++dir) {
-        const int j = nbr(g, s, mu, dir == 0 ? +1 : -1);
-        float2 u[9];
-        if (dir == 0) load_link9(a.fat[par] + (size_t)mu * 9 * Vh, Vh, i, u);  // F_mu(n)
-        else load_link9(a.fat[q] + (size_t)mu * 9 * Vh, Vh, j, u);             // F_mu(n - mu)
-        const int tap = 1 + 2 * mu + dir;
-        if constexpr (COUT == 1 && CIN > 1) {
-          // one output channel: the weights mix channels and the link acts on colour, so
-          // sum_ci w_ci (U v_ci) = U (sum_ci w_ci v_ci): mix first, transport once
-          float2 m[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll 2
-          for (int ci = 0; ci < CIN; ++ci) {
-            float2 v[3];
-            load_in(ci, q, j, v);
-            const float2 w = W[tap * CIN + ci];
+        for (int c = 0; c < 3; ++c) h[c] = __ldg(a.pre + at + (size_t)c * Vh);
+        gate_backward(h, ga, gb, acc, da, db);
+        if (valid)
 #pragma unroll
-            for (int c = 0; c < 3; ++c) cmac(m[c], w, v[c]);
-          }
-          float2 t[3];
-          apply_link(u, dir == 1, m, t);
+          for (int c = 0; c < 3; ++c) a.out[at + (size_t)c * Vh] = acc[c];
+        red[o][(2 * k + par) * 32 + lane] = valid ? da : 0.f;
+        red[CH + o][(2 * k + par) * 32 + lane] = valid ? db : 0.f;
+      } else if (valid) {
+        float n2 = 0.f;
 #pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            acc[0][c].x += t[c].x;
-            acc[0][c].y += t[c].y;
-          }
-        } else {
-#pragma unroll 2
-          for (int ci = 0; ci < CIN; ++ci) {
-            float2 v[3], t[3];
-            load_in(ci, q, j, v);
-            apply_link(u, dir == 1, v, t);
-            mix(tap, t, ci);
-          }
+        for (int c = 0; c < 3; ++c) n2 = fmaf(acc[c].x, acc[c].x, fmaf(acc[c].y, acc[c].y, n2));
+        const float gf = 1.f / (1.f + __expf(-(ga * n2 + gb)));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          if (OUT == OUT_GATE_TRAIN) a.pre[at + (size_t)c * Vh] = acc[c];
+          a.out[at + (size_t)c * Vh] = make_float2(acc[c].x * gf, acc[c].y * gf);
         }
       }
     }
+    if (TILES > 1) __syncthreads();  // t is read before the next tile's is written; red is complete after the last
   }
-  // epilogue
-  if (OUT == OUT_EVEN_SCALED) {
+  if constexpr (OUT == OUT_GATE_BWD)
+    if (threadIdx.x < 128) gate_partials<64 * TILES>(red, a.partials);
+}
+
+// 8 -> 1, onto the even sites: the weights mix channels and the link acts on colour, so sum_ci w_ci (U v_ci) =
+// U (sum_ci w_ci v_ci): warp h < 8 mixes hop h's eight channels and transports the sum once, warp 8 mixes the site's
+// own; then warp c adds colour c of the nine.
+constexpr int kTapThreads = 288;
+
+__global__ void __launch_bounds__(kTapThreads, 4) k_conv_8to1(ConvArgs a) {
+  __shared__ float2 t[NT][3][32];
+  __shared__ double dots[2][3];
+  pdl_wait();
+  pdl_launch_dependents();
+  if (a.st && !gate_open(a.st, a.gate)) return;
+  const Geom& g = a.g;
+  const int Vh = g.Vh;
+  const int lane = threadIdx.x & 31, hop = threadIdx.x >> 5;
+  const int gid = blockIdx.x * 32 + lane;
+  const bool valid = gid < Vh;
+  const int i = valid ? gid : 0;
+  const int mu = hop >> 1, dir = hop & 1;
+  const bool self = hop == 8;
+  const int tap = self ? 0 : 1 + hop;
+  int j = i;
+  if (!self) j = nbr(g, site_of(g, i, 0), mu, dir == 0 ? +1 : -1);
+  float2 m[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+  for (int ci = 0; ci < CH; ++ci) {
+    const float2 w = __ldg(a.W + tap * CH + ci);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) cmac(m[c], w, __ldg(a.in + (((size_t)ci * 2 + (self ? 0 : 1)) * 3 + c) * Vh + j));
+  }
+  if (!self) {
+    float2 u[9], tv[3];
+    if (dir == 0) load_link9(a.fat[0] + (size_t)mu * 9 * Vh, Vh, i, u);  // F_mu(n)
+    else load_link9(a.fat[1] + (size_t)mu * 9 * Vh, Vh, j, u);           // F_mu(n - mu)
+    apply_link(u, dir == 1, m, tv);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) m[c] = tv[c];
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) t[tap][c][lane] = m[c];
+  __syncthreads();
+  const int c = hop;
+  if (c < 3) {
+    float2 z = t[0][c][lane];
+#pragma unroll
+    for (int k = 1; k < NT; ++k) {
+      z.x += t[k][c][lane].x;
+      z.y += t[k][c][lane].y;
+    }
     const float os = (float)*a.scale;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      float2 z = make_float2(acc[0][c].x * os, acc[0][c].y * os);
-      if (a.sub) {
-        const float2 e = __ldg(a.sub + (size_t)c * Vh + i);
-        z.x -= e.x;
-        z.y -= e.y;
-      }
-      a.out[(size_t)c * Vh + i] = z;
+    z.x *= os;
+    z.y *= os;
+    const size_t at = (size_t)c * Vh + i;
+    if (a.sub) {
+      const float2 e = __ldg(a.sub + at);
+      z.x -= e.x;
+      z.y -= e.y;
     }
-  } else if constexpr (OUT == OUT_GATE_BWD) {
-    __shared__ float red[2 * CH][kThreads + 1];
-#pragma unroll
-    for (int o = 0; o < COUT; ++o) {
-      float2 h[3];
-      float da, db;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) h[c] = __ldg(a.pre + (((size_t)o * 2 + par) * 3 + c) * Vh + i);
-      gate_backward(h, a.gate_a[o], a.gate_b[o], acc[o], da, db);
-      if (valid)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) a.out[(((size_t)o * 2 + par) * 3 + c) * Vh + i] = acc[o][c];
-      red[o][threadIdx.x] = valid ? da : 0.f;
-      red[CH + o][threadIdx.x] = valid ? db : 0.f;
-    }
-    __syncthreads();
-    gate_partials<kThreads>(red, a.partials);
-  } else {
-#pragma unroll
-    for (int o = 0; o < COUT; ++o) {
-      float gf = 1.f;
-      if (OUT == OUT_GATE_TRAIN || OUT == OUT_GATE_INFER) {
-        float n2 = 0.f;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) n2 = fmaf(acc[o][c].x, acc[o][c].x, fmaf(acc[o][c].y, acc[o][c].y, n2));
-        gf = 1.f / (1.f + __expf(-(a.gate_a[o] * n2 + a.gate_b[o])));
-      }
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const size_t k = (((size_t)o * 2 + par) * 3 + c) * Vh + i;
-        if (OUT == OUT_GATE_TRAIN) a.pre[k] = acc[o][c];
-        a.out[k] = make_float2(acc[o][c].x * gf, acc[o][c].y * gf);
-      }
+    if (valid) a.out[at] = z;
+    if (a.dot_r) {
+      const float2 r = __ldg(a.dot_r + at), o = __ldg(a.dot_o + at);
+      const float u = valid ? fmaf(z.x, r.x, z.y * r.y) : 0.f, v = valid ? fmaf(z.x, o.x, z.y * o.y) : 0.f;
+      const double d = sum2<32>((double)u, (double)v);
+      if ((lane & 15) == 0) dots[lane >> 4][c] = d;
     }
   }
+  if (!a.dot_r) return;
+  __syncthreads();
+  if (threadIdx.x < 2)
+    a.partials[(size_t)threadIdx.x * gridDim.x + blockIdx.x] =
+        (dots[threadIdx.x][0] + dots[threadIdx.x][1]) + dots[threadIdx.x][2];
 }
 
 // The 8 -> 8 layer with two lanes per site. Each lane accumulates 4 of the 8 output
@@ -340,7 +354,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_conv(ConvArgs a) {
 // takes part in the shuffles.
 template <int OUT>
 __global__ void __launch_bounds__(kThreads, 5) k_conv88(ConvArgs a) {
-  if (a.st && !gate_open(a.st, a.gate)) return;
+  pdl_launch_dependents();
   // weights as [tap][c_in][c_out], each complex w stored as (w.x, w.x, -w.y, w.y): the two packed
   // operands of acc += w t in two-lane FMAs, acc = (w.x, w.x) (t.x, t.y) + (-w.y, w.y) (t.y, t.x) + acc,
   // which rounds exactly as the scalar complex multiply-add (same products, same order per lane)
@@ -350,6 +364,8 @@ __global__ void __launch_bounds__(kThreads, 5) k_conv88(ConvArgs a) {
     const float2 w = a.W[j];
     W[(tap * CH + ci) * CH + o] = make_float4(w.x, w.x, -w.y, w.y);
   }
+  pdl_wait();
+  if (a.st && !gate_open(a.st, a.gate)) return;
   __syncthreads();
   const Geom& g = a.g;
   const int Vh = g.Vh;
@@ -503,7 +519,7 @@ __device__ __forceinline__ int tc_half(int row, int half) { return half ^ ((row 
 
 template <int OUT>
 __global__ void __launch_bounds__(kThreads, 3) k_conv88_tc(ConvArgs a) {
-  if (a.st && !gate_open(a.st, a.gate)) return;
+  pdl_launch_dependents();
   constexpr int kWarps = kThreads / 32;
   // B fragments [tap][nt][half][lane]: rows k = 2 ci + comp (ci = t, t + 4 for half 0, 1), column n = g of
   // each 8-column half nt, i.e. output channel o = 4 nt + g / 2, component g % 2 (lane = 4 g + t)
@@ -516,6 +532,8 @@ __global__ void __launch_bounds__(kThreads, 3) k_conv88_tc(ConvArgs a) {
     // (re, im) input component -> output component oc: re: (w.x, -w.y); im: (w.y, w.x)
     sB[tap][nt][half][l] = oc == 0 ? pack_bf16(w.x, -w.y) : pack_bf16(w.y, w.x);
   }
+  pdl_wait();  // the weights were there before the kernel in front was launched
+  if (a.st && !gate_open(a.st, a.gate)) return;
   __syncthreads();
   const Geom& g = a.g;
   const int Vh = g.Vh;
@@ -822,12 +840,13 @@ __global__ void __launch_bounds__(1024) k_sum_partials(SumSegments S, float* gra
   }
 }
 
-// generic FP32 two-vector dot products over even vectors [3][Vh]: sum Re<a, b>
+// FP32 two-vector dot products over even vectors [3][Vh], sum Re<a, b>, in FP64 (whose rate bounds it: a SM does 2
+// operations a clock, so warps that walk over several sites and reduce once beat one site a thread); the second
+// sum's partials follow the first's.
 __global__ void __launch_bounds__(kRedThreads) k_dot2(const float2* a1, const float2* b1, const float2* a2,
                                                       const float2* b2, int Vh, double* partials) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
   double u = 0.0, v = 0.0;
-  if (i < Vh) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Vh; i += gridDim.x * blockDim.x) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const size_t k = (size_t)c * Vh + i;
@@ -839,20 +858,30 @@ __global__ void __launch_bounds__(kRedThreads) k_dot2(const float2* a1, const fl
       }
     }
   }
-  block_partial2(u, v, partials);
+  if (a2) {
+    block_partial2(u, v, partials);
+  } else {
+    u = block_sum(u);
+    if (threadIdx.x == 0) {
+      partials[blockIdx.x] = u;
+      partials[gridDim.x + blockIdx.x] = 0.0;
+    }
+  }
 }
 
 // two-sum finisher into nn scalars: mode 0: scal[0] = s = sqrt(3Vh/a), scal[1] = 1/s (input scale);
 // mode 1: scal[2] = <e,r> = b, scal[3] += <d,Ad>/<e,r> = a/b (loss), scal[4] = 2 / (b s), which takes A d to
 // dL/d(network output before the output scale)
 __global__ void k_nn_finish(const double* partials, int n, double* scal, int mode, int Vh) {
+  pdl_wait();
+  pdl_launch_dependents();
   double a = 0.0, b = 0.0;
   for (int j = threadIdx.x; j < n; j += blockDim.x) {
     a += partials[j];
-    b += partials[n + j];
+    if (mode) b += partials[n + j];
   }
   a = block_sum(a);
-  b = block_sum(b);
+  if (mode) b = block_sum(b);
   if (threadIdx.x == 0) {
     if (mode == 0) {
       scal[0] = (a > 0) ? sqrt(3.0 * Vh / a) : 0.0;
@@ -941,9 +970,13 @@ constexpr size_t kScalGradBytes = 8 * sizeof(double) + NPARAM * sizeof(float);
 
 int conv_launch(sqcg_nn* nn, int layer, bool adjoint, int in_mode, int out_mode, const float2* in, float2* out,
                 float2* pre, int par0, int npar, const SolverState* st, int gate, const double* scale,
-                cudaStream_t s, const float2* sub = nullptr, double* partials = nullptr) {
+                cudaStream_t s, const float2* sub = nullptr, double* partials = nullptr, bool pdl = false,
+                const float2* dot_r = nullptr, const float2* dot_o = nullptr) {
   sqcg_ctx* ctx = nn->ctx;
+  pdl = pdl && ctx->pdl;
   ConvArgs a;
+  a.dot_r = dot_r;
+  a.dot_o = dot_o;
   a.g = ctx->g;
   const size_t Vh = ctx->g.Vh;
   a.fat[0] = ctx->fat32;
@@ -964,49 +997,59 @@ int conv_launch(sqcg_nn* nn, int layer, bool adjoint, int in_mode, int out_mode,
   a.gate = gate;
   a.par0 = par0;
   a.npar = npar;
-  const int grid = nn_grid(npar * (int)Vh);
+  const int grid = nn_grid(npar * (int)Vh), tiles = grid_for((int)Vh, 32);
   const int grid2 = nn_grid(2 * npar * (int)Vh);  // the two-lane 8 -> 8 kernel
   // channel counts of the (possibly adjoint) layer
   int cin = (layer == 0) ? 1 : CH, cout = (layer == 2) ? 1 : CH;
   if (adjoint) { const int t = cin; cin = cout; cout = t; }
+  cudaError_t e = cudaSuccess;
   if (cin == 1 && cout == CH && in_mode == IN_EVEN_SCALED && out_mode == OUT_GATE_INFER)
-    k_conv<1, CH, IN_EVEN_SCALED, OUT_GATE_INFER><<<grid, kThreads, 0, s>>>(a);
+    e = launch_kernel(k_conv_1to8<OUT_GATE_INFER>, tiles, kHopThreads, 0, s, pdl, a);
   else if (cin == 1 && cout == CH && in_mode == IN_EVEN_SCALED && out_mode == OUT_GATE_TRAIN)
-    k_conv<1, CH, IN_EVEN_SCALED, OUT_GATE_TRAIN><<<grid, kThreads, 0, s>>>(a);
+    e = launch_kernel(k_conv_1to8<OUT_GATE_TRAIN>, tiles, kHopThreads, 0, s, pdl, a);
   else if (cin == CH && cout == CH && in_mode == IN_FULL && out_mode == OUT_GATE_INFER && !adjoint &&
            nn->mixing == SQCG_NN_MIX_BF16)
-    k_conv88_tc<OUT_GATE_INFER><<<grid_for(npar * (int)Vh, kThreads / 2), kThreads, 0, s>>>(a);
+    e = launch_kernel(k_conv88_tc<OUT_GATE_INFER>, grid_for(npar * (int)Vh, kThreads / 2), kThreads, 0, s, pdl, a);
   else if (cin == CH && cout == CH && in_mode == IN_FULL && out_mode == OUT_GATE_INFER)
-    k_conv88<OUT_GATE_INFER><<<grid2, kThreads, 0, s>>>(a);
+    e = launch_kernel(k_conv88<OUT_GATE_INFER>, grid2, kThreads, 0, s, pdl, a);
   else if (cin == CH && cout == CH && in_mode == IN_FULL && out_mode == OUT_GATE_TRAIN)
-    k_conv88<OUT_GATE_TRAIN><<<grid2, kThreads, 0, s>>>(a);
+    e = launch_kernel(k_conv88<OUT_GATE_TRAIN>, grid2, kThreads, 0, s, pdl, a);
   else if (cin == CH && cout == CH && in_mode == IN_FULL && out_mode == OUT_GATE_BWD)
-    k_conv88<OUT_GATE_BWD><<<grid2, kThreads, 0, s>>>(a);
+    e = launch_kernel(k_conv88<OUT_GATE_BWD>, grid2, kThreads, 0, s, pdl, a);
   else if (cin == CH && cout == 1 && in_mode == IN_FULL && out_mode == OUT_EVEN_SCALED)
-    k_conv<CH, 1, IN_FULL, OUT_EVEN_SCALED><<<grid, kThreads, 0, s>>>(a);
+    e = launch_kernel(k_conv_8to1, tiles, kTapThreads, 0, s, pdl, a);
   else if (cin == 1 && cout == CH && in_mode == IN_EVEN_SCALED && out_mode == OUT_GATE_BWD)
-    k_conv<1, CH, IN_EVEN_SCALED, OUT_GATE_BWD><<<grid, kThreads, 0, s>>>(a);
+    e = launch_kernel(k_conv_1to8<OUT_GATE_BWD>, grid, kHopThreads, 0, s, pdl, a);  // 64 sites of each parity a block
   else
     return SQCG_ERR_INVALID_ARG;
-  SQCG_CUDA_TRY(cudaGetLastError());
+  SQCG_CUDA_TRY(e);
   return SQCG_OK;
 }
 
-// z = N(r) on the even sites (inference). scale[0] must hold s, scale[1] 1/s.
+// z = N(r) on the even sites (inference). scale[0] must hold s, scale[1] 1/s. pdl: a kernel is in front of it, and one
+// launched without programmatic dependent launch in front of that or nearer (the weights are read ahead of the wait).
+// dot_r: the sums of <z, dot_r>, then of <z, dot_o>, over blocks of 32 sites go to the context's partials.
 int nn_forward_infer(sqcg_nn* nn, const float2* r, float2* z, const double* scale, const SolverState* st, int gate,
-                     cudaStream_t s) {
-  SQCG_TRY(conv_launch(nn, 0, false, IN_EVEN_SCALED, OUT_GATE_INFER, r, nn->h1, nullptr, 0, 2, st, gate, scale, s));
-  SQCG_TRY(conv_launch(nn, 1, false, IN_FULL, OUT_GATE_INFER, nn->h1, nn->h2, nullptr, 0, 2, st, gate, nullptr, s));
-  SQCG_TRY(conv_launch(nn, 2, false, IN_FULL, OUT_EVEN_SCALED, nn->h2, z, nullptr, 0, 1, st, gate, scale + 1, s));
-  return SQCG_OK;
+                     cudaStream_t s, bool pdl, const float2* dot_r = nullptr, const float2* dot_o = nullptr) {
+  SQCG_TRY(conv_launch(nn, 0, false, IN_EVEN_SCALED, OUT_GATE_INFER, r, nn->h1, nullptr, 0, 2, st, gate, scale, s,
+                       nullptr, nullptr, pdl));
+  SQCG_TRY(conv_launch(nn, 1, false, IN_FULL, OUT_GATE_INFER, nn->h1, nn->h2, nullptr, 0, 2, st, gate, nullptr, s,
+                       nullptr, nullptr, true));
+  return conv_launch(nn, 2, false, IN_FULL, OUT_EVEN_SCALED, nn->h2, z, nullptr, 0, 1, st, gate, scale + 1, s,
+                     nullptr, nn->ctx->partials, true, dot_r, dot_o);
+}
+
+int dot2_grid(const sqcg_nn* nn) {
+  const int full = grid_for(nn->ctx->g.Vh, kRedThreads), two = 2 * nn->ctx->nsm;
+  return full < two ? full : two;
 }
 
 // scale of r into scal[0..1] (no solver state involved)
 int nn_input_scale(sqcg_nn* nn, const float2* r, cudaStream_t s) {
-  const int Vh = nn->ctx->g.Vh, grid = (Vh + kRedThreads - 1) / kRedThreads;
+  const int Vh = nn->ctx->g.Vh, grid = dot2_grid(nn);
   k_dot2<<<grid, kRedThreads, 0, s>>>(r, r, nullptr, nullptr, Vh, nn->partials);
-  k_nn_finish<<<1, kRedThreads, 0, s>>>(nn->partials, grid, nn->scal, 0, Vh);
   SQCG_CUDA_TRY(cudaGetLastError());
+  SQCG_CUDA_TRY(launch_kernel(k_nn_finish, 1, kRedThreads, 0, s, nn->ctx->pdl != 0, nn->partials, grid, nn->scal, 0, Vh));
   return SQCG_OK;
 }
 
@@ -1081,17 +1124,19 @@ int nn_pair(sqcg_nn* nn, double sigma, const float2* r, const float2* e, cudaStr
   sqcg_ctx* ctx = nn->ctx;
   const int Vh = ctx->g.Vh;
   SQCG_TRY(nn_input_scale(nn, r, s));
-  SQCG_TRY(conv_launch(nn, 0, false, IN_EVEN_SCALED, OUT_GATE_TRAIN, r, nn->h1, nn->a1, 0, 2, nullptr, 0, nn->scal, s));
-  SQCG_TRY(conv_launch(nn, 1, false, IN_FULL, OUT_GATE_TRAIN, nn->h1, nn->h2, nn->a2, 0, 2, nullptr, 0, nullptr, s));
+  SQCG_TRY(conv_launch(nn, 0, false, IN_EVEN_SCALED, OUT_GATE_TRAIN, r, nn->h1, nn->a1, 0, 2, nullptr, 0, nn->scal, s, nullptr, nullptr,
+                       true));
+  SQCG_TRY(conv_launch(nn, 1, false, IN_FULL, OUT_GATE_TRAIN, nn->h1, nn->h2, nn->a2, 0, 2, nullptr, 0, nullptr, s, nullptr,
+                       nullptr, true));
   // d = z - e; Ad = (sigma - D_eo D_oe) d in FP32; <d,Ad>, <e,r>
   SQCG_TRY(conv_launch(nn, 2, false, IN_FULL, OUT_EVEN_SCALED, nn->h2, nn->d, nullptr, 0, 1, nullptr, 0,
-                       nn->scal + 1, s, e));
+                       nn->scal + 1, s, e, nullptr, true));
   DslashLaunch L = {};
   L.out_parity = 1; L.prec = L.out_prec = SQCG_F32; L.epi = EPI_PLAIN; L.in = nn->d; L.out = nn->tmp;
   SQCG_TRY(launch_dslash(ctx, L, s));
   L.out_parity = 0; L.epi = EPI_NORMAL; L.in = nn->tmp; L.out = nn->Ad; L.y = nn->d; L.sigma = sigma;
   SQCG_TRY(launch_dslash(ctx, L, s));
-  const int grid = (Vh + kRedThreads - 1) / kRedThreads;
+  const int grid = dot2_grid(nn);
   if (nn->loss_norm == 2) {
     // L = <Ad, Ad> / <r, r>; dL/dz = 2 A (A d) / <r, r>   (A e = r: the preconditioned residual)
     L = DslashLaunch{};
@@ -1242,7 +1287,7 @@ int sqcg_nn_apply(sqcg_nn* nn, const void* r, void* z) {
   if (!nn || !r || !z || r == z) return SQCG_ERR_INVALID_ARG;
   cudaStream_t s = nn->ctx->stream;
   SQCG_TRY(nn_input_scale(nn, (const float2*)r, s));
-  return nn_forward_infer(nn, (const float2*)r, (float2*)z, nn->scal, nullptr, GATE_NONE, s);
+  return nn_forward_infer(nn, (const float2*)r, (float2*)z, nn->scal, nullptr, GATE_NONE, s, true);
 }
 
 int sqcg_nn_loss_grad(sqcg_nn* nn, double sigma, const void* r, const void* e, double* loss, float* grad) {
@@ -1305,6 +1350,7 @@ __global__ void __launch_bounds__(kRedThreads, 5) k_fcg_update(double2* __restri
                                                             float2* __restrict__ r_old, const float2* __restrict__ p,
                                                             const float2* __restrict__ q, int Vh, SolverState* st,
                                                             double* partials) {
+  pdl_wait();
   if (!gate_open(st, GATE_ITER)) return;
   const double alpha = st->alpha;
   const float fa = (float)alpha;
@@ -1339,34 +1385,8 @@ __global__ void __launch_bounds__(kRedThreads, 5) k_fcg_update(double2* __restri
   block_partial(nrm, partials);
 }
 
-// <z, r> and <z, r_old> partials: each site's sum in FP32, the sums over sites in FP64
-__global__ void __launch_bounds__(kRedThreads) k_fcg_dots(const float2* __restrict__ z, const float2* __restrict__ r,
-                                                          const float2* __restrict__ r_old, int Vh,
-                                                          const SolverState* st, double* partials) {
-  if (!gate_open(st, GATE_ITER)) return;
-  double a = 0.0, b = 0.0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Vh; i += gridDim.x * blockDim.x) {
-    float2 zc[3], rc[3], oc[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const size_t k = (size_t)c * Vh + i;
-      zc[c] = z[k];
-      rc[c] = r[k];
-      oc[c] = r_old[k];
-    }
-    float pa = 0.f, pb = 0.f;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      pa = fmaf(zc[c].x, rc[c].x, fmaf(zc[c].y, rc[c].y, pa));
-      pb = fmaf(zc[c].x, oc[c].x, fmaf(zc[c].y, oc[c].y, pb));
-    }
-    a += (double)pa;
-    b += (double)pb;
-  }
-  block_partial2(a, b, partials);
-}
-
-// |r|^2 partials for the network input scale (gated)
+// |r|^2 partials for the scale of the first residual (later ones have theirs from the update's or the reliable
+// update's norm)
 __global__ void __launch_bounds__(kRedThreads) k_norm_gated(const float2* __restrict__ r, int Vh, const SolverState* st,
                                                             double* partials) {
   if (!gate_open(st, GATE_ITER)) return;
@@ -1386,6 +1406,7 @@ __global__ void __launch_bounds__(kRedThreads) k_norm_gated(const float2* __rest
 // p = z + beta p over the 3 Vh colour components
 __global__ void __launch_bounds__(kRedThreads) k_fcg_xpay(const float2* __restrict__ z, float2* __restrict__ p, int n,
                                                           const SolverState* st) {
+  pdl_wait();
   if (!gate_open(st, GATE_ITER)) return;
   const float b = (float)st->beta;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -1402,16 +1423,6 @@ __global__ void k_copy2(const float2* __restrict__ a, float2* __restrict__ b, in
   if (i < n) b[i] = a[i];
 }
 
-// z = N(r) with the input scale taken from the solver state
-int fcg_precondition(sqcg_nn* nn, int gate, cudaStream_t s) {
-  sqcg_ctx* ctx = nn->ctx;
-  const int Vh = ctx->g.Vh, grid = blas_grid(ctx);
-  k_norm_gated<<<grid, kRedThreads, 0, s>>>(ctx->r32, Vh, ctx->st, ctx->partials);
-  SQCG_CUDA_TRY(cudaGetLastError());
-  SQCG_TRY(launch_finish(ctx, grid, FIN_NN_SCALE, gate, s));
-  return nn_forward_infer(nn, ctx->r32, nn->z, &ctx->st->nn_s, ctx->st, gate, s);
-}
-
 // One flexible-CG iteration in three parts: head (A p, <p,Ap>, alpha; x, r update, |r|^2), the
 // FP64 reliable update (fcg_reliable), tail (z = N(r), beta, p = z + beta p).
 int fcg_head(sqcg_nn* nn, void* x, cudaStream_t cs) {
@@ -1423,23 +1434,22 @@ int fcg_head(sqcg_nn* nn, void* x, cudaStream_t cs) {
   SQCG_TRY(launch_dslash(ctx, L, cs));
   L = DslashLaunch{};
   L.out_parity = 0; L.prec = L.out_prec = SQCG_F32; L.epi = EPI_NORMAL_DOT; L.in = ctx->tmp32; L.out = ctx->Ap32;
-  L.y = ctx->p32; L.sigma_dev = &ctx->st->sigma; L.gate = GATE_ITER; L.fin = FIN_FCG_PAP;
+  L.y = ctx->p32; L.sigma_dev = &ctx->st->sigma; L.gate = GATE_ITER; L.fin = FIN_FCG_PAP; L.pdl = 1;
   SQCG_TRY(launch_dslash(ctx, L, cs));
-  k_fcg_update<<<grid, kRedThreads, 0, cs>>>((double2*)x, ctx->r32, nn->r_old, ctx->p32, ctx->Ap32, Vh, ctx->st,
-                                             ctx->partials);
-  SQCG_CUDA_TRY(cudaGetLastError());
-  return launch_finish(ctx, grid, FIN_UPDATE, GATE_ITER, cs);
+  const bool pdl = ctx->pdl != 0;
+  SQCG_CUDA_TRY(launch_kernel(k_fcg_update, grid, kRedThreads, 0, cs, pdl, (double2*)x, ctx->r32, nn->r_old, ctx->p32,
+                              ctx->Ap32, Vh, ctx->st, ctx->partials));
+  return launch_finish(ctx, grid, FIN_UPDATE, GATE_ITER, cs, pdl);
 }
 
 int fcg_tail(sqcg_nn* nn, cudaStream_t cs) {
   sqcg_ctx* ctx = nn->ctx;
-  const int Vh = ctx->g.Vh, grid = blas_grid(ctx);
-  SQCG_TRY(fcg_precondition(nn, GATE_ITER, cs));
-  k_fcg_dots<<<grid, kRedThreads, 0, cs>>>(nn->z, ctx->r32, nn->r_old, Vh, ctx->st, ctx->partials);
-  SQCG_CUDA_TRY(cudaGetLastError());
-  SQCG_TRY(launch_finish2(ctx, grid, FIN_FCG_BETA, GATE_ITER, cs));
-  k_fcg_xpay<<<grid, kRedThreads, 0, cs>>>(nn->z, ctx->p32, 3 * Vh, ctx->st);
-  SQCG_CUDA_TRY(cudaGetLastError());
+  const int Vh = ctx->g.Vh;
+  const bool pdl = ctx->pdl != 0;
+  // the conditional node in front of the network has no programmatic edge; the last layer forms the dot products
+  SQCG_TRY(nn_forward_infer(nn, ctx->r32, nn->z, &ctx->st->nn_s, ctx->st, GATE_ITER, cs, false, ctx->r32, nn->r_old));
+  SQCG_TRY(launch_finish2(ctx, grid_for(Vh, 32), FIN_FCG_BETA, GATE_ITER, cs, pdl));
+  SQCG_CUDA_TRY(launch_kernel(k_fcg_xpay, blas_grid(ctx), kRedThreads, 0, cs, pdl, nn->z, ctx->p32, 3 * Vh, ctx->st));
   return SQCG_OK;
 }
 
@@ -1648,22 +1658,29 @@ extern "C" int sqcg_fcg_solve_nn(sqcg_ctx* ctx, sqcg_nn* nn, double mass, const 
     status = h->status;  // x0 solves the system, or a non-finite start
     rel = sqrt(h->rr_true / h->bb);
   } else {
-    // z0 = N(r0); p0 = z0; <z0, r0> (first of the two sums of k_fcg_dots)
+    // z0 = N(r0); p0 = z0; <z0, r0> (first of the last layer's two sums)
     const int grid = blas_grid(ctx);
-    SQCG_TRY(fcg_precondition(nn, GATE_ITER, s));
-    k_fcg_dots<<<grid, kRedThreads, 0, s>>>(nn->z, ctx->r32, ctx->r32, Vh, ctx->st, ctx->partials);
+    k_norm_gated<<<grid, kRedThreads, 0, s>>>(ctx->r32, Vh, ctx->st, ctx->partials);
     SQCG_CUDA_TRY(cudaGetLastError());
-    SQCG_TRY(launch_finish(ctx, grid, FIN_FCG_INIT, GATE_ITER, s));
+    SQCG_TRY(launch_finish(ctx, grid, FIN_NN_SCALE, GATE_ITER, s));
+    SQCG_TRY(nn_forward_infer(nn, ctx->r32, nn->z, &ctx->st->nn_s, ctx->st, GATE_ITER, s, false, ctx->r32, ctx->r32));
+    SQCG_TRY(launch_finish(ctx, grid_for(Vh, 32), FIN_FCG_INIT, GATE_ITER, s));
     k_copy2<<<nn_grid(3 * Vh), kThreads, 0, s>>>(nn->z, ctx->p32, 3 * Vh);
     SQCG_CUDA_TRY(cudaGetLastError());
-    launches += 8;
+    launches += 7;
     const char* mode = getenv("SQCG_LAUNCH_MODE");
     const bool eager = mode && strcmp(mode, "eager") == 0;
     if (!eager && (!nn->fcg_exec || nn->fcg_b != b || nn->fcg_x != x || nn->fcg_gen != ctx->links_gen)) {
       SQCG_CUDA_TRY(cudaStreamSynchronize(s));
       if (nn->fcg_exec) cudaGraphExecDestroy(nn->fcg_exec);
       nn->fcg_exec = nullptr;
-      SQCG_TRY(fcg_graph(nn, b, x, &nn->fcg_exec, &nn->fcg_hw, &nn->fcg_hif));
+      int rc = fcg_graph(nn, b, x, &nn->fcg_exec, &nn->fcg_hw, &nn->fcg_hif);
+      if (rc == SQCG_ERR_CUDA && ctx->pdl) {  // a driver without programmatic edges in conditional nodes: plain edges
+        cudaGetLastError();
+        ctx->pdl = 0;
+        rc = fcg_graph(nn, b, x, &nn->fcg_exec, &nn->fcg_hw, &nn->fcg_hif);
+      }
+      SQCG_TRY(rc);
       nn->fcg_b = b;
       nn->fcg_x = x;
       nn->fcg_gen = ctx->links_gen;
@@ -1686,7 +1703,7 @@ extern "C" int sqcg_fcg_solve_nn(sqcg_ctx* ctx, sqcg_nn* nn, double mass, const 
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) { sqcg_set_last_cuda_error(e, "flexible CG", __FILE__, __LINE__); return SQCG_ERR_CUDA; }
     }
-    launches += h->loop_count * 14 + h->updates * 3;
+    launches += h->loop_count * 11 + h->updates * 3;
     iters = h->iter;
     updates = h->updates;
     status = h->done ? h->status : SQCG_ERR_NOT_CONVERGED;

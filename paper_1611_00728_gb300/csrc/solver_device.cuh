@@ -65,6 +65,18 @@ __device__ __forceinline__ double block_sum(double v) {
   return v;
 }
 
+// Two FP64 sums over SUB consecutive lanes (SUB <= 32) with the additions of one: the lower half of the lanes goes
+// on with a, the upper half with b. Totals: a in the first lane, b in lane SUB / 2. (An FP64 addition holds its
+// scheduler for 64 cycles on this GPU, whatever the lanes in it.)
+template <int SUB>
+__device__ __forceinline__ double sum2(double a, double b) {
+  const bool upper = (threadIdx.x + threadIdx.y * blockDim.x) & (SUB / 2);
+  double v = (upper ? b : a) + __shfl_xor_sync(0xffffffffu, upper ? a : b, SUB / 2);
+#pragma unroll
+  for (int o = SUB / 4; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o, SUB / 2);
+  return v;
+}
+
 // ---------------------------------------------------------------------------
 // scalar steps (run by thread 0 of the finisher, after the partials are summed;
 // the multi-shift steps run on the whole block, see solver_finish_ms)
@@ -73,6 +85,12 @@ __device__ __forceinline__ void finish_breakdown(SolverState* s) {
   s->status = SQCG_ERR_BREAKDOWN;
   s->done = 1;
   s->need_update = 0;
+}
+
+// scale of the network's input to unit RMS: v = |r|^2
+__device__ __forceinline__ void nn_scale(SolverState* s, double v) {
+  s->nn_s = sqrt(3.0 * (double)s->vh / v);
+  s->nn_inv_s = 1.0 / s->nn_s;
 }
 
 __device__ inline void solver_finish(SolverState* s, int fin, double v) {
@@ -112,6 +130,7 @@ __device__ inline void solver_finish(SolverState* s, int fin, double v) {
       }
       if (s->iter >= s->max_iter) s->need_update = 1;  // final true residual, then stop
       if (s->use_if) cudaGraphSetConditional((cudaGraphConditionalHandle)s->h_if, s->need_update ? 1u : 0u);
+      if (s->vh && !s->need_update) nn_scale(s, v);  // flexible CG: r goes into the network next
       break;
     }
     case FIN_TRUE_RESID: {  // r = b - A x recomputed in FP64 and copied to the working r
@@ -132,13 +151,13 @@ __device__ inline void solver_finish(SolverState* s, int fin, double v) {
       } else {
         s->beta = v / s->rr_prev;  // continue from the true residual
         s->rr = v;
+        if (s->vh) nn_scale(s, v);
       }
       break;
     }
     case FIN_NN_SCALE:  // |r|^2 of the network input
       if (!(v > 0.0) || !isfinite(v)) { finish_breakdown(s); s->nn_s = s->nn_inv_s = 0.0; break; }
-      s->nn_s = sqrt(3.0 * (double)s->vh / v);
-      s->nn_inv_s = 1.0 / s->nn_s;
+      nn_scale(s, v);
       break;
     case FIN_FCG_PAP:  // alpha = <z_k, r_k> / <p_k, A p_k>
       s->pAp = v;

@@ -310,7 +310,7 @@ int launch_finish_ffs(sqcg_ctx* ctx, int nblocks, int fin, int gate, cudaStream_
 // which runs iterations until the state asks for a reliable update or the solve ends
 int persistent_grid(sqcg_ctx* ctx);
 int launch_sr_persistent(sqcg_ctx* ctx, int max_steps, cudaStream_t s);
-int launch_finish2(sqcg_ctx* ctx, int nblocks, int fin, int gate, cudaStream_t s);
+int launch_finish2(sqcg_ctx* ctx, int nblocks, int fin, int gate, cudaStream_t s, bool pdl = false);
 // the single-reduction step's finisher: sums <r,s> = partials[0, n), <r,q> = partials[coff, coff + cn),
 // |r|^2 = partials[2n, 3n)
 int launch_finish_sr(sqcg_ctx* ctx, int nblocks, int coff, int cn, int gate, cudaStream_t s, bool pdl = false);

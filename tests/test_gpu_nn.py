@@ -384,3 +384,33 @@ def test_gradient_at_remainders_of_its_chunks(sqcg, links_cache, L, norm):
     assert abs(loss - want_l) <= 1e-4 * abs(want_l)
     assert rel(grad, params_to_flat(want_g)) <= 1e-4
     assert again[0] == loss and np.array_equal(again[1], grad)
+
+
+@pytest.mark.parametrize("mixing", ["FP32", "BF16"])
+@pytest.mark.parametrize("L", [(6, 6, 6, 6), (4, 6, 6, 10)])
+def test_network_and_fcg_at_remainders_of_their_blocks(sqcg, links_cache, L, mixing):
+    """Sites that fill no whole number of 32-site blocks (648 and 720 a parity): the layers against the oracle at
+    1e-5 (FP32 mixing), and the flexible CG, whose dot products the last layer forms, to its tolerance on the FP64
+    residual without falling back."""
+    fat, lng = links_cache(L, 71)
+    r = to_f32(synth.gaussian_source(L, 72))
+    with sqcg.Lattice(L) as lat:
+        lat.load_links(fat, lng)
+        net = sqcg.Network(lat)
+        net.set_params(params_to_flat(onn.init_params(5, scale=0.6)))
+        net.set_mixing(getattr(sqcg, "NN_MIX_" + mixing))
+        if mixing == "FP32":
+            z = net.apply(lat.pack(r, sqcg.F32), lat.new_spinor(sqcg.F32))
+            want = onn.apply(L, fat, flat_to_params(net.get_params(bf16_rounded=True)), r)
+            assert rel(lat.unpack(z, sqcg.F32), want) <= 1e-5
+        d = onn.init_params(5, scale=0.0)  # open gates and self taps only: N(r) is r, and the solve plain CG
+        d["gates"] = [(np.zeros(8), np.full(8, 20.0))] * 2
+        d["W"][0][0] += 1.0
+        d["W"][1][0] += np.eye(8)
+        d["W"][2][0] += 0.125
+        net.set_params(params_to_flat(d))
+        x = lat.new_spinor()
+        info = net.fcg_solve(0.2, lat.pack(r), x, tol=1e-9, max_iter=2000)
+        assert info.status == 0 and not info.fallback
+        assert oracle.true_rel_residual(L, fat, lng, 0.16, r, lat.unpack(x)) <= 1e-9
+        net.close()
