@@ -200,7 +200,9 @@ template <int OUT>
 __global__ void __launch_bounds__(kHopThreads, 5) k_conv_1to8(ConvArgs a) {
   pdl_wait();
   pdl_launch_dependents();
-  if (a.st && !gate_open(a.st, a.gate)) return;
+  const int gate = a.st ? a.gate : GATE_NONE;
+  const GateWords gw = gate_load(a.st, gate, threadIdx.x == 0);  // in flight while the block loads
+  __shared__ int open;
   constexpr int TILES = OUT == OUT_GATE_BWD ? 2 : 1;
   __shared__ float2 t[NT][3][32];  // the even site's vector, the odd site's transported ones
   __shared__ float red[OUT == OUT_GATE_BWD ? 2 * CH : 1][64 * TILES + 1];
@@ -236,7 +238,9 @@ __global__ void __launch_bounds__(kHopThreads, 5) k_conv_1to8(ConvArgs a) {
 #pragma unroll
     for (int tap = 0; tap < NT; ++tap) w[tap] = __ldg(a.W + tap * CH + o);
     const float ga = a.gate_a[o], gb = a.gate_b[o];
+    if (threadIdx.x == 0) open = gate_value(gw, gate);
     __syncthreads();
+    if (!open) return;
 #pragma unroll
     for (int par = 0; par < 2; ++par) {
       float2 acc[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
@@ -284,7 +288,9 @@ __global__ void __launch_bounds__(kTapThreads, 4) k_conv_8to1(ConvArgs a) {
   __shared__ double dots[2][3];
   pdl_wait();
   pdl_launch_dependents();
-  if (a.st && !gate_open(a.st, a.gate)) return;
+  const int gate = a.st ? a.gate : GATE_NONE;
+  const GateWords gw = gate_load(a.st, gate, threadIdx.x == 0);  // in flight while the block loads
+  __shared__ int open;
   const Geom& g = a.g;
   const int Vh = g.Vh;
   const int lane = threadIdx.x & 31, hop = threadIdx.x >> 5;
@@ -313,7 +319,9 @@ __global__ void __launch_bounds__(kTapThreads, 4) k_conv_8to1(ConvArgs a) {
   }
 #pragma unroll
   for (int c = 0; c < 3; ++c) t[tap][c][lane] = m[c];
+  if (threadIdx.x == 0) open = gate_value(gw, gate);
   __syncthreads();
+  if (!open) return;
   const int c = hop;
   if (c < 3) {
     float2 z = t[0][c][lane];
@@ -354,7 +362,11 @@ __global__ void __launch_bounds__(kTapThreads, 4) k_conv_8to1(ConvArgs a) {
 // takes part in the shuffles.
 template <int OUT>
 __global__ void __launch_bounds__(kThreads, 5) k_conv88(ConvArgs a) {
+  pdl_wait();
   pdl_launch_dependents();
+  const int gate = a.st ? a.gate : GATE_NONE;
+  const GateWords gw = gate_load(a.st, gate, threadIdx.x == 0);  // in flight while the block loads
+  __shared__ int open;
   // weights as [tap][c_in][c_out], each complex w stored as (w.x, w.x, -w.y, w.y): the two packed
   // operands of acc += w t in two-lane FMAs, acc = (w.x, w.x) (t.x, t.y) + (-w.y, w.y) (t.y, t.x) + acc,
   // which rounds exactly as the scalar complex multiply-add (same products, same order per lane)
@@ -364,9 +376,9 @@ __global__ void __launch_bounds__(kThreads, 5) k_conv88(ConvArgs a) {
     const float2 w = a.W[j];
     W[(tap * CH + ci) * CH + o] = make_float4(w.x, w.x, -w.y, w.y);
   }
-  pdl_wait();
-  if (a.st && !gate_open(a.st, a.gate)) return;
+  if (threadIdx.x == 0) open = gate_value(gw, gate);
   __syncthreads();
+  if (!open) return;
   const Geom& g = a.g;
   const int Vh = g.Vh;
   const int gid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -519,7 +531,11 @@ __device__ __forceinline__ int tc_half(int row, int half) { return half ^ ((row 
 
 template <int OUT>
 __global__ void __launch_bounds__(kThreads, 3) k_conv88_tc(ConvArgs a) {
+  pdl_wait();
   pdl_launch_dependents();
+  const int gate = a.st ? a.gate : GATE_NONE;
+  const GateWords gw = gate_load(a.st, gate, threadIdx.x == 0);  // in flight while the block loads
+  __shared__ int open;
   constexpr int kWarps = kThreads / 32;
   // B fragments [tap][nt][half][lane]: rows k = 2 ci + comp (ci = t, t + 4 for half 0, 1), column n = g of
   // each 8-column half nt, i.e. output channel o = 4 nt + g / 2, component g % 2 (lane = 4 g + t)
@@ -532,9 +548,9 @@ __global__ void __launch_bounds__(kThreads, 3) k_conv88_tc(ConvArgs a) {
     // (re, im) input component -> output component oc: re: (w.x, -w.y); im: (w.y, w.x)
     sB[tap][nt][half][l] = oc == 0 ? pack_bf16(w.x, -w.y) : pack_bf16(w.y, w.x);
   }
-  pdl_wait();  // the weights were there before the kernel in front was launched
-  if (a.st && !gate_open(a.st, a.gate)) return;
+  if (threadIdx.x == 0) open = gate_value(gw, gate);
   __syncthreads();
+  if (!open) return;
   const Geom& g = a.g;
   const int Vh = g.Vh;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1026,8 +1042,7 @@ int conv_launch(sqcg_nn* nn, int layer, bool adjoint, int in_mode, int out_mode,
   return SQCG_OK;
 }
 
-// z = N(r) on the even sites (inference). scale[0] must hold s, scale[1] 1/s. pdl: a kernel is in front of it, and one
-// launched without programmatic dependent launch in front of that or nearer (the weights are read ahead of the wait).
+// z = N(r) on the even sites (inference). scale[0] must hold s, scale[1] 1/s. pdl: a kernel is in front of it.
 // dot_r: the sums of <z, dot_r>, then of <z, dot_o>, over blocks of 32 sites go to the context's partials.
 int nn_forward_infer(sqcg_nn* nn, const float2* r, float2* z, const double* scale, const SolverState* st, int gate,
                      cudaStream_t s, bool pdl, const float2* dot_r = nullptr, const float2* dot_o = nullptr) {
