@@ -132,7 +132,9 @@ int sqcg_create(const int dims[4], int flags, void* cuda_stream, sqcg_ctx** out)
 /* Free everything the context owns (device links, workspace, graphs). NULL is a no-op. */
 int sqcg_destroy(sqcg_ctx* ctx);
 
-/* Change the stream later calls queue their work on. */
+/* Change the stream later calls queue their work on. The calls of a context share its workspace: where some on the
+ * old stream may still be running, order the new one behind it. Only the loading of links (sqcg_load_links,
+ * sqcg_hisq_load_links) needs no such order: what earlier calls queued on any stream runs on the links of its time. */
 int sqcg_set_stream(sqcg_ctx* ctx, void* cuda_stream);
 
 /* Reliable-update trigger of the mixed-precision solvers on this context: the

@@ -144,6 +144,7 @@ int sqcg_destroy(sqcg_ctx* ctx) {
 
 int sqcg_set_stream(sqcg_ctx* ctx, void* cuda_stream) {
   if (!ctx) return SQCG_ERR_INVALID_ARG;
+  if (ctx->stream != (cudaStream_t)cuda_stream) ctx->streams_mixed = true;
   ctx->stream = (cudaStream_t)cuda_stream;
   return SQCG_OK;
 }

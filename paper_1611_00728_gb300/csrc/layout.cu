@@ -244,11 +244,15 @@ int recon_check(sqcg_ctx* ctx, const double2* lng, const double* first, double* 
   return h ? SQCG_ERR_RECON_REJECTED : SQCG_OK;
 }
 
-int ensure_stage(sqcg_ctx* ctx, size_t bytes) {
-  if (ctx->stage_bytes >= bytes) return SQCG_OK;
-  if (ctx->stage) cudaFree(ctx->stage);
+void free_stage(sqcg_ctx* ctx) {
+  cudaFree(ctx->stage);
   ctx->stage = nullptr;
   ctx->stage_bytes = 0;
+}
+
+int ensure_stage(sqcg_ctx* ctx, size_t bytes) {
+  if (ctx->stage_bytes >= bytes) return SQCG_OK;
+  free_stage(ctx);
   if (cudaMalloc(&ctx->stage, bytes) != cudaSuccess) {
     cudaGetLastError();
     return SQCG_ERR_NO_MEMORY;
@@ -297,7 +301,11 @@ int ensure_links(sqcg_ctx* ctx, int nl32, bool eightway) {
   return SQCG_OK;
 }
 
-// fat, lng: host order [V][4][3][3] complex, in host memory or (on_device) in device memory
+// fat, lng: host order [V][4][3][3] complex, in host memory or (on_device) in device memory.
+// What earlier calls queued on this stream is over before a kept array or the staging is written again. Work that
+// they left on another stream may still be reading: where the context has been on several, both are given back and
+// allocated anew instead (the runtime frees memory only once nothing on the device uses it; that also holds for
+// streams that are gone or being captured, which nothing here could wait for).
 int load_links(sqcg_ctx* ctx, const double* fat, const double* lng, int opts, bool on_device) {
   if (!fat || !lng) return SQCG_ERR_INVALID_ARG;
   if (opts & ~(SQCG_RECON12_LONG | SQCG_EIGHT_WAY)) return SQCG_ERR_INVALID_ARG;
@@ -312,6 +320,7 @@ int load_links(sqcg_ctx* ctx, const double* fat, const double* lng, int opts, bo
   void* raw = nullptr;
   if (!on_device) {
     if (bytes <= kKeptStage) {
+      if (ctx->streams_mixed) free_stage(ctx);
       SQCG_TRY(ensure_stage(ctx, bytes));
       raw = ctx->stage;
     } else if (cudaMalloc(&own, bytes) != cudaSuccess) {
@@ -354,6 +363,11 @@ int load_links(sqcg_ctx* ctx, const double* fat, const double* lng, int opts, bo
   ctx->have_links = false;
   free_graphs(ctx);
   free_batch_plan(ctx);
+  if (ctx->streams_mixed) {
+    free_links(ctx);
+    if (on_device) free_stage(ctx);  // host links: done above, or staged elsewhere
+    ctx->streams_mixed = false;
+  }
   if (rc == SQCG_OK) rc = ensure_links(ctx, nl32, eightway);
   const int fold = (ctx->flags & SQCG_PHASES_FOLDED) ? 0 : 1;
   const unsigned grid = (unsigned)((V + kPackSites - 1) / kPackSites);

@@ -169,6 +169,7 @@ struct sqcg_ctx {
   int flags;
   Geom g;
   cudaStream_t stream;
+  bool streams_mixed;       // calls have gone to another stream since the links were loaded (see load_links)
   cudaStream_t cap_stream;  // private stream used only to capture graphs
   int nsm;                  // SMs of the device the context was created on
 

@@ -10,6 +10,7 @@ the oracle computes one by one, plus the free-field closed form at every site.
 
 import numpy as np
 import pytest
+import torch
 
 import oracle
 import synth
@@ -299,3 +300,36 @@ def test_links_reloaded_in_other_forms(sqcg, links_cache):
                     lat.dslash(par, lat.pack(psi, prec), out, prec)
                     want = oracle.dslash(L, fat, lng, psi, par)
                     assert rel(lat.unpack(out, prec), want) <= bar, (k, prec, par)
+
+
+@pytest.mark.parametrize("recon", [False, True])
+def test_links_reloaded_behind_work_on_another_stream(sqcg, links_cache, recon):
+    """Operators and a pack that wait on a side stream while the default stream loads other links of the same form,
+    whose arrays and staging are kept: they run on the links and the vector of their time. The side stream is held
+    back by a tenth of a second, the packed vector is pinned, so that nothing of it has run when the loading starts."""
+    L = (6, 8, 10, 12)
+    old, new = links_cache(L, 1005), links_cache(L, 1006)
+    psi = synth.gaussian_source(L, 2007)
+    pinned = torch.from_numpy(synth.gaussian_source(L, 2008).view(np.float64)).pin_memory().numpy().view(np.complex128)
+    side = torch.cuda.Stream()
+    with sqcg.Lattice(L) as lat:
+        lat.load_links(*old, recon12=recon)
+        vecs = {prec: lat.pack(psi, prec) for prec in (0, 1)}
+        outs = {prec: [lat.new_spinor(prec) for _ in range(20)] for prec in (0, 1)}
+        packed = lat.new_spinor()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(200_000_000)
+            lat.pack(pinned, out=packed)
+            for prec in (0, 1):
+                for out in outs[prec]:
+                    lat.normal_op(0.04, vecs[prec], out, prec)
+        lat.load_links(*new, recon12=recon)
+        side.synchronize()
+        want, want_new = (oracle.normal_op(L, *links, 0.04, psi) for links in (old, new))
+        assert np.array_equal(lat.unpack(packed), pinned)
+        for prec in (0, 1):
+            for out in outs[prec]:
+                assert rel(lat.unpack(out, prec), want) <= TOL[prec]
+            lat.normal_op(0.04, vecs[prec], outs[prec][0], prec)
+            assert rel(lat.unpack(outs[prec][0], prec), want_new) <= TOL[prec]
