@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(kCheckThreads) k_recon_check(const double2* __
     det.y += d.y;
   }
   const double s = cbrt(det.x), s2 = s * s;
+  const bool far = !(s2 > 1e-100 && s2 < 1e100);  // squares of the products below may leave the range of FP64
   bool ok = fabs(s) > 0.0 && isfinite(s) && fabs(det.y) <= 1e-12 * fabs(s2 * s);
 #pragma unroll
   for (int a = 0; a < 3; ++a)
@@ -101,7 +102,7 @@ __global__ void __launch_bounds__(kCheckThreads) k_recon_check(const double2* __
         re += u.x * v.x + u.y * v.y;
         im += u.y * v.x - u.x * v.y;
       }
-      ok = ok && re * re + im * im <= 1e-24 * s2 * s2;  // false for a NaN
+      ok = ok && (far ? hypot(re, im) <= 1e-12 * s2 : re * re + im * im <= 1e-24 * s2 * s2);  // false for a NaN
     }
   double f = 1.0;
   if (folded) {

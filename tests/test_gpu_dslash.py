@@ -284,6 +284,23 @@ def test_recon12_check_finds_one_link(sqcg, links_cache, where, folded):
             lat.load_links(fat, changed(kind, 1e-14), recon12=True)
 
 
+@pytest.mark.parametrize("power", [-300, 300])
+def test_recon12_check_at_the_ends_of_the_range(sqcg, links_cache, power):
+    """Long links scaled so far that the squares of their products leave the range of FP64 (their determinants do
+    not): a link whose rows are not of one length, with the determinant of the others, is refused, the links themselves
+    pass."""
+    L = (4, 4, 4, 4)
+    fat, lng = links_cache(L, 1005)
+    lng = lng * 2.0 ** power
+    bad = lng.copy()
+    bad[5, 1] *= np.array([1 + 1e-6, 1 / (1 + 1e-6), 1])[:, None]
+    with sqcg.Lattice(L) as lat:
+        lat.load_links(fat, lng, recon12=True)
+        with pytest.raises(sqcg.SqcgError) as err:
+            lat.load_links(fat, bad, recon12=True)
+        assert err.value.name == "RECON_REJECTED"
+
+
 def test_links_reloaded_in_other_forms(sqcg, links_cache):
     """Links loaded again and again into one context, with other values and in every storage form (arrays of the same
     size are used again), on a lattice whose last 32-site block is half filled."""
