@@ -400,9 +400,8 @@ int run_persistent(sqcg_ctx* ctx, const void* b, void* x, double tol, int max_it
   h->use_if = 0;
   SQCG_TRY(write_state(ctx, s));
   *segments = 0;
-  int queue = tol < 1.0 ? (int)ceil(log(tol) / log(ctx->ru_delta)) : 1;
-  if (queue < 1) queue = 1;
-  if (queue > 8) queue = 8;
+  const double falls = tol < 1.0 ? log(tol) / log(ctx->ru_delta) : 1.0;  // huge where the factor is next to 1
+  int queue = falls > 8.0 ? 8 : falls > 1.0 ? (int)ceil(falls) : 1;
   while (*segments < max_iter + 4) {
     for (int k = 0; k < queue; ++k) {
       SQCG_TRY(launch_sr_persistent(ctx, max_iter + 2, s));

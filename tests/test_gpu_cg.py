@@ -390,6 +390,21 @@ def test_reliable_update_settings(sqcg, links_cache, delta, interval):
 
 
 
+def test_reliable_update_factor_next_to_one(sqcg, links_cache):
+    """The largest factor the trigger takes: the segments that the persistent loop queues at once are bounded, whatever
+    the quotient of the logarithms."""
+    L, m, tol = (8, 8, 8, 8), 0.1, 1e-9
+    fat, lng = links_cache(L, 1001)
+    b = synth.gaussian_source(L, 2702)
+    with sqcg.Lattice(L) as lat:
+        lat.load_links(fat, lng)
+        lat.set_reliable_update(float(np.nextafter(1.0, 0.0)), 100)
+        x = lat.new_spinor()
+        info = lat.cg_solve(m, lat.pack(b), x, tol=tol, max_iter=5000, mode=sqcg.MODE_MIXED)
+        assert info.status == 0 and info.launches <= 5 * (info.reliable_updates + 8) + 10
+        assert oracle.true_rel_residual(L, fat, lng, 4 * m * m, b, lat.unpack(x)) <= tol
+
+
 @pytest.mark.parametrize("mode", [0, 1])
 def test_rational_apply_matches_oracle(sqcg, links_cache, mode):
     """RHMC use of the multi-mass CG: a0 b + sum_s a_s (sigma_s - D_eo D_oe)^-1 b with 9 poles."""
