@@ -294,8 +294,9 @@ int sqcg_rational_apply(sqcg_ctx* ctx, int nshift, const double* shifts, const d
  * the site-block size, the warp shape and the shared-memory carveout are picked on the first
  * call for a given set of lattices by timing the multi-RHS Dslash (cached per
  * process, and in the file named by the environment variable SQCG_TUNE_CACHE
- * if set; SQCG_TUNE_VERBOSE=1 prints each timed candidate to stderr), unless
- * sqcg_batched_pin_tuning has fixed them.
+ * if set, where another build's choices are left alone; SQCG_TUNE_VERBOSE=1
+ * prints each timed candidate to stderr), unless sqcg_batched_pin_tuning has
+ * fixed them.
  * ctx[k]: distinct contexts with links loaded, all on the current device; the
  * work runs on ctx[0]'s stream. b[k], x[k]: device arrays of nrhs[k]
  * consecutive FP64 device vectors ([nrhs][3][Vh] complex double); x[k] holds

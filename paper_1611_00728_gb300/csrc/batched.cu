@@ -1367,9 +1367,12 @@ void tune_file_store(const std::string& key, const TuneChoice& c) {
   fclose(f);
 }
 
+// What a choice was timed on: the kernels and candidates (the number, which goes up with them, so that an older file's
+// choices are not taken for this build's), the SMs, and the batch.
 std::string tune_key(const BatchPlan& P) {
-  std::string k = "mrhs_dslash_smem_f32";
   char buf[128];
+  snprintf(buf, sizeof(buf), "mrhs_dslash_f32.2:%dsm", P.ctx[0]->nsm);
+  std::string k = buf;
   for (int j = 0; j < P.nlat; ++j) {
     const Geom& g = P.host[j].g;
     snprintf(buf, sizeof(buf), ":%dx%dx%dx%d/r%d/n%d", g.Lx, g.Ly, g.Lz, g.Lt, P.host[j].recon, P.nrhs[j]);

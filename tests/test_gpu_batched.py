@@ -7,6 +7,10 @@ the single-RHS solver. The full batched workload (16 sources each on 16^4,
 every one of its 48 solutions.
 """
 
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -310,3 +314,30 @@ def test_batched_hops_split_over_warps(sqcg, links_cache, W, nrhs, recon):
                 assert oracle.true_rel_residual(L, *links[n], 4 * m * m, srcs[n][j], lats[n].unpack(xs[n][j])) <= tol
             lats[n].close()
     assert all(a <= 1.1 * b + 5 for a, b in zip(iters[4], iters[32]))
+
+
+def test_tuning_file_of_an_older_build_is_not_taken(sqcg, tmp_path):
+    """A tuning file's choice holds for the kernels that it was timed on: a line of the build before the hop-split
+    kernel does not keep a single right-hand side on the staged one, and the choice made instead is what the next
+    process takes from the file, unchanged. (A process each: the file is read once in one.)"""
+    path = tmp_path / "tune.txt"
+    path.write_text("mrhs_dslash_smem_f32:16x16x16x16/r0/n1 16 1 32 75 32\n")
+    code = """
+import sys, torch, synth
+import paper_1611_00728_gb300 as sq
+L = (16, 16, 16, 16)
+with sq.Lattice(L) as lat:
+    lat.load_links(*synth.fat_long_links(L, 1001))
+    b = torch.stack([lat.pack(synth.gaussian_source(L, 1))])
+    sq.cg_solve_batched([lat], [0.5], [b], [torch.zeros_like(b)], tol=1e-3)
+    print("choice", *sq.batched_tuning_ex(lat).values())
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    choice = []
+    for _ in range(2):
+        out = subprocess.run([sys.executable, "-c", code], cwd=root, env={**os.environ, "SQCG_TUNE_CACHE": str(path)},
+                             capture_output=True, text=True, timeout=300)
+        assert out.returncode == 0, out.stderr
+        choice.append(out.stdout.split("choice", 1)[1].split())
+    assert choice[0] != ["16", "1", "32", "75", "32"] and choice[1] == choice[0]
+    assert len(path.read_text().splitlines()) == 2
