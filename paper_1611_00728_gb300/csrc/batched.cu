@@ -215,8 +215,10 @@ __device__ void rhs_block_partial(double (&v)[WT], const LatDev& L, int wbase, i
   }
 }
 
-// Which RHS blocks need the reliable update -> IF condition; run by a whole block, a thread per RHS block.
+// Which RHS blocks need the reliable update -> IF condition; run by a whole block, a thread per RHS block. Where
+// some do, also the list of the float-float passes' blocks that hold one.
 __device__ void update_control(BatchState* st, const LatDev* lats, int nlat, int W) {
+  __shared__ unsigned char asked[SQCG_MAX_BATCH_RHS];
   int any = 0;
   for (int b = threadIdx.x; b < st->nblk; b += blockDim.x) {
     int k = 0;
@@ -233,6 +235,30 @@ __device__ void update_control(BatchState* st, const LatDev* lats, int nlat, int
   if (threadIdx.x == 0) {
     st->if_runs += any ? 1 : 0;
     if (st->use_graph) cudaGraphSetConditional((cudaGraphConditionalHandle)st->h_if, any ? 1u : 0u);
+  }
+  if (!any) return;
+  const int W64 = min(W, kW64);
+  const int n64 = lats[nlat - 1].rb640 + lats[nlat - 1].nrb64;
+  for (int b = threadIdx.x; b < n64; b += blockDim.x) {
+    int k = 0;
+    for (int j = 1; j < nlat; ++j)
+      if (b >= lats[j].rb640) k = j;
+    const LatDev& L = lats[k];
+    const int w0 = (b - L.rb640) * W64;
+    int u = 0;
+    for (int w = w0; w < min(w0 + W64, L.nrhs); ++w) {
+      const volatile RhsScalars& r = st->r[L.rhs0 + w];
+      u |= r.need_update && r.active;
+    }
+    asked[b] = u;
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < nlat; k += blockDim.x) {
+    const LatDev& L = lats[k];
+    int n = 0;
+    for (int rb = 0; rb < L.nrb64; ++rb)
+      if (asked[L.rb640 + rb]) st->ff_blk[L.rb640 + n++] = rb;
+    st->ff_n[k] = n;
   }
 }
 
@@ -576,16 +602,22 @@ __global__ void __launch_bounds__(128, 6) k_mrhs_dslash_ff(MArgs a) {
   const int k = have_tile ? find_lat(a.lats, a.nlat, tile, true) : 0;
   const LatDev& L = a.lats[k];
   const int local = tile - L.tile640;
-  // site blocks fastest: the slices of a CTA have the same right-hand sides, so in an update of a few of them whole
-  // CTAs have nothing to do (with RHS blocks fastest two thirds of every CTA idled in an 11-RHS solve: 421 us a pass
-  // for one right-hand side at 32^4, 254 now)
-  const int rb = have_tile ? local / L.nsb : 0, sb = have_tile ? local % L.nsb : 0;
+  // The tiles of a lattice are its site blocks times the RHS blocks that run (an update: those that asked), those of a
+  // site block side by side, so that its links come once from HBM; the tiles left over are whole CTAs with nothing to
+  // do. All RHS blocks side by side left two thirds of every CTA idle where one of eleven right-hand sides asked (421
+  // us a pass at 32^4, 254 so); one RHS block after the other reads the links once for each. The three orders, this one
+  // last: 16 sources on 16^4 and 32^4 to 1e-8 251.1 / 257.1 / 251.4 ms, 16 on each of 16^4, 24^4 and 32^3x64 795.8 /
+  // 798.3 / 789.1, 12 at 32^4 193.6 / 194.7 / 192.0, the refinement of 11 shifts at 32^4 to 1e-11 (whole solve, in
+  // the last two) 157.8 / 156.7.
+  const bool upd = a.gate == GATE_UPDATE;
+  const int nblk = upd ? a.st->ff_n[k] : L.nrb64;
+  const bool run = have_tile && local < L.nsb * nblk;
+  const int at = run ? local % nblk : 0, sb = run ? local / nblk : 0;
+  const int rb = upd && run ? a.st->ff_blk[L.rb640 + at] : at;
   const int wbase = rb * WT;
-  const int nw_tile = have_tile ? min(WT, L.nrhs - wbase) : 0;
+  const int nw_tile = run ? min(WT, L.nrhs - wbase) : 0;
   const int w0 = wbase;
-  const int nw = have_tile ? max(0, min(WT, L.nrhs - w0)) : 0;
-  const int blk = L.rb0 + wbase / a.W;
-  bool run = have_tile && !(a.gate == GATE_UPDATE && !a.st->blk_update[blk]);
+  const int nw = run ? max(0, min(WT, L.nrhs - w0)) : 0;
   const Geom& g = L.g;
   const int Vh = g.Vh;
   const int i = sb * blockDim.x + threadIdx.x;

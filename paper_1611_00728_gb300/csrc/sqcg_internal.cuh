@@ -131,6 +131,8 @@ struct BatchState {
   RhsScalars r[SQCG_MAX_BATCH_RHS];
   int blk_active[SQCG_MAX_BATCH_RHS];  // RHS block has an active RHS
   int blk_update[SQCG_MAX_BATCH_RHS];  // RHS block runs the FP64 reliable update
+  int ff_n[SQCG_MAX_LATTICES];     // of a lattice's RHS blocks of the float-float passes, how many run the update ...
+  int ff_blk[SQCG_MAX_BATCH_RHS];  // ... and which, from the lattice's rb640 on
 };
 
 struct BatchPlan;  // defined in batched.cu

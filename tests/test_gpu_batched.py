@@ -316,6 +316,37 @@ def test_batched_hops_split_over_warps(sqcg, links_cache, W, nrhs, recon):
     assert all(a <= 1.1 * b + 5 for a, b in zip(iters[4], iters[32]))
 
 
+@pytest.mark.parametrize("nrhs", [(11, 3), (4, 9), (1, 6)])
+def test_batched_updates_of_some_right_hand_sides(sqcg, links_cache, nrhs):
+    """Reliable updates that some of the right-hand sides ask for, at different times on two lattices whose blocks of
+    the float-float passes are full, ragged or single: point, Gaussian and smoothed sources fall at different rates, and
+    each ends on the oracle's residual."""
+    m, tol = 0.1, 1e-9
+    lats, bs, xs, srcs, links = [], [], [], [], []
+    for k, (L, n) in enumerate(zip(((8, 8, 8, 8), (6, 8, 10, 12)), nrhs)):
+        fat, lng = links_cache(L, 400 + k)
+        lat = sqcg.Lattice(L)
+        lat.load_links(fat, lng)
+        s = []
+        for j in range(n):
+            v = synth.gaussian_source(L, 5500 + 20 * k + j)
+            if j % 3 == 1:
+                v = np.where(np.arange(v.shape[0])[:, None] == 7 * j, v, 0)
+            if j % 3 == 2:
+                for _ in range(2 * j):
+                    v = 8.0 * v - oracle.normal_op(L, fat, lng, 0.0, v)
+            s.append(v)
+        b, x = make_batch(sqcg, lat, s)
+        lats.append(lat); bs.append(b); xs.append(x); srcs.append(s); links.append((L, fat, lng))
+    infos = sqcg.cg_solve_batched(lats, [m, m], bs, xs, tol=tol, max_iter=5000)
+    assert max(nrhs) < 3 or len({(i.iters, i.reliable_updates) for r in infos for i in r}) > 2
+    for k, (L, fat, lng) in enumerate(links):
+        for j, s in enumerate(srcs[k]):
+            assert infos[k][j].status == 0
+            assert oracle.true_rel_residual(L, fat, lng, 4 * m * m, s, lats[k].unpack(xs[k][j])) <= tol
+        lats[k].close()
+
+
 def test_tuning_file_of_an_older_build_is_not_taken(sqcg, tmp_path):
     """A tuning file's choice holds for the kernels that it was timed on: a line of the build before the hop-split
     kernel does not keep a single right-hand side on the staged one, and the choice made instead is what the next
