@@ -185,3 +185,21 @@ def test_binding_network_layout_matches_the_library(libpath):
         covered[ga] += 1
         covered[gb] += 1
     assert np.all(covered == 1)
+
+
+@pytest.mark.parametrize("missing", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
+def test_binding_finds_the_stream_without_torch_internals(monkeypatch, missing):
+    """The stream's handle comes from names that torch does not publish, and from its public call where a release has
+    no such name."""
+    import types
+
+    import paper_1611_00728_gb300 as sq
+
+    internal = {"_cuda_getCurrentRawStream": lambda dev: 100 + dev, "_cuda_getDevice": lambda: 3}
+    fake = types.SimpleNamespace(
+        _C=types.SimpleNamespace(**internal),
+        cuda=types.SimpleNamespace(current_stream=lambda: types.SimpleNamespace(cuda_stream=77)))
+    monkeypatch.setattr(sq, "_torch_module", fake)
+    assert sq._current_stream() == 103
+    delattr(fake._C, missing)
+    assert sq._current_stream() == 77
