@@ -735,7 +735,9 @@ extern "C" int sqcg_multishift_cg_solve(sqcg_ctx* ctx, int nshift, const double*
     ctx->ms_nalloc = nshift;
     ctx->ms_prec = mixed;
     ctx->ms_unroll = 1;
-    if (mixed) {  // without room for it the loop applies every step by itself
+    // without room for it the loop applies every step by itself (SQCG_TEST_MS_NO_RING=1: as if there were none)
+    const char* no_ring = getenv("SQCG_TEST_MS_NO_RING");
+    if (mixed && !(no_ring && strcmp(no_ring, "1") == 0)) {
       if (cudaMalloc(&ctx->ms_ring, kMSUnroll * wbytes) == cudaSuccess) ctx->ms_unroll = kMSUnroll;
       else { cudaGetLastError(); ctx->ms_ring = nullptr; }
     }

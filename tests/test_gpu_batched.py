@@ -372,3 +372,30 @@ with sq.Lattice(L) as lat:
         choice.append(out.stdout.split("choice", 1)[1].split())
     assert choice[0] != ["16", "1", "32", "75", "32"] and choice[1] == choice[0]
     assert len(path.read_text().splitlines()) == 2
+
+
+@pytest.mark.parametrize("cfg", [(8, 2, 64, 16), (4, 4, 32, 4)])
+def test_batched_programmatic_dependent_launch_changes_nothing(sqcg, links_cache, monkeypatch, cfg):
+    """The batched loop with and without programmatic dependent launch, staged and hop-split: the same bits."""
+    W, WT, T, ws = cfg
+    specs = [((8, 8, 8, 8), 5, 0.1), ((6, 8, 10, 12), 3, 0.05)]
+    out = []
+    sqcg.pin_batched_tuning(W, WT, T, -1, ws)
+    try:
+        for pdl in ("1", "0"):
+            monkeypatch.setenv("SQCG_PDL", pdl)
+            lats, bs, xs = [], [], []
+            for n, (L, nr, m) in enumerate(specs):
+                fat, lng = links_cache(L, 420 + n)
+                lat = sqcg.Lattice(L)
+                lat.load_links(fat, lng, recon12=n == 1)
+                b, x = make_batch(sqcg, lat, [synth.gaussian_source(L, 5300 + 10 * n + j) for j in range(nr)])
+                lats.append(lat); bs.append(b); xs.append(x)
+            infos = sqcg.cg_solve_batched(lats, [m for _, _, m in specs], bs, xs, tol=1e-9, max_iter=5000)
+            out.append(([x.cpu().numpy() for x in xs], [(i.status, i.iters) for r in infos for i in r]))
+            for lat in lats:
+                lat.close()
+    finally:
+        sqcg.pin_batched_tuning(0)
+    assert out[0][1] == out[1][1]
+    assert all(np.array_equal(a, b) for a, b in zip(out[0][0], out[1][0]))

@@ -804,3 +804,27 @@ def test_multishift_passes_that_end_early(sqcg, links_cache, flags, nshift, tol)
             assert infos[j].status == 0
             assert oracle.true_rel_residual(L, fat, lng, s, src, lat.unpack(xs[j])) <= tol
             assert infos[j].iters <= 1.1 * ref[j].iters + 5
+
+
+@pytest.mark.parametrize("flags", ["", "MS_SHIFT_RU", "MS_NO_RU"])
+@pytest.mark.parametrize("eager", [False, True])
+def test_multishift_without_room_for_passes(sqcg, links_cache, monkeypatch, flags, eager):
+    """Where the residuals of a pass of several steps find no memory, every step applies its updates by itself: the
+    same operations in the same order, so the same solutions bit for bit."""
+    L, tol = (6, 6, 6, 10), 1e-7
+    fat, lng = links_cache(L, 680)
+    shifts = np.logspace(-2, 0, 5).tolist()
+    src = synth.gaussian_source(L, 7900)
+    if eager:
+        monkeypatch.setenv("SQCG_LAUNCH_MODE", "eager")
+    out = []
+    for no_ring in ("0", "1"):
+        monkeypatch.setenv("SQCG_TEST_MS_NO_RING", no_ring)
+        with sqcg.Lattice(L) as lat:
+            lat.load_links(fat, lng)
+            xs = [lat.new_spinor() for _ in shifts]
+            infos = lat.multishift_cg_solve(shifts, lat.pack(src), xs, tol=tol,
+                                            mode=sqcg.MODE_MIXED | (getattr(sqcg, flags) if flags else 0))
+            out.append(([i.iters for i in infos], [lat.unpack(x) for x in xs]))
+    assert out[0][0] == out[1][0]
+    assert all(np.array_equal(u, v) for u, v in zip(out[0][1], out[1][1]))

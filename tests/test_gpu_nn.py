@@ -414,3 +414,32 @@ def test_network_and_fcg_at_remainders_of_their_blocks(sqcg, links_cache, L, mix
         assert info.status == 0 and not info.fallback
         assert oracle.true_rel_residual(L, fat, lng, 0.16, r, lat.unpack(x)) <= 1e-9
         net.close()
+
+
+@pytest.mark.parametrize("mixing", ["NN_MIX_FP32", "NN_MIX_BF16"])
+def test_network_programmatic_dependent_launch_changes_nothing(sqcg, links_cache, monkeypatch, mixing):
+    """The network alone, its gradient and the flexible CG, with and without programmatic dependent launch: the same
+    bits. Two applications follow one another without a wait, the second over the first's activations."""
+    L, m, tol = (8, 10, 12, 14), 0.05, 1e-8
+    fat, lng = links_cache(L, 62)
+    r, e, b = (synth.gaussian_source(L, 93 + k) for k in range(3))
+    d = onn.init_params(8, scale=0.02)
+    for w in d["W"]:
+        w[0, 0, 0] += 1.0
+    d["gates"] = [(np.zeros(8), np.full(8, 10.0)), (np.zeros(8), np.full(8, 10.0))]
+    out = []
+    for pdl in ("1", "0"):
+        monkeypatch.setenv("SQCG_PDL", pdl)
+        with sqcg.Lattice(L) as lat:
+            lat.load_links(fat, lng)
+            net = sqcg.Network(lat)
+            net.set_params(params_to_flat(d))
+            net.set_mixing(getattr(sqcg, mixing))
+            dr, de = lat.pack(r, sqcg.F32), lat.pack(e, sqcg.F32)
+            z = [net.apply(v, lat.new_spinor(sqcg.F32)) for v in (dr, de)]
+            loss, grad = net.loss_grad(0.05, dr, de)
+            x = lat.new_spinor()
+            info = net.fcg_solve(m, lat.pack(b), x, tol=tol)
+            out.append([*(lat.unpack(v, sqcg.F32) for v in z), np.float64(loss), grad, np.int64(info.iters), lat.unpack(x)])
+            net.close()
+    assert all(np.array_equal(u, v) for u, v in zip(*out))
