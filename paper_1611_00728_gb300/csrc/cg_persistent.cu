@@ -167,6 +167,8 @@ struct UpdatedIn {
   }
 };
 
+constexpr size_t kMaxSmem = 206 * 1024;    // dynamic shared memory of a launch; k_sr_persistent's own comes on top
+constexpr size_t kBlockSmem = 227 * 1024;  // what a block can have
 constexpr int kLinkFloats = 9 * 32;  // float2 of one hop's links of a 32-site group in shared memory
 
 // Hop h of site i of group t (parity par's output): index of the neighbour, with the sign bit set where the
@@ -226,6 +228,9 @@ __global__ void __launch_bounds__(32 * NW, 1) k_sr_persistent(PArgs a) {
   constexpr int NH = 16 / SPLIT;  // hops of a warp
   constexpr int PT = 32 * NW;
   static_assert(3 * NG < NW, "a warp per group and colour in the epilogue");
+  // without this no block is resident, and the solve goes to the graph loop, correct but slower
+  static_assert(kMaxSmem + sizeof(SolverState) + (9 * NG * 32 + NW) * sizeof(float2) + 128 <= kBlockSmem,
+                "shared memory of a block: the state, part, wcross and a few words, beside kMaxSmem");
   // dynamic shared memory: the hops' partial sums [2][NW][3][32] (alternating by round: one barrier a
   // round), the neighbour indices [2][max_mine][16][32], then the cached links
   extern __shared__ float2 smx[];
@@ -488,8 +493,6 @@ __global__ void __launch_bounds__(32 * NW, 1) k_sr_persistent(PArgs a) {
   __syncthreads();
   for (int k = threadIdx.x; k < kWords; k += PT) reinterpret_cast<W*>(a.st)[k] = reinterpret_cast<const W*>(&ss)[k];
 }
-
-constexpr size_t kMaxSmem = 206 * 1024;  // of the 227 KB a block can have; a little static shared memory comes on top
 
 struct PKernel {
   void* fn;
