@@ -226,7 +226,7 @@ int sqcg_normal_op_noalloc(sqcg_ctx* ctx, double sigma, int prec, const void* x,
  * (SQCG_ERR_NOT_CONVERGED, x = last iterate). mode: SQCG_MODE_F64 or
  * SQCG_MODE_MIXED (FP32 Krylov vectors with reliable updates). The FP64 mode
  * runs as one CUDA graph launch; the mixed mode too (eight steps per WHILE
- * pass), except on lattices of at most five 128-site tiles per SM, where one
+ * pass), except on lattices of at most 24 groups of 32 sites of a parity per SM, where one
  * persistent cooperative kernel runs each segment between reliable updates
  * (environment SQCG_PERSISTENT=0 or 1 forces one form; SQCG_LAUNCH_MODE=eager
  * launches the graph's kernels one at a time, for profilers; SQCG_PDL=0, read

@@ -26,9 +26,12 @@ constexpr int kSRKernelsPerIter = 4;  // enqueue_sr_head (2 + finisher) + the up
 // about 3.4 us and a WHILE pass 3.5 us (a CUDA-graph probe of empty bodies), against ~200 us a step
 // at 32^4; the 32^4 mixed solve took 44.6, 43.5, 43.0 and 42.9 ms with 1, 2, 4 and 8 steps a pass.
 constexpr int kSRUnroll = 8;
-// the persistent loop runs where a parity has at most this many 32-site groups a SM. Measured, us an iteration,
-// persistent / graph loop: 18^4 (11 groups) 22.6 / 27.8, 20^4 (17) 36.1 / 40.3, 22^4 (25) 83 / 63
-constexpr int kPersistentMaxGroupsPerSM = 20;
+// the persistent loop runs where a parity has at most this many 32-site groups a SM. Measured, us an iteration of a
+// solve to 1e-11, persistent / graph loop, 12-real links (full): 8^4 (1 group) 7.9 / 16.3, 16^4 (7) 15.6 / 24.1
+// (15.4 / 24.4), 20^4 (17) 29.5 / 37.8 (34.7 / 49.4), 20x20x22x22 (20) 37.4 / 46.4 (48.6 / 62.0), 20x20x24x24 (24)
+// 55.0 / 60.1 (62.6 / 71.1), 18x20x24x28 (25) 62.4 / 62.2 (69.8 / 73.0), 18x18x26x30 (26) 67.0 / 64.3 (72.1 / 75.4),
+// 24^4 (35) 98 / 77 (110 / 88)
+constexpr int kPersistentMaxGroupsPerSM = 24;
 constexpr int kSRKernelsPerUpdatePersistent = 4;  // flush, Dslash pair, finisher (no head)
 constexpr int kSRKernelsPerUpdate = 7;  // enqueue_sr_reliable: flush, 2 FP64 + finisher, 2 FP32 + finisher
 

@@ -23,14 +23,15 @@
 // What bounds it, and what the layout answers (one step at 8^4 took 23.9 us in the form before this one: one
 // thread a site, a block per 128 sites; cycles of that step in brackets):
 //  * a thread's chain of 16 hops, each waiting for L2 (2 x 7000): a group goes to SPLIT warps that share its
-//    hops and meet in shared memory. Neighbour indices and as many of the groups' links as fit are
+//    hops and meet in shared memory. Neighbour indices and, of few groups, as many of their links as fit are
 //    kept in shared memory from the launch on, the 12-real rows already rebuilt. (2 x 1500 now)
 //  * the grid barriers (2 x 4000): one counter that only grows, arrived at with a release and polled with an
 //    acquire, by one block a SM. A tagged-slot barrier in which every block polled every other's sums took 8000.
 //  * the sums (3300): three warps add one sum each, one round of loads for the 152 blocks (1250)
 //  * the scalar step in FP64 (2500; an FP64 operation holds its scheduler for 64 cycles): in float-float, with
 //    the FP64 state and the reciprocal of gamma formed by other warps at the next barrier (step_ff; 500)
-// A step takes 5.2 us at 8^4, 8.1 on 10x12x14x16 (23), 13.6 at 16^4 (25.4) and 27.4 at 20^4 (37.5).
+// A step takes 5.6 us at 8^4, 7.9 on 10x12x14x16 and 13.0 at 16^4; an iteration of a solve, launches and reliable
+// updates with it, 7.9 (22.1), 9.8 (22.4), 15.6 (25.1) and at 20^4 29.5 (36.7; full links 34.7 / 43.8).
 //
 // The kernel returns when the step asks for a reliable update or the solve is done, with r and q
 // in the context's buffers; block 0 writes its state copy back. The true-residual pass (float-float or FP64
@@ -512,17 +513,27 @@ PKernel kernel_for(const sqcg_ctx* ctx) {
   return ctx->recon ? kernel_of<true, false, SPLIT, NW, FUSE>() : kernel_of<false, false, SPLIT, NW, FUSE>();
 }
 
-// The kernel for the context's link form and lattice, by the 32-site groups of the block that has most.
-// Measured (us an iteration of a solve, SPLIT x warps): 8^4 (1 group) 16x16 fused 8.0, 8x24 fused 8.8, 8x32
-// 10.2; 10x12x14x16 (3) 8x24 fused 10.2, 8x32 11.5, 16x16 fused 10.5; 14^4 (4) 8x32 12.9, 8x24 fused 13.2; 16^4
-// (7) 8x32 16.0, 8x24 fused 16.7, 4x24 18.0; 18^4 (11) 4x24 22.6, 8x32 23.0; 20^4 (17) 4x24 36.1, 8x32 37.9. Forming
-// r_new on the fly trades a barrier for three times the gathers, which pays only while a block has few groups.
+// The kernel for the context's link form and lattice, by the 32-site groups of the block that has most. Measured, us an
+// iteration of a solve (12-real, to 1e-11), SPLIT x warps: fused 16x16 / fused 8x24 / 8x32 / 4x24:
+//    1 group  (8^4)           7.9 /  8.7 / 10.3 / 11.1     11 groups (18^4)         28.2 / 22.7 / 21.9 / 21.2
+//    2 groups (8^3x32)        7.5 /  7.4 /  9.0 /  9.7     12 groups (18^3x20)      28.7 / 23.6 / 22.4 / 21.6
+//    3 groups (10x12x14x16)  10.6 /  9.8 / 10.9 / 11.3     14 groups (16x18x20x22)  30.4 / 25.7 / 24.2 / 24.5
+//    4 groups (14^4)         13.0 / 12.8 / 12.5 / 12.6     15 groups (18x18x20x22)  41.7 / 29.9 / 26.1 / 26.5
+//    5 groups (12x14x16x18)  14.5 / 13.4 / 14.2 / 13.1     16 groups (16x20x22x22)  44.0 / 33.1 / 27.1 / 27.9
+//    6 groups (14^3x18)      16.3 / 14.3 / 14.5 / 13.5     17 groups (20^4)         50.5 / 34.8 / 30.8 / 29.4
+//    7 groups (16^4)         17.9 / 16.6 / 15.6 / 17.3     18 groups (18x20x22x22)  57.4 / 38.6 / 32.9 / 31.9
+//    8 groups (16^3x18)      19.6 / 17.5 / 16.7 / 18.3     19 groups (20^3x22)      60.9 / 43.7 / 34.1 / 37.9
+//    9 groups (16x16x18x18)  21.7 / 18.5 / 19.1 / 18.9     20 groups (20x20x22x22)  70.3 / 49.1 / 37.4 / 42.5
+//   10 groups (16x18x16x20)  23.4 / 21.0 / 20.0 / 19.3     22 groups (22x22x20x22)  80.7 / 58.1 / 48.1 / 48.9
+// Forming r_new on the fly trades a barrier for three times the gathers, which pays only while a block has few groups.
+// Above, a block takes four groups a round with 8x32 and six with 4x24, whose rounds take about half as long again:
+// 4x24 where 8x32 needs one and a half times the rounds.
 PKernel persistent_kernel(const sqcg_ctx* ctx) {
   const int mine = (grid_for(ctx->g.Vh, 32) + ctx->nsm - 1) / ctx->nsm;
   if (mine <= 1) return kernel_for<16, 16, true>(ctx);
   if (mine <= 3) return kernel_for<8, 24, true>(ctx);
-  if (mine <= 9) return kernel_for<8, 32, false>(ctx);
-  return kernel_for<4, 24, false>(ctx);
+  const int rounds32 = (mine + 3) / 4, rounds24 = (mine + 5) / 6;
+  return 2 * rounds32 >= 3 * rounds24 ? kernel_for<4, 24, false>(ctx) : kernel_for<8, 32, false>(ctx);
 }
 
 DArgs<float> dargs(const sqcg_ctx* ctx, int par, const float2* in, float2* out) {
@@ -548,13 +559,19 @@ DArgs<float> dargs(const sqcg_ctx* ctx, int par, const float2* in, float2* out) 
 }
 
 // Dynamic shared memory of a launch: the kernel's own, the neighbour indices of the fullest block's groups where
-// they fit (*max_mine, else 0), and as many of their hop links (*ncached) as still do.
+// they fit (*max_mine, else 0), and as many of their hop links (*ncached) as still do, where that is a sixth of them
+// (an eighth of 8-way 12-real ones, which no other site reads): what a block does not take is L1, which serves the
+// gathers. us an iteration with / without links in shared memory: 16^4 (7 groups a block, a quarter of them) 15.8 / 16.7,
+// 16^3x18 (8) 16.7 / 17.3, 16x18x16x20 (10, 18%) 19.4 / 19.6, 18^4 (11, 16%) 21.7 / 21.2 (full 23.1 / 21.2; 8-way
+// 12-real 28.1 / 30.3), 20^4 (17) 31.8 / 29.9 (full 43.2 / 35.5), 20^3x22 (19) 40.8 / 34.3 (full 54.9 / 42.4).
 size_t smem_bytes(const PKernel& k, const sqcg_ctx* ctx, int* max_mine, int* ncached) {
   const size_t mine = (grid_for(ctx->g.Vh, 32) + ctx->nsm - 1) / ctx->nsm;
   const size_t base = k.smem_fixed + 2 * mine * 512 * sizeof(int), link = kLinkFloats * sizeof(float2);
   *max_mine = *ncached = 0;
   if (base > kMaxSmem) return k.smem_fixed;
-  const size_t fit = (kMaxSmem - base) / link, all = 32 * mine, n = fit < all ? fit : all;
+  const size_t fit = (kMaxSmem - base) / link, all = 32 * mine;
+  size_t n = fit < all ? fit : all;
+  if ((ctx->eightway && ctx->recon ? 8 : 6) * n < all) n = 0;
   *max_mine = (int)mine;
   *ncached = (int)n;
   return base + n * link;

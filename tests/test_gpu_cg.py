@@ -760,6 +760,29 @@ def test_persistent_loop_by_groups_per_block(sqcg, links_cache, monkeypatch, L, 
         assert oracle.true_rel_residual(L, fat, lng, 4 * m * m, b, lat.unpack(x)) <= tol
 
 
+# ... and where the shape of the loop changes: five groups a block (686) in one round of six, eleven (1641) and nineteen
+# (2750) without links in shared memory, eleven with an eighth of them (8-way, 12-real).
+@pytest.mark.parametrize("L,recon,eight", [((14, 14, 14, 16), True, False), ((14, 14, 14, 16), False, True),
+                                           ((18, 18, 18, 18), True, True), ((18, 18, 18, 18), False, True),
+                                           ((20, 20, 20, 22), True, False), ((20, 20, 20, 22), False, False)])
+def test_persistent_loop_where_its_shape_changes(sqcg, links_cache, monkeypatch, L, recon, eight):
+    m, tol = 0.1, 1e-9
+    fat, lng = links_cache(L, 1007)
+    b = synth.gaussian_source(L, 2700)
+    with sqcg.Lattice(L) as lat:
+        lat.load_links(fat, lng, recon12=recon, eight_way=eight)
+        db = lat.pack(b)
+        iters = []
+        for loop in ("0", "1"):
+            monkeypatch.setenv("SQCG_PERSISTENT", loop)
+            x = lat.new_spinor()
+            info = lat.cg_solve(m, db, x, tol=tol, max_iter=5000, mode=sqcg.MODE_MIXED)
+            assert info.status == 0
+            assert oracle.true_rel_residual(L, fat, lng, 4 * m * m, b, lat.unpack(x)) <= tol
+            iters.append(info.iters)
+        assert abs(iters[0] - iters[1]) <= 2, iters
+
+
 @pytest.mark.parametrize("power", [-50, 50])
 def test_persistent_loop_outside_the_float_float_step(sqcg, links_cache, monkeypatch, power):
     """A source scaled by a power of two (exact in every precision) far enough that |r|^2 leaves the range of the
