@@ -188,18 +188,6 @@ def _torch():
     return _torch_module
 
 
-def _current_stream() -> int:
-    """Handle of torch's current CUDA stream."""
-    # the handle of torch.cuda.current_stream() without the Stream object around it: with this, the addresses as
-    # plain integers and torch imported once, an 8^4 Dslash call takes 4.6 us instead of 9.1 (its kernel 2.5). Both
-    # names are torch's own, not its public interface: where one is missing, the public call serves
-    torch = _torch()
-    try:
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
-    except AttributeError:
-        return torch.cuda.current_stream().cuda_stream
-
-
 class Lattice:
     """One lattice geometry with its links on the current CUDA device.
 
@@ -251,7 +239,15 @@ class Lattice:
         _check(library().sqcg_set_update_arithmetic(self._h, int(prec)), "sqcg_set_update_arithmetic")
 
     def _sync_stream(self):
-        library().sqcg_set_stream(self._h, _current_stream())
+        # the handle of torch.cuda.current_stream() without the Stream object around it: with this, the addresses as
+        # plain integers and torch imported once, an 8^4 Dslash call takes 4.6 us instead of 9.1 (its kernel 2.5). Both
+        # names are torch's own, not its public interface: where one is missing, the public call serves
+        cuda = _torch()._C
+        try:
+            stream = cuda._cuda_getCurrentRawStream(cuda._cuda_getDevice())
+        except AttributeError:
+            stream = _torch().cuda.current_stream().cuda_stream
+        library().sqcg_set_stream(self._h, stream)
 
     # -- data -------------------------------------------------------------
     def load_links(self, fat: np.ndarray, lng: np.ndarray, recon12: bool = False, eight_way: bool = False):

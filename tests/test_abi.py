@@ -199,7 +199,13 @@ def test_binding_finds_the_stream_without_torch_internals(monkeypatch, missing):
     fake = types.SimpleNamespace(
         _C=types.SimpleNamespace(**internal),
         cuda=types.SimpleNamespace(current_stream=lambda: types.SimpleNamespace(cuda_stream=77)))
+    handles = []
     monkeypatch.setattr(sq, "_torch_module", fake)
-    assert sq._current_stream() == 103
+    monkeypatch.setattr(sq, "library",
+                        lambda: types.SimpleNamespace(sqcg_set_stream=lambda ctx, stream: handles.append(stream)))
+    lat = object.__new__(sq.Lattice)
+    lat._h = None
+    lat._sync_stream()
     delattr(fake._C, missing)
-    assert sq._current_stream() == 77
+    lat._sync_stream()
+    assert handles == [103, 77]
