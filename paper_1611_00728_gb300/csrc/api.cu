@@ -214,6 +214,7 @@ int sqcg_normal_op(sqcg_ctx* ctx, double sigma, int prec, const void* x, void* y
   L.out_parity = 1;
   L.prec = L.out_prec = prec;
   L.epi = EPI_PLAIN;
+  L.pair = 1;
   L.in = x;
   L.out = tmp;
   SQCG_TRY(launch_dslash(ctx, L, ctx->stream));

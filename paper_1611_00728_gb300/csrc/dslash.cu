@@ -14,6 +14,8 @@
 // Neighbour indices are computed from the site coordinates (no index tables).
 // With 12-real long links (FP32 copy only) the third row is rebuilt as
 // conj(row0 x row1) / s, s = s0 * eta_mu * boundary sign of that link.
+#include <math.h>
+
 #include "dslash_core.cuh"
 namespace {
 
@@ -254,7 +256,7 @@ int launch_t(sqcg_ctx* ctx, const DslashLaunch& L, cudaStream_t s) {
   a.out_f32 = sizeof(RO) == 4;
   const bool sr = L.epi == EPI_SR_DOTS || L.epi == EPI_SR_DOTS2;
   const bool reduces = (L.epi == EPI_NORMAL_DOT || sr || L.epi == EPI_TRUE_RESID) && L.fin != FIN_NONE;
-  const int split = dslash_split(ctx, L.prec, L.gate != GATE_NONE);
+  const int split = dslash_split(ctx, L.prec, L.gate != GATE_NONE, L.pair != 0);
   const int grid = grid_for(ctx->g.Vh, split > 1 ? 32 : kThreads);
   if (reduces && grid > ctx->max_blocks) return SQCG_ERR_INVALID_ARG;  // partials hold 3 sums and more
   // programmatic dependent launch where the caller says a kernel precedes this one, and for the
@@ -297,25 +299,47 @@ int launch_r(sqcg_ctx* ctx, const DslashLaunch& L, cudaStream_t s) {
 
 }  // namespace
 
-// Measured on the GB300 (us a pass, links in L2 up to 20^4; 128-site tiles a SM in brackets), with
-// 1 / 4 / 8 warps a site group:
-//   FP32 full links   8^4 [0.1] 7.7/5.1/2.5, 16^4 [1.7] 8.0/6.2/5.5, 20^4 [4.1] 14.6/17.0/11.3,
-//                     24^4 [8.5] 33.2/41.1/31.4, 32^4 [27] 97.8/119.5/91.0: 8 everywhere outside captured
-//                     loops (on large lattices eight short chains keep more of the link loads in flight than
-//                     one thread can hold). Inside them a block also waits for the pass before it, and the
-//                     mixed CG's step takes 52.6/52.0/49.3 at 20^4 but 235/270/261 at 32^4
-//   FP32 12-real      8^4 5.2/3.3/2.5, 10x12x14x16 [0.7] 5.3/3.8/3.5, 16^4 5.9/5.0/5.5, 20^4 8.8/10.2/11.8,
-//                     32^4 78.8/83.1/82.9 (CG step: 12^4 [0.5] 24.4/19.6/18.6, 14^4 [1.0] 24.2/21.5/22.7,
-//                     16^4 25.7/25.3/26.1, 18^4 [2.7] 28.2/32.7/32.1); 8-way: 24^4 32.9/29.4/29.2,
-//                     28^4 [16] 46.3/50.5/50.9
-//   FP64              8^4 22.8/8.5/7.3, 10x12x14x16 23.1/16.4/17.6, 16^4 37.8/35.9/37.8, 20^4 99.6/85.5/89.4,
-//                     24^4 169.6/170.6/179.0 (there the FP64 pipe is the bound)
-//   float-float       8^4 14.4/5.1/3.8, 16^4 16.5/12.2/13.5, 24^4 85.9/68.0/72.8, 28^4 114.2/118.1/131.2
-int dslash_split(const sqcg_ctx* ctx, int prec, bool gated) {
-  const int tiles = grid_for(ctx->g.Vh, kThreads), nsm = ctx->nsm;
-  if (prec == SQCG_F32 && !ctx->recon) return gated && tiles > 5 * nsm ? 1 : 8;
-  if (prec == SQCG_F32) return 4 * tiles <= 3 * nsm ? 8 : tiles <= (ctx->eightway && !gated ? 9 : 2) * nsm ? 4 : 1;
-  return 2 * tiles <= nsm ? 8 : tiles <= (prec == SQCG_FF ? 10 : 5) * nsm ? 4 : 1;
+// By t, the 128-site tiles a SM. Two things decide: the chain of a site's 16 hops, which the split shortens where a SM
+// has few warps, and how full the last wave is. One thread a site: 10 blocks of 128 a SM are resident (FP32, full
+// links; 9 with 12-real ones, 8 with 8-way 12-real ones and in float-float), and a wave that ends just full beats the
+// split, which does more work a site; one that starts anew loses to it. FP64 is bound by its pipe: a tile a SM
+// takes 20 us, whole tiles with one thread a site, 32-site groups (of 5.4) with four warps.
+// Measured on the GB300 (us a call, back to back; 1 / 4 / 8 warps a site group; loops: us of a whole solve):
+//   FP32 full      Dslash   8^4 [t 0.1] 10.3/6.0/4.5, 16^4 [1.7] 10.3/6.3/8.2, 20^4 [4.1] 16.9/15.5/14.5, 22^4 [6.0]
+//                           30.8/30.8/26.8, 24^4 [8.5] 35.0/39.0/35.0, 22x24x26x28 [9.9] 38.9/42.9/40.8, 26^4 [11.8]
+//                           57.5/50.9/45.8, 32^4 [27] 98.5/104/94.9
+//                  normal   18x20^3 [3.7] 28.8/28.6/27.1, 16x24x28x30 [8.3] 69.6/77.8/70.4, 24^4 70.0/79.8/73.3,
+//                           20x20x28x32 [9.2] 74.0/82.7/78.1, 16x24x32x32 [10.1] 109/92/83
+//                  8-way    normal 18x22x24x32 [7.8] 69.8/72.2/68.6, 24^4 72.1/75.9/73.3, 20x20x28x32 74.6/79.8/78.2
+//                  CG loop  20x20x22x22 [5.0] 12797/12809/12656, 22^4 14591/16688/15314; multi-shift, 4 shifts, 16^3x32
+//                           26246/23711/21970
+//   FP32 12-real   Dslash   8^4 6.3/4.7/4.6, 14^4 [1.0] 8.2/6.0/6.1, 16^4 8.3/6.3/8.3, 14^2x24^2 8.3/10.3/10.4, 32^4
+//                           81.8/83/83
+//                  8-way    Dslash 12x14x24x24 [2.5] 8.3/8.3/10.3, 18^4 8.3/10.3/10.3, 18x22x24x32 26.0/30.8/29.2, 16x22x28x32
+//                           [8.1] 34.9/30.8/30.8, 20x20x28x32 35.5/35.0/33.7; normal (both parities' links, past L2
+//                           sooner) 18^4 29.0/26.8/25.5, 18x20x20x24 [4.4] 37.6/37.0/39.8, 20^3x22 [4.5] 37.5/42.5/39.4,
+//                           24^4 63.6/64.7/66.6
+//   FP64           Dslash   8^4 22.8/8.5/7.3, 14^4 24.7/22.7/24.7, 16^4 39.1/37.0/39.1, 12x18x18x20 [2.0] 41.1/43.2/45.2,
+//                           14^2x24^2 59.6/63.7/65.7, 18x20^3 80.1/78.0/80.2, 16x18x18x30 [4.0] 80.1/82.4/86.1, 22^4
+//                           133.5/124.9/129.3, 24^4 172/171/179; CG loop 16^4 14893/15286/14206, 12x16x16x22 [1.74]
+//                           16989/17517/16223, 12x14x20x22 [1.9] 17383/19364/18707
+//   float-float    Dslash   8^4 14.4/5.1/3.8, 16^4 16.6/14.4/14.5, 20x20x22x22 46.7/43.4/45.2, 18x20x22x26 [5.3] 48.4/
+//                           51.3/51.1, 18x22x24x32 60.1/67.6/69.3, 16x22x28x32 86.3/68.2/72.6, 24x24x24x32 [11.4] 95/93/98
+int dslash_split(const sqcg_ctx* ctx, int prec, bool loop, bool pair) {
+  const double t = (double)grid_for(ctx->g.Vh, kThreads) / ctx->nsm;
+  if (prec == SQCG_F32 && !ctx->recon) {
+    if (loop) return t > 5 ? 1 : 8;
+    return t > (pair ? 8.4 : 9) && t <= 10 ? 1 : 8;
+  }
+  if (prec == SQCG_F32) {
+    if (t <= 2) return t <= 0.75 ? 8 : 4;
+    if (!ctx->eightway || loop) return 1;
+    return pair ? (t <= 4.45 ? 4 : 1) : t <= 2.5 || (t > 8 && t <= 9) ? 4 : 1;
+  }
+  if (t <= 0.5) return 8;
+  if (prec == SQCG_FF) return t <= 5 || (t > 8 && t <= 10) ? 4 : 1;
+  if (t > 5 || (t > 1.5 && ceil(t) - t <= 0.16)) return 1;
+  return loop && t > 1.65 && t <= 1.8 ? 8 : 4;
 }
 
 int launch_dslash(sqcg_ctx* ctx, const DslashLaunch& L, cudaStream_t s) {

@@ -283,7 +283,7 @@ int launch_dslash_ff(sqcg_ctx* ctx, const FFLaunch& L, cudaStream_t s) {
   a.gate = L.gate;
   a.fin = L.fin;
   if ((L.gate != GATE_NONE || L.fin != FIN_NONE) && (!ctx->st || !ctx->partials)) return SQCG_ERR_INVALID_ARG;
-  const int split = dslash_split(ctx, SQCG_FF, L.gate != GATE_NONE);
+  const int split = dslash_split(ctx, SQCG_FF, L.gate != GATE_NONE, false);
   const int grid = grid_for(ctx->g.Vh, split > 1 ? 32 : kThreads);
   if (L.true_resid) {
     if (!L.out32 || !L.x || !L.b) return SQCG_ERR_INVALID_ARG;

@@ -1147,7 +1147,7 @@ int nn_pair(sqcg_nn* nn, double sigma, const float2* r, const float2* e, cudaStr
   SQCG_TRY(conv_launch(nn, 2, false, IN_FULL, OUT_EVEN_SCALED, nn->h2, nn->d, nullptr, 0, 1, nullptr, 0,
                        nn->scal + 1, s, e, nullptr, true));
   DslashLaunch L = {};
-  L.out_parity = 1; L.prec = L.out_prec = SQCG_F32; L.epi = EPI_PLAIN; L.in = nn->d; L.out = nn->tmp;
+  L.out_parity = 1; L.prec = L.out_prec = SQCG_F32; L.epi = EPI_PLAIN; L.pair = 1; L.in = nn->d; L.out = nn->tmp;
   SQCG_TRY(launch_dslash(ctx, L, s));
   L.out_parity = 0; L.epi = EPI_NORMAL; L.in = nn->tmp; L.out = nn->Ad; L.y = nn->d; L.sigma = sigma;
   SQCG_TRY(launch_dslash(ctx, L, s));
@@ -1155,7 +1155,7 @@ int nn_pair(sqcg_nn* nn, double sigma, const float2* r, const float2* e, cudaStr
   if (nn->loss_norm == 2) {
     // L = <Ad, Ad> / <r, r>; dL/dz = 2 A (A d) / <r, r>   (A e = r: the preconditioned residual)
     L = DslashLaunch{};
-    L.out_parity = 1; L.prec = L.out_prec = SQCG_F32; L.epi = EPI_PLAIN; L.in = nn->Ad; L.out = nn->tmp;
+    L.out_parity = 1; L.prec = L.out_prec = SQCG_F32; L.epi = EPI_PLAIN; L.pair = 1; L.in = nn->Ad; L.out = nn->tmp;
     SQCG_TRY(launch_dslash(ctx, L, s));
     L.out_parity = 0; L.epi = EPI_NORMAL; L.in = nn->tmp; L.out = nn->zbuf; L.y = nn->Ad; L.sigma = sigma;
     SQCG_TRY(launch_dslash(ctx, L, s));

@@ -56,6 +56,7 @@ extern "C" int sqcg_normal_op_noalloc(sqcg_ctx* ctx, double sigma, int prec, con
   L.out_parity = 1;
   L.prec = L.out_prec = prec;
   L.epi = EPI_PLAIN;
+  L.pair = 1;
   L.in = x;
   L.out = tmp;
   SQCG_TRY(launch_dslash(ctx, L, ctx->stream));

@@ -277,12 +277,14 @@ struct DslashLaunch {
   int gate;
   int fin;
   int pdl;  // the kernel before it on the stream is a kernel: launch with programmatic dependent launch
+  int pair;  // one of the two passes of a normal operator outside a captured loop
 };
 
 int launch_dslash(sqcg_ctx* ctx, const DslashLaunch& L, cudaStream_t s);
 // warps that share a site's hops in the Dslash of this precision (SQCG_F64, SQCG_F32, SQCG_FF) on this
-// lattice; 1: one thread does them all. gated: a pass of a captured loop, which reads the solver state first
-int dslash_split(const sqcg_ctx* ctx, int prec, bool gated);
+// lattice; 1: one thread does them all. loop: a pass of a captured loop, which reads the solver state first; pair:
+// see DslashLaunch
+int dslash_split(const sqcg_ctx* ctx, int prec, bool loop, bool pair);
 
 int launch_cg_update_x(sqcg_ctx* ctx, int mixed, double2* x, cudaStream_t s);
 int launch_loop_control(sqcg_ctx* ctx, cudaStream_t s);

@@ -369,6 +369,23 @@ def test_persistent_loop_ends_on_max_iter(sqcg, links_cache, monkeypatch):
         assert abs(res - lib_res) <= 1e-6 * res, (loop, res, lib_res)
 
 
+@pytest.mark.parametrize("L", [(12, 16, 16, 22), (12, 14, 20, 22)])
+def test_f64_cg_by_the_last_wave(sqcg, links_cache, L):
+    """FP64 loops where eight warps, or one thread, take a site's hops by how full the last wave is (1.74 and 1.90 tiles
+    a SM of 152)."""
+    m, tol = 0.1, 1e-10
+    fat, lng = links_cache(L, 1008)
+    b = synth.gaussian_source(L, 2703)
+    with sqcg.Lattice(L) as lat:
+        lat.load_links(fat, lng)
+        db, x = lat.pack(b), lat.new_spinor()
+        info = lat.cg_solve(m, db, x, tol=tol, mode=sqcg.MODE_F64)
+        assert info.status == 0 and oracle.true_rel_residual(L, fat, lng, 4 * m * m, b, lat.unpack(x)) <= tol
+        xs = [lat.new_spinor() for _ in range(2)]
+        for i, s, xx in zip(lat.multishift_cg_solve([0.04, 0.5], db, xs, tol=tol, mode=sqcg.MODE_F64), [0.04, 0.5], xs):
+            assert i.status == 0 and oracle.true_rel_residual(L, fat, lng, s, b, lat.unpack(xx)) <= tol
+
+
 @pytest.mark.parametrize("delta,interval", [(0.001, 100), (0.01, 100), (0.5, 5), (0.1, 1000), (1e-5, 100)])
 def test_reliable_update_settings(sqcg, links_cache, delta, interval):
     """Any trigger setting still ends on the FP64 true residual; the count follows the setting."""

@@ -248,6 +248,27 @@ def test_split_dslash_remainders(sqcg, links_cache, L, recon, eight):
                 assert rel(lat.unpack(out, prec), want_a) <= bar, prec
 
 
+# Where the rule turns by how full the last wave of one thread a site is (152 SMs): 1.90 tiles a SM (FP64: one thread),
+# 5.30 (float-float: one thread; 8-way 12-real: alone one thread), 8.53 (full links: the normal operator one thread).
+@pytest.mark.parametrize("L,recon,eight", [((12, 14, 20, 22), False, False), ((18, 20, 22, 26), True, True),
+                                           ((24, 24, 24, 24), False, False), ((24, 24, 24, 24), True, True)])
+def test_split_dslash_by_the_last_wave(sqcg, links_cache, L, recon, eight):
+    fat, lng = links_cache(L, 1003)
+    psi = synth.gaussian_source(L, 2003)
+    want = [oracle.dslash(L, fat, lng, psi, par) for par in (0, 1)]
+    want_a = oracle.normal_op(L, fat, lng, 0.04, psi)
+    with sqcg.Lattice(L) as lat:
+        lat.load_links(fat, lng, recon12=recon, eight_way=eight)
+        for prec, bar in ((0, 1e-12), (1, 1e-5), (2, 1e-12)):
+            d_in, out = lat.pack(psi, prec), lat.new_spinor(prec)
+            for par in (0, 1):
+                lat.dslash(par, d_in, out, prec)
+                assert rel(lat.unpack(out, prec), want[par]) <= bar, (prec, par)
+            if prec != 2:
+                lat.normal_op(0.04, d_in, out, prec)
+                assert rel(lat.unpack(out, prec), want_a) <= bar, prec
+
+
 @pytest.mark.parametrize("where", [(0, 0), (1, 2), (-1, 3)])
 @pytest.mark.parametrize("folded", [False, True])
 def test_recon12_check_finds_one_link(sqcg, links_cache, where, folded):
