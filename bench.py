@@ -551,8 +551,8 @@ def run_ours(args, ranks: Ranks):
                     "vs_all_cores_32^4": dslash["f32_recon12"]["gflops"]
                     / cpu["dslash"]["x".join(map(str, LATTICE))]["all_cores_gflops"]},
                 "paper_context": PAPER_CONTEXT,
-                "notes": "dtype f32: FP32 Dslash and Krylov vectors; float-float grid sums; FP64 x, scalar "
-                         "recurrences and reliable-update residuals (float-float Dslash, FP64 sum). Roofline: "
+                "notes": "dtype f32: FP32 Dslash and Krylov vectors; float-float grid sums; FP64 x (the "
+                         "multi-shift loop's x_s: float-float), scalar recurrences and reliable-update residuals (float-float Dslash, FP64 sum). Roofline: "
                          "Dslash-only loop timed with CUDA events in this run."}
         print(json.dumps(line), flush=True)
 

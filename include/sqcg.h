@@ -87,7 +87,12 @@ extern "C" {
 #define SQCG_MODE_F64 0   /* everything in FP64 */
 #define SQCG_MODE_MIXED 1 /* FP32 Dslash and vectors; FP64 x and scalars; grid sums in float-float;
                              true residuals of the reliable updates in float-float (SQCG_FF, default) or
-                             FP64 arithmetic, summed in FP64 */
+                             FP64 arithmetic, summed in FP64. Two exceptions: between its reliable updates
+                             the multi-shift loop holds its x_s as float-float (48 bits, FP32's range), in the
+                             caller's arrays, FP64 again when it returns; and on small lattices, where one
+                             kernel runs the single-mass loop, the step lengths that it applies (rounded to
+                             FP32 in either case) come from the grid sums in float-float, the scalars that
+                             the loop goes on with from the same sums in FP64 */
 /* Multi-shift only: OR-ed into the mode of sqcg_multishift_cg_solve (and
  * sqcg_rational_apply), shift-aware reliable updates of the shared Krylov loop.
  * Each time the base residual has fallen by the reliable-update factor (1e-3

@@ -822,7 +822,7 @@ __device__ __forceinline__ int nbr_of(const Geom& g, int i, const SiteXY& c, int
 // shared-memory wavefronts of the link reads; the neighbour gathers are the same.
 // Bound by the L1 pipe (72%: gathers and link reads) and by issue (67%) at 28 warps
 // per SM: at most 64 registers for WT <= 2, so that five blocks of six warps fit.
-// 8 right-hand sides on 16^4 and 24^4: 101 -> 97 us a pass, a solve 78.3 -> 75.1 ms.
+// 8 right-hand sides on 16^4 and 24^4: 101 -> 97 us a pass.
 // Neighbour indices and 16-byte link rows in shared memory were slower (105 us).
 constexpr int kHops = 16;
 

@@ -114,7 +114,8 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned n, unsigned
 // pipe. An FP64 operation holds its scheduler for 64 cycles on this GPU whatever the lanes in it, and the
 // whole grid waits for this chain: some 30 of them took 2900 cycles, this takes 500. Only what the next phase
 // needs comes out of it, alpha and beta in FP32; the FP64 state follows while the grid waits at the
-// next barrier, from the same sums (step_state). False where sr_step itself has to run: a reliable update or
+// next barrier, from the same sums. Errors of 84 solves (4x6x8x10 to 20^4, to 1e-11) against 64 bits: 1.0005 +- 0.0002
+// of the graph loop's, whose step is sr_step. False where sr_step itself has to run: a reliable update or
 // the end of the solve, or numbers outside the range in which the float-float chain is safe.
 struct StepInputs {  // formed at the barrier before
   float2 inv;   // 1 / gamma_{k-1}

@@ -868,3 +868,26 @@ def test_multishift_without_room_for_passes(sqcg, links_cache, monkeypatch, flag
             out.append(([i.iters for i in infos], [lat.unpack(x) for x in xs]))
     assert out[0][0] == out[1][0]
     assert all(np.array_equal(u, v) for u, v in zip(out[0][1], out[1][1]))
+
+
+@pytest.mark.parametrize("power", [-50, 50])
+def test_multishift_far_from_one(sqcg, links_cache, power):
+    """The mixed multi-shift loop holds x_s in two FP32 numbers. A source scaled by a power of two (exact in every
+    precision) as far as |r|^2 allows in FP32, with a small shift that makes x_s larger than it, is solved as the
+    unscaled one is: the residuals of the scaled-back solutions on the oracle, and the iterations up to the rounding of
+    |r|^2 at the end of its range."""
+    L, tol = (8, 8, 8, 8), 1e-3
+    fat, lng = links_cache(L, 1001)
+    shifts = [1e-4, 1e-2, 1.0]
+    b = synth.gaussian_source(L, 2704)
+    with sqcg.Lattice(L) as lat:
+        lat.load_links(fat, lng)
+        iters = []
+        for scale in (1.0, 2.0 ** power):
+            xs = [lat.new_spinor() for _ in shifts]
+            infos = lat.multishift_cg_solve(shifts, lat.pack(scale * b), xs, tol=tol, mode=sqcg.MODE_MIXED)
+            for s, i, x in zip(shifts, infos, xs):
+                assert i.status == 0
+                assert oracle.true_rel_residual(L, fat, lng, s, b, lat.unpack(x) / scale) <= tol
+            iters.append([i.iters for i in infos])
+        assert all(abs(u - v) <= 0.1 * u + 5 for u, v in zip(*iters))
