@@ -820,8 +820,9 @@ __device__ __forceinline__ int nbr_of(const Geom& g, int i, const SiteXY& c, int
 // a warp holds 16 sites of two groups, so each link element a warp reads from
 // shared memory serves both groups in one access (a broadcast), which halves the
 // shared-memory wavefronts of the link reads; the neighbour gathers are the same.
-// Bound by the L1 pipe (72%: gathers and link reads) and by issue (67%) at 28 warps
-// per SM: at most 64 registers for WT <= 2, so that five blocks of six warps fit.
+// Bound by the latency of the gathers beside an L1 pipe 66% and issue slots 67% busy at
+// 25 warps per SM (8 right-hand sides on 16^4 and 24^4; 73%, 75% and 31 warps for 16 at
+// 32^4; profiles/mrhs_dslash_smem_32x32x32x32_w16.md): at most 64 registers for WT <= 2, so that five blocks of six warps fit.
 // 8 right-hand sides on 16^4 and 24^4: 101 -> 97 us a pass.
 // Neighbour indices and 16-byte link rows in shared memory were slower (105 us).
 constexpr int kHops = 16;

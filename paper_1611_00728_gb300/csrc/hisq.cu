@@ -45,7 +45,7 @@
 // products of a wrap keep their rows. With whole matrices in a thread these kernels took 168-232 registers, so that
 // 12-24% of the warp slots hid the latency of the accumulation chains (FMA pipe 52-60% busy). A block is 64 sites
 // x 3 rows, so the right factors that three threads read come from L1 for two of them. 24^3 x 32: 12.8 -> 9.9 ms,
-// the packed instructions (two pipe slots each) filling 72% of the FMA pipe; kernel A 1.33 -> 1.06 ms, B 2.63 -> 2.12,
+// the packed instructions (two pipe slots each) filling 71% of the FMA pipe (profiles/hisq_smear_32x32x32x32.md); kernel A 1.33 -> 1.06 ms, B 2.63 -> 2.12,
 // C 1.66 -> 1.14 (level 1), at 5, 4 and 4 blocks a SM (one fewer each: 10.9 ms; five for all: 10.0).
 #include <math.h>
 #include <string.h>

@@ -187,9 +187,10 @@ __device__ __forceinline__ void gate_partials(const float (&red)[2 * CH][SITES +
 
 // The layers with one input or one output channel: a block is 32 sites, each warp transports one hop of all of them,
 // so a site's eight gathers are in flight together in eight warps (bound by their latency: one lane a site walked the
-// hops in turn, on two blocks an SM at 16^4). The sums over the taps keep the order of the taps. 8 -> 1 at 24^4 53 -> 43
-// us (ncu; the 163 MB take 24); both, with five and four blocks an SM, take a network application there from 281 to
-// 263 us and one at 16^4 from 75 to 65 (one parity's sites a block in the first layer: 267 and 66).
+// hops in turn, on two blocks an SM at 16^4). The sums over the taps keep the order of the taps. 8 -> 1 at 24^4 53 -> 41
+// us (ncu, profiles/fcg_learned_32x32x32x32_launches.md; the 163 MB take 24), though 122 -> 142 at 32^4; both, with five
+// and four blocks an SM, take a network application at 24^4 from 281 to 263 us, one at 16^4 from 75 to 65 (one parity's
+// sites a block in the first layer: 267 and 66) and, with the launches, one at 32^4 from 757 to 726.
 
 // 1 -> 8, from the even sites: the odd sites' hops meet in shared memory beside the even sites' own vectors, then warp
 // o mixes output channel o of both. TILES: groups of 32 sites of each parity that a block takes in turn (with gate
