@@ -1401,7 +1401,7 @@ void tune_file_store(const std::string& key, const TuneChoice& c) {
 }
 
 // What a choice was timed on: the kernels and candidates (the number, which goes up with them, so that an older file's
-// choices are not taken for this build's), the SMs, and the batch.
+// choices, timed on other kernels, are not taken), the SMs, and the batch.
 std::string tune_key(const BatchPlan& P) {
   char buf[128];
   snprintf(buf, sizeof(buf), "mrhs_dslash_f32.2:%dsm", P.ctx[0]->nsm);

@@ -778,10 +778,11 @@ def test_persistent_loop_by_groups_per_block(sqcg, links_cache, monkeypatch, L, 
 
 
 # ... and where the shape of the loop changes: five groups a block (686) in one round of six, eleven (1641) and nineteen
-# (2750) without links in shared memory, eleven with an eighth of them (8-way, 12-real).
+# (2750) without links in shared memory, eleven with an eighth of them (8-way, 12-real), and twenty-four (3600), the most.
 @pytest.mark.parametrize("L,recon,eight", [((14, 14, 14, 16), True, False), ((14, 14, 14, 16), False, True),
                                            ((18, 18, 18, 18), True, True), ((18, 18, 18, 18), False, True),
-                                           ((20, 20, 20, 22), True, False), ((20, 20, 20, 22), False, False)])
+                                           ((20, 20, 20, 22), True, False), ((20, 20, 20, 22), False, False),
+                                           ((20, 20, 24, 24), True, False)])
 def test_persistent_loop_where_its_shape_changes(sqcg, links_cache, monkeypatch, L, recon, eight):
     m, tol = 0.1, 1e-9
     fat, lng = links_cache(L, 1007)
